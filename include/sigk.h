@@ -76,7 +76,10 @@ typedef enum { SIGK_F32 = 0, SIGK_F64 = 1 } sigk_dtype;   /* storage AND arithme
  *    that a contraction kernel first writes into a banded buffer in the
  *    workspace (4 bytes per coarse cell); CHAIN and AUTO take it for f32
  *    pairs that fit a warp but are too wide (d > 16) for inline products.
- *  AUTO: CHAIN for f32 (PLAIN when CHAIN has no instance), PLAIN for f64. */
+ *  AUTO: CHAIN for f32 (PLAIN when CHAIN has no instance).  For f64 pairs of
+ *    uniform lengths and Grams the register wavefront with one cluster of
+ *    blocks per pair (dyadic_order <= 3 and increments that fit a block's
+ *    shared memory; forward and backward), else PLAIN. */
 typedef enum {
     SIGK_REC_AUTO = 0, SIGK_REC_CHAIN = 1, SIGK_REC_PLAIN = 2, SIGK_REC_STRIP = 3, SIGK_REC_BAND = 4
 } sigk_rec;

@@ -8,8 +8,9 @@
 // c = 1/2 4^-lambda <dx_p, dy_q>, p = (a-1) >> lambda, q = (b-1) >> lambda.
 // In single precision it runs the difference form (Q = K(a,b) - K(a,b-1)),
 // like the chained kernel.  This kernel is the comparison baseline for the
-// chained FP32 kernel and the general path for shapes that kernel has no
-// instance for (uneven lengths, long pairs, high dyadic orders, wide d).
+// chained FP32 kernel and the general path for shapes that the others have no
+// instance for: high dyadic orders, wide d, and in double precision uneven
+// lengths, the surface and increments too large for a block (wave64.cu).
 #include "sigk_internal.cuh"
 
 namespace sigk {

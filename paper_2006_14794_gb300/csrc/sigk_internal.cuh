@@ -276,6 +276,24 @@ cudaError_t launch_strip_bwd(const PairSrc &src, int64_t n, int lam, int dtype, 
                              cudaStream_t st, int64_t max_la, int64_t max_lb, int64_t rowsA,
                              int64_t rowsB, int coef_path);
 
+// FP64 pairs of uniform lengths, La <= Lb (wave64.cu): the schedule for these
+// sizes (false: no instance, or the increments fit no block) and the launches.
+struct Wave64Plan {
+    int R, lam, pre, wpc, cluster, threads, vrows, smem;
+};
+bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kernel, Wave64Plan &p);
+cudaError_t launch_wave64(const PairSrc &src, const Wave64Plan &p, int64_t n, double *out, cudaStream_t st);
+// the backward: grid blocks of the workspace hold `slot` doubles each
+constexpr int64_t W64_BWD_WS_CAP = 2LL << 30;
+struct Wave64BwdPlan {
+    int R, lam, W, threads, vrows, smem;
+    int64_t slot, grid;
+};
+bool wave64_bwd_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kernel, Wave64BwdPlan &p);
+// adds into dA / dB (zeroed by the caller, or on accumulate what they hold)
+cudaError_t launch_wave64_bwd(const PairSrc &src, const Wave64BwdPlan &p, int64_t n, const double *gout, double *dA,
+                              double *dB, void *ws, cudaStream_t st);
+
 // Support reduction (support.cu): largest N one block holds, and the launch.
 int64_t support_max_n(int dtype);
 cudaError_t launch_support(const void *K, const void *alpha, void *beta, int64_t N, double gamma,
