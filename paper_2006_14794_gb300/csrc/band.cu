@@ -11,16 +11,16 @@
 // macro-step pos of a pair (columns pos*NG .. pos*NG + NG - 1 of the padded
 // coarse grid, NG = R / 2^lambda coarse rows per lane), window w, group g of
 // lane l is at coarse cell (P, Q) = (l*NG + g, pos*NG + w - g).  Slot (pair,
-// pos, lane) holds these NG x NG values as [w][g]: in each window a lane reads
-// NG consecutive floats, and a warp reads 32 slots of one pair position, so
-// every load is a full 32-byte sector.  Cells with Q < 0 (pos = 0, w < g) are
-// the previous pair's last columns, which rows that have not turned over yet
-// still need: they are stored in the next pair's slot 0, so the chain reads
-// pair k's coefficients, tail included, from slots (k, 0 .. TperR - 1) and
-// (k + 1, 0).  Virtual rows and columns (padding, as in fwd_chain.cu) hold 0.
+// pos, lane) holds these NG x NG values as [w][g]; where its elements lie:
+// band_row, band_off.  Cells with Q < 0 (pos = 0, w < g) are the previous pair's
+// last columns, which rows that have not turned over yet still need: they are
+// stored in the next pair's slot 0, so the chain reads pair k's coefficients,
+// tail included, from slots (k, 0 .. TperR - 1) and (k + 1, 0).  Virtual rows
+// and columns (padding, as in fwd_chain.cu) hold 0.  What the sweeps write per
+// cell (dk/dc, the surface's nodes) goes to the same slots, TperR + 1 a pair,
+// each lane's kept whole ([pair][pos][lane][w][g]).
 #include <string.h>
 
-#include "rbf.cuh"
 #include "sigk_internal.cuh"
 #include "tc5.cuh"
 
@@ -29,8 +29,6 @@ namespace sigk {
 namespace {
 
 constexpr int BAND_WARPS = 2;   // warps per CTA of the sweep
-constexpr int BC_THREADS = 256; // threads per CTA of the contraction
-constexpr int BC_DC = 32;       // channels staged per pass of the contraction
 
 struct BandCoefArgs {
     PairSrc src;
@@ -40,165 +38,11 @@ struct BandCoefArgs {
     float *band;
 };
 
-// Shared memory of the contraction: increments of one pair, channel-major.
-//   dx: [BC_DC][32*NG + 4]      row P (padded, virtual rows zero)
-//   dy: [BC_DC][ystride]        index Q + NG - 1 (zeros for Q < 0 and Q >= NQ)
-template <int NG>
-__host__ __device__ constexpr int bc_xstride() { return 32 * NG + 4; }
-__host__ __device__ inline int bc_ystride(int NQ, int NG) { return ((NQ + 2 * NG + 3) / 4) * 4 + 4; }
-
-// Position of row P of the staged row increments: with 8 rows per lane the
-// two 16-byte halves of a lane's rows are swapped for lanes 4..7 of every 8,
-// so the 8 lanes of a shared-memory phase read 8 distinct bank quads.
-template <int NG>
-__device__ __forceinline__ int bc_xpos(int P) {
-    if constexpr (NG == 8) return P ^ (((P >> 5) & 1) << 2);
-    else return P;
-}
-
 // Order of the groups inside a window of a slot: g and g + NG/2 side by side
 // (the sweeps carry groups g and g + NG/2 as one float2).
 template <int NG>
 __host__ __device__ constexpr int band_gpos(int g) {
     return g < NG / 2 ? 2 * g : 2 * (g - NG / 2) + 1;
-}
-
-// One thread per slot (lane l, position pos) of the pair: the NG x NG cells
-// (l*NG + g, pos*NG + w - g), each a d-term dot product of increments.
-// Position TperR is the pair's tail (the cells with w < g there), written into
-// slot 0 of the next pair.  Each block takes a contiguous run of pairs, so
-// consecutive pairs of a Gram row share the row path and its staged
-// increments.
-template <int NG>
-__global__ void __launch_bounds__(BC_THREADS, 2) band_coef_kernel(BandCoefArgs a) {
-    extern __shared__ __align__(16) float bcs[];
-    constexpr int NPP = 32 * NG;
-    constexpr int XS = bc_xstride<NG>();
-    constexpr int SLOT = NG * NG;
-    const int YS = bc_ystride(a.NQ, NG);
-    float *dxs = bcs;
-    float *dys = bcs + BC_DC * XS;
-    const int64_t d = a.src.d;
-    const int nslots = 32 * (a.TperR + 1);
-    const int64_t per = (a.n_pairs + gridDim.x - 1) / gridDim.x;
-    const int64_t kbeg = (int64_t)blockIdx.x * per;
-    const int64_t kend = kbeg + per < a.n_pairs ? kbeg + per : a.n_pairs;
-    int64_t staged_x = -1;   // point row of the row path whose increments dxs holds (d <= BC_DC)
-    for (int64_t k = kbeg; k < kend; ++k) {
-        const PairRef pr = pair_ref(a.src, k);
-        const float *x = (const float *)a.src.A + pr.a_row0 * d;
-        const float *y = (const float *)a.src.B + pr.b_row0 * d;
-        const int nx = (int)pr.la - 1, ny = (int)pr.lb - 1;   // real coarse rows / columns
-        for (int base = 0; base < nslots; base += BC_THREADS) {
-            const int u = base + (int)threadIdx.x;
-            const int l = u & 31, pos = u >> 5;
-            float acc[NG][NG];
-#pragma unroll
-            for (int w = 0; w < NG; ++w)
-#pragma unroll
-                for (int g = 0; g < NG; ++g) acc[w][g] = 0.f;
-            for (int64_t c0 = 0; c0 < d; c0 += BC_DC) {
-                if (d > BC_DC || base == 0) {
-                    __syncthreads();
-                    // stage channels c0 .. c0 + BC_DC - 1 (consecutive threads take
-                    // consecutive channels of a row: coalesced loads)
-                    if (d > BC_DC || staged_x != pr.a_row0) {
-                        for (int v = threadIdx.x; v < BC_DC * NPP; v += BC_THREADS) {
-                            const int P = v / BC_DC, c = v - (v / BC_DC) * BC_DC;
-                            const int p = P - a.vrows;
-                            float e = 0.f;
-                            if (p >= 0 && p < nx && c0 + c < d)
-                                e = __ldg(x + (int64_t)(p + 1) * d + c0 + c) - __ldg(x + (int64_t)p * d + c0 + c);
-                            dxs[c * XS + bc_xpos<NG>(P)] = e;
-                        }
-                        staged_x = pr.a_row0;
-                    }
-                    for (int v = threadIdx.x; v < BC_DC * YS; v += BC_THREADS) {
-                        const int iq = v / BC_DC, c = v - (v / BC_DC) * BC_DC;
-                        const int q = iq - (NG - 1) - a.NQV;   // real column
-                        float e = 0.f;
-                        if (q >= 0 && q < ny && iq - (NG - 1) < a.NQ && c0 + c < d)
-                            e = __ldg(y + (int64_t)(q + 1) * d + c0 + c) - __ldg(y + (int64_t)q * d + c0 + c);
-                        dys[c * YS + iq] = e;
-                    }
-                    __syncthreads();
-                }
-                if (u < nslots) {
-                    const int cn = (int)(d - c0 < BC_DC ? d - c0 : BC_DC);
-#pragma unroll 2
-                    for (int c = 0; c < cn; ++c) {
-                        float xv[NG], yv[2 * NG];
-                        const float *xr = dxs + c * XS + l * NG;
-                        const float *yr = dys + c * YS + pos * NG;   // Q = pos*NG - (NG-1) + j
-                        if constexpr (NG >= 4) {
-                            const int sw = NG == 8 ? ((l >> 2) & 1) : 0;   // see bc_xpos
-#pragma unroll
-                            for (int h = 0; h < NG / 4; ++h) {
-                                const float4 v = *reinterpret_cast<const float4 *>(xr + 4 * (h ^ sw));
-                                xv[4 * h] = v.x; xv[4 * h + 1] = v.y; xv[4 * h + 2] = v.z; xv[4 * h + 3] = v.w;
-                            }
-#pragma unroll
-                            for (int h = 0; h < NG / 2; ++h) {
-                                const float4 v = *reinterpret_cast<const float4 *>(yr + 4 * h);
-                                yv[4 * h] = v.x; yv[4 * h + 1] = v.y; yv[4 * h + 2] = v.z; yv[4 * h + 3] = v.w;
-                            }
-                        } else {
-                            const float2 v = *reinterpret_cast<const float2 *>(xr);
-                            xv[0] = v.x; xv[1] = v.y;
-                            const float2 w0 = *reinterpret_cast<const float2 *>(yr);
-                            const float2 w1 = *reinterpret_cast<const float2 *>(yr + 2);
-                            yv[0] = w0.x; yv[1] = w0.y; yv[2] = w1.x; yv[3] = w1.y;
-                        }
-#pragma unroll
-                        for (int w = 0; w < NG; ++w)
-#pragma unroll
-                            for (int g = 0; g < NG; ++g)
-                                acc[w][g] = fmaf(xv[g], yv[w - g + NG - 1], acc[w][g]);
-                    }
-                }
-            }
-            if (u >= nslots) continue;
-#pragma unroll
-            for (int w = 0; w < NG; ++w)
-#pragma unroll
-                for (int g = 0; g < NG; ++g) acc[w][g] = scheme_coef(acc[w][g] * a.scale, a.src.scheme);
-            if (pos < a.TperR && pos > 0) {
-                float4 *dst = reinterpret_cast<float4 *>(a.band + (((k * a.TperR + pos) * 32) + l) * SLOT);
-                if constexpr (NG >= 4) {
-#pragma unroll
-                    for (int w = 0; w < NG; ++w)
-#pragma unroll
-                        for (int h = 0; h < NG / 4; ++h)
-                            dst[w * (NG / 4) + h] = make_float4(acc[w][2 * h], acc[w][2 * h + NG / 2],
-                                                                acc[w][2 * h + 1], acc[w][2 * h + 1 + NG / 2]);
-                } else {
-                    dst[0] = make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1]);
-                }
-            } else if (pos == 0) {
-                // the pair's own cells (w >= g); the cells w < g belong to the
-                // previous pair's block, which writes them (pair 0: zeros)
-                float *dst = a.band + ((k * a.TperR) * 32 + l) * SLOT;
-#pragma unroll
-                for (int w = 0; w < NG; ++w)
-#pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        if (w >= g) dst[w * NG + band_gpos<NG>(g)] = acc[w][g];
-                        else if (k == 0) dst[w * NG + band_gpos<NG>(g)] = 0.f;
-                    }
-            } else {
-                // pos == TperR: the tail (w < g) into slot 0 of the next pair; after
-                // the last pair the slot has no owner, so its own cells are zeroed
-                float *dst = a.band + (((k + 1) * a.TperR) * 32 + l) * SLOT;
-#pragma unroll
-                for (int w = 0; w < NG; ++w)
-#pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        if (w < g) dst[w * NG + band_gpos<NG>(g)] = acc[w][g];
-                        else if (k == a.n_pairs - 1) dst[w * NG + band_gpos<NG>(g)] = 0.f;
-                    }
-            }
-        }
-    }
 }
 
 struct BandArgs {
@@ -222,11 +66,13 @@ struct BandArgs {
 
 constexpr int BAND_CK = 8;   // macro-steps between checkpoints of the forward state
 
+// Window w of the slot at p (band_row).
 template <int NG>
-__device__ __forceinline__ void load_window(float (&v)[NG], const float *p) {
+__device__ __forceinline__ void load_window(float (&v)[NG], const float *slot, int w) {
+    const float *p = slot + band_off(w * NG);
     if constexpr (NG == 8) {
         const float4 a = __ldcs(reinterpret_cast<const float4 *>(p));
-        const float4 b = __ldcs(reinterpret_cast<const float4 *>(p) + 1);
+        const float4 b = __ldcs(reinterpret_cast<const float4 *>(p + 128));
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
         v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
     } else if constexpr (NG == 4) {
@@ -300,7 +146,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
     // slot that holds that pair's tail)
     auto slot = [&](int kk, int pp) -> const float * {
         if (kk < 0 || kk > np || (kk == np && pp != 0)) return nullptr;
-        return a.band + (((k0 + kk) * TperR + pp) * 32 + lane) * (int64_t)SLOT;
+        return a.band + band_row((k0 + kk) * TperR + pp, lane, NG);
     };
 
     int kl = (lane == 0) ? 0 : -((lane + TperR - 1) / TperR);
@@ -309,7 +155,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
         const float *p0 = slot(kl, pos);
 #pragma unroll
         for (int w = 0; w < NG; ++w) {
-            if (p0) load_window<NG>(cb[w], p0 + w * NG);
+            if (p0) load_window<NG>(cb[w], p0, w);
             else
 #pragma unroll
                 for (int g = 0; g < NG; ++g) cb[w][g] = 0.f;
@@ -333,7 +179,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
                 CO[g] = CN[g];
                 CN[g] = make_float2(cb[w][2 * g], cb[w][2 * g + 1]);   // groups g, g + NH
             }
-            if (pn) load_window<NG>(cb[w], pn + w * NG);
+            if (pn) load_window<NG>(cb[w], pn, w);
             else
 #pragma unroll
                 for (int g = 0; g < NG; ++g) cb[w][g] = 0.f;
@@ -416,23 +262,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
     }
 }
 
-template <int NG>
-cudaError_t launch_coef(const BandCoefArgs &a, int sms, cudaStream_t st) {
-    const int smem = (int)sizeof(float) * BC_DC * (bc_xstride<NG>() + bc_ystride(a.NQ, NG));
-    auto kern = band_coef_kernel<NG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BC_THREADS, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    int64_t grid = (int64_t)sms * per_sm;
-    if (grid > a.n_pairs) grid = a.n_pairs;
-    kern<<<(int)grid, BC_THREADS, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-// The same band on the fifth-generation tensor cores (tcgen05), for d <= 64.
+// The band's coefficients on the fifth-generation tensor cores (tcgen05), for d <= 64.
 // A block takes a contiguous run of pairs; per pair, per 128-row tile of the
 // padded rows: the row increments (scaled by 1/2 4^-lambda) are split into
 // TF32 hi and lo parts and staged once, then the padded columns are walked in
@@ -491,8 +321,8 @@ __global__ void __launch_bounds__(BT5_T, 1) band_coef_tc5_kernel(BandCoefArgs a,
             for (int v = tid; v < 32 * SLOT; v += BT5_T) {
                 const int l = v / SLOT, e = v - l * SLOT, w = e / NG, gp = e - w * NG;
                 const int g = (gp & 1) ? gp / 2 + NG / 2 : gp / 2;   // inverse of band_gpos
-                if (k == 0 && w < g) a.band[(int64_t)l * SLOT + e] = 0.f;
-                if (k == a.n_pairs - 1 && w >= g) a.band[(((k + 1) * TperR) * 32 + l) * (int64_t)SLOT + e] = 0.f;
+                if (k == 0 && w < g) a.band[band_row(0, l, NG) + band_off(e)] = 0.f;
+                if (k == a.n_pairs - 1 && w >= g) a.band[band_row((k + 1) * TperR, l, NG) + band_off(e)] = 0.f;
             }
         }
         for (int P0 = 0; P0 < NPP && !failed; P0 += BT5_M) {
@@ -585,12 +415,12 @@ __global__ void __launch_bounds__(BT5_T, 1) band_coef_tc5_kernel(BandCoefArgs a,
                     const float *srow = St + (P - P0) * BT5_SS;
                     // destination slot: the pair's own, or (the tail) the next pair's slot 0
                     const bool tail = pos == TperR;
-                    float *dst = a.band + ((tail ? (k + 1) * TperR : k * TperR + pos) * 32 + l) * (int64_t)SLOT + gp;
+                    float *dst = a.band + band_row(tail ? (k + 1) * TperR : k * TperR + pos, l, NG);
 #pragma unroll
                     for (int w = 0; w < NG; ++w) {
                         const int Q = pos * NG + w - g;
                         const bool own = tail ? (w < g) : (Q >= 0);
-                        if (own && Q >= Q0 && Q < Q0 + BT5_N) dst[w * NG] = srow[Q - Q0];
+                        if (own && Q >= Q0 && Q < Q0 + BT5_N) dst[band_off(w * NG + gp)] = srow[Q - Q0];
                     }
                 }
                 __syncthreads();
@@ -822,7 +652,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
     };
     auto slot_ptr = [&](int kk, int pp) -> const float * {
         if (kk < 0 || kk > np || (kk == np && pp != 0)) return nullptr;
-        return a.band + (((k0 + kk) * TperR + pp) * 32 + lane) * (int64_t)SLOT;
+        return a.band + band_row((k0 + kk) * TperR + pp, lane, NG);
     };
     // window w of macro-step m (slot src, null outside the chain) into buffer m & 1;
     // with window NG-1 also the last row's Q
@@ -832,16 +662,16 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float *dd = dst + 4 * chunk(2 * w + h);
-                if (src) cp_async<16>(dd, src + w * NG + 4 * h);
+                if (src) cp_async<16>(dd, src + band_off(w * NG + 4 * h));
                 else *reinterpret_cast<float4 *>(dd) = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         } else if constexpr (NG == 4) {
             float *dd = dst + 4 * chunk(w);
-            if (src) cp_async<16>(dd, src + w * NG);
+            if (src) cp_async<16>(dd, src + band_off(w * NG));
             else *reinterpret_cast<float4 *>(dd) = make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
             float *dd = dst + 2 * w;
-            if (src) cp_async<8>(dd, src + w * NG);
+            if (src) cp_async<8>(dd, src + band_off(w * NG));
             else *reinterpret_cast<float2 *>(dd) = make_float2(0.f, 0.f);
         }
         if (w == NG - 1 && lane == 31) {
@@ -1581,13 +1411,13 @@ bool band_geometry(int64_t La, int64_t Lb, int lam, int rows_per_lane, BandPlan 
 
 // workspace: a 256-byte header (the status word of bounded waits), then the band
 int64_t band_bytes(const BandPlan &p, int64_t n_pairs) {
-    return 256 + (int64_t)sizeof(float) * (n_pairs * p.TperR + 1) * p.slot_floats;
+    return 256 + (int64_t)sizeof(float) * (n_pairs * p.TperR + 32) * p.slot_floats;
 }
 
 // The surface's band-layout values (TperR + 1 slots per pair) after the band:
 // their float offset from the band's start, and the whole workspace.
 int64_t band_surface_offset(const BandPlan &p, int64_t n_pairs) {
-    return ((n_pairs * p.TperR + 1) * p.slot_floats + 63) / 64 * 64;
+    return ((n_pairs * p.TperR + 32) * p.slot_floats + 63) / 64 * 64;
 }
 int64_t band_surface_bytes(const BandPlan &p, int64_t n_pairs) {
     return 256 + (int64_t)sizeof(float) *
@@ -1595,81 +1425,18 @@ int64_t band_surface_bytes(const BandPlan &p, int64_t n_pairs) {
 }
 
 namespace {
-// The band coefficients: the FMA contraction, or on request (coef_path 3,
-// d <= 64) the tcgen05 kernel.  The FMA kernel is the default: it runs two
-// blocks per SM and overlaps staging with arithmetic, where the tensor-core
-// kernel's one block per SM serialises staging, MMAs and the scattered band
-// write-back (measured on the 128 x 128 MMD Gram, d = 32: 1.5 vs 4.8 ms).
-// Band layout of the RBF-lifted coefficients (rbf.cuh): coarse cell (p, q) of
-// pair k is the padded cell (P, Q) = (p + vrows, q + NQV), read by lane P / NG
-// as group g = P % NG at the position pos and window w with pos NG + w = Q + g;
-// pos = TperR is the pair's tail, in slot 0 of pair k + 1.
-template <int NG>
-struct BandRbfLayout {
-    PairSrc src;
-    float *band;
-    int TperR, NQV, vrows;
-    struct Geo {
-        const float *rows, *cols;
-        int nx, ny;
-        int64_t k;
-    };
-    struct Row {
-        int64_t lane_off;   // (lane) * NG^2 + band_gpos(g)
-        int gr;             // group of the row within its lane
-    };
-    __device__ Geo geo(int64_t k) const {
-        const PairRef pr = pair_ref(src, k);
-        Geo g;
-        g.rows = (const float *)src.A + pr.a_row0 * src.d;
-        g.cols = (const float *)src.B + pr.b_row0 * src.d;
-        g.nx = (int)pr.la - 1;
-        g.ny = (int)pr.lb - 1;
-        g.k = k;
-        return g;
-    }
-    __device__ Row row(const Geo &, int p) const {
-        const int P = p + vrows;
-        Row r;
-        r.gr = P % NG;
-        r.lane_off = (int64_t)(P / NG) * (NG * NG) + band_gpos<NG>(r.gr);
-        return r;
-    }
-    __device__ void store(const Geo &g, const Row &r, int q, float c) const {
-        const int t = q + NQV + r.gr, pos = t / NG, w = t % NG;
-        const int64_t slot = pos < TperR ? g.k * TperR + pos : (g.k + 1) * TperR;
-        band[slot * (32 * NG * NG) + r.lane_off + w * NG] = c;
-    }
-};
-
-template <int NG>
-cudaError_t launch_band_rbf(const BandCoefArgs &c, int sms, cudaStream_t st) {
-    BandRbfLayout<NG> lay;
-    lay.src = c.src;
-    lay.band = c.band;
-    lay.TperR = c.TperR;
-    lay.NQV = c.NQV;
-    lay.vrows = c.vrows;
-    const size_t bytes = sizeof(float) * (size_t)(c.n_pairs * c.TperR + 1) * 32 * NG * NG;
-    return launch_rbf_coef<float>(lay, c.n_pairs, c.src.La - 1, c.src.Lb - 1, c.src.d, c.src.sigma,
-                                  (double)c.scale, c.src.scheme, c.band, bytes, sms, st);
-}
-
-cudaError_t launch_band_coef(const BandCoefArgs &c, int NG, int sms, int *status, cudaStream_t st,
+// The band coefficients: the FP32 kernel of band_coef.cu, or on request
+// (coef_path 3, d <= 64, linear kernel) the tcgen05 kernel, whose one block per
+// SM serialises staging, MMAs and the scattered band write-back (measured on
+// the 128 x 128 MMD Gram, d = 32: 4.8 ms against 2.3).
+cudaError_t launch_band_coef(const BandCoefArgs &c, const BandPlan &p, int sms, int *status, cudaStream_t st,
                              int coef_path) {
-    if (c.src.kernel == SIGK_KERNEL_RBF) {
-        if (NG == 8) return launch_band_rbf<8>(c, sms, st);
-        if (NG == 4) return launch_band_rbf<4>(c, sms, st);
-        return launch_band_rbf<2>(c, sms, st);
-    }
-    if (coef_path == 3 && c.src.d <= 64) {
-        if (NG == 8) return launch_coef_tc5<8>(c, sms, status, st);
-        if (NG == 4) return launch_coef_tc5<4>(c, sms, status, st);
+    if (c.src.kernel == SIGK_KERNEL_LINEAR && coef_path == 3 && c.src.d <= 64) {
+        if (p.NG == 8) return launch_coef_tc5<8>(c, sms, status, st);
+        if (p.NG == 4) return launch_coef_tc5<4>(c, sms, status, st);
         return launch_coef_tc5<2>(c, sms, status, st);
     }
-    if (NG == 8) return launch_coef<8>(c, sms, st);
-    if (NG == 4) return launch_coef<4>(c, sms, st);
-    return launch_coef<2>(c, sms, st);
+    return launch_band_coefs(c.src, p, c.n_pairs, c.band, sms, st);
 }
 }  // namespace
 
@@ -1693,7 +1460,7 @@ cudaError_t launch_band_f32(const PairSrc &src, const BandPlan &p, int64_t n_pai
     c.vrows = p.vrows;
     c.scale = 0.5f / (float)(1 << (2 * p.lam));
     c.band = band;
-    if ((e = launch_band_coef(c, p.NG, sms, status, st, coef_path)) != cudaSuccess) return e;
+    if ((e = launch_band_coef(c, p, sms, status, st, coef_path)) != cudaSuccess) return e;
 
     const int per_sm = band_occupancy_of(p.R, p.lam);
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -2015,7 +1782,7 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
         c.vrows = p.vrows;
         c.scale = scale;
         c.band = band;
-        if ((e = launch_band_coef(c, p.NG, sms, status, st, coef_path)) != cudaSuccess) return e;
+        if ((e = launch_band_coef(c, p, sms, status, st, coef_path)) != cudaSuccess) return e;
         // 2. the forward sweep, keeping what the adjoint needs
         const int64_t warps = (int64_t)sms * per_sm * BAND_WARPS;
         BandArgs f;

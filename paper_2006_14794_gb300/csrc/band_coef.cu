@@ -1,0 +1,532 @@
+// The band form's coefficients (FP32): every coarse cell's c of every pair of
+// a launch, written straight into the banded buffer that the sweeps of band.cu
+// read (its layout: there), from the paths' points; linear kernel and RBF lift.
+//
+// A thread owns the slots of a lane l at one or more consecutive positions: the
+// NG x NG cells (l NG + g, pos NG + w - g) of each, rows g and g + NG/2 as one
+// float2 (FFMA2: the FP32 pipe's rate at half the issue slots, and the band's own
+// order).  A warp covers 8 lanes by 4 positions (narrow lanes: 16 by 2): a read
+// of the rows' float4s or of a position's column pairs is then one wavefront
+// (32 lanes of one position took four for the rows), and a store meets 11 rows
+// of the band where 32 lanes of one position would meet 32: those stores, not
+// the FMAs, were what bounded the earlier form of this kernel.  Columns are kept
+// as the pairs (column, column - NG/2) that rows g and g + NG/2 meet in a window.
+// A block (one per SM at the larger sizes) walks a contiguous run of units, a
+// unit being a pair's positions or, of long pairs, an even share of at most
+// TILE of them.  Consecutive pairs of a Gram row share the row path and keep
+// its staged values, and the next unit's column points arrive by cp.async
+// while the current one is computed.
+//
+// RBF lift (Sec. 2.2; rbf_second_difference in sigk_internal.cuh): the second
+// difference over cell (p, q) is kappa(p,q) (a b + (1 + a)(1 + b) e) with
+//   a = expm1(A), A = s (2 <u,dy> - |dy|^2),   b = expm1(B), B = -s (2 <u,dx> + |dx|^2),
+//   e = expm1(C), C = 2 s <dx,dy>,             u = x_p - y_q,
+// and neighbouring cells share all but C: A(p+1,q) = A(p,q) + C(p,q), B(p,q+1)
+// = B(p,q) + C(p,q), kappa(p,q+1) = kappa(p,q) (1 + a(p,q)), so
+//   a(p+1,q) = a + (1 + a) e,   b(p,q+1) = b + (1 + b) e.
+// Only a slot's first cell of each row takes kappa, a and b from the points,
+// and its first row takes a in every column; every other cell adds its own
+// <dx,dy> and about 14 operations.  Carried values keep FP32 accuracy while a
+// and b stay of order one or below, so a slot with an |A| or |B| above
+// KC_CARRY, or C's that could add up to it, forms every cell from its points.  Before, each cell formed all six sums
+// (9 d operations), three series and two exponentials, 183 instructions at
+// d = 8, and stored its value alone into a zero-filled band.
+//
+// Measured: the lift over 3840 pairs of 256-point paths, d = 32, order 1, 2.9 ->
+// 1.16 ms; over a 256 x 256 Gram of 128-point paths, d = 8, order 2, 7.4 (zero
+// fill included) -> 2.9 ms; the linear kernel over the 3840 pairs 0.62 -> 0.54 ms
+// (0.67 in this form with 32 lanes of one position a warp).
+// Padding: rows and columns outside the path repeat its end points, so their
+// increments and with them c are exactly zero.
+#include "sigk_internal.cuh"
+
+namespace sigk {
+
+namespace {
+
+constexpr int KC_CH = 32;          // channels staged at a time
+// Lanes a warp covers, positions a thread, most positions a unit, most warps a
+// block.  12 warps a SM have 168 registers each; a pair of 33 positions (256
+// points at dyadic order 1) is 36 warp items, three a warp.
+template <int NG, bool RBF>
+struct KcShape {
+    static constexpr int LW = NG == 8 ? 8 : 16, NP = NG == 8 ? 1 : NG == 4 ? 2 : 4;
+    static constexpr int GP = 32 / LW * NP;   // positions a warp item
+    static constexpr int TILE = 36, WARPS = NG == 8 ? 12 : 9, MINB = NG == 8 ? 1 : 2;
+};
+constexpr float KC_CARRY = 0.5f;   // see above: a, b <= e^1 - 1 along a slot
+
+struct KcArgs {
+    PairSrc src;
+    float *band;
+    int64_t n_pairs;
+    int TperR, NQV, vrows;
+    int tiles, tp, passes;   // units a pair, positions a unit, positions a warp
+    float scale, s;       // 1/2 4^-lambda, 1/(2 sigma^2)
+};
+
+__device__ __forceinline__ void kc_cp4(float *dst, const float *src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void kc_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void kc_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+template <int NG>
+__host__ __device__ constexpr int kc_xs() { return 32 * NG + 4; }
+// a unit's columns, from NG - 1 before its first position's, and one more for
+// the last increment (tp: rounded up to whole threads' positions)
+__host__ __device__ inline int kc_ys(int tp, int NG) { return (tp * NG + NG + 3) / 4 * 4 + 4; }
+// per channel: rows' increments, the next unit's column points, pairs of column
+// increments; lift: and this unit's column points (as pairs too where they
+// fit: not for NG = 8), row points, the squares
+template <int NG>
+__host__ __device__ constexpr int kc_pp() { return NG == 8 ? 1 : 2; }
+template <int NG, bool RBF>
+__host__ __device__ inline int kc_smem_floats(int tp, int nch) {
+    const int ys = kc_ys(tp, NG), xs = kc_xs<NG>();
+    return RBF ? nch * ((3 + kc_pp<NG>()) * ys + 2 * xs) + ys + xs : nch * (3 * ys + xs);
+}
+// threads that share a staged point's channels: the power of two at or above nc (32 at most)
+__device__ __forceinline__ int kc_group(int nc) { return nc > 16 ? 32 : nc > 8 ? 16 : nc > 4 ? 8 : 4; }
+
+// Where padded row P is staged: a lane's rows in the band's order (g, g + NG/2
+// side by side), and with 8 of them the two 16-byte halves swapped for lanes
+// 4..7 of every 8, so that the 8 lanes of a phase read 8 distinct bank quads.
+template <int NG>
+__device__ __forceinline__ int kc_xpos(int P) {
+    const int l = P / NG, g = P - l * NG;
+    const int at = g < NG / 2 ? 2 * g : 2 * (g - NG / 2) + 1;
+    return l * NG + (NG == 8 ? at ^ (l & 4) : at);
+}
+// the lane's rows as pairs (h, h + NG/2)
+template <int NG>
+__device__ __forceinline__ void kc_rows(float2 (&v)[NG / 2], const float *r, int l) {
+    if constexpr (NG >= 4) {
+        const int sw = NG == 8 ? (l >> 2) & 1 : 0;
+#pragma unroll
+        for (int h = 0; h < NG / 4; ++h) {
+            const float4 t = *reinterpret_cast<const float4 *>(r + l * NG + 4 * (h ^ sw));
+            v[2 * h] = make_float2(t.x, t.y);
+            v[2 * h + 1] = make_float2(t.z, t.w);
+        }
+    } else {
+        v[0] = *reinterpret_cast<const float2 *>(r + l * NG);
+    }
+}
+// N column pairs from r (16-byte aligned for NG > 2)
+template <int NG, int N>
+__device__ __forceinline__ void kc_cols(float2 (&v)[N], const float2 *r) {
+    if constexpr (NG == 2) {
+#pragma unroll
+        for (int h = 0; h < N; ++h) v[h] = r[h];
+        return;
+    }
+#pragma unroll
+    for (int h = 0; h < N / 2; ++h) {
+        const float4 t = *reinterpret_cast<const float4 *>(r + 2 * h);
+        v[2 * h] = make_float2(t.x, t.y);
+        v[2 * h + 1] = make_float2(t.z, t.w);
+    }
+    if constexpr (N % 2) v[N - 1] = r[N - 1];
+}
+
+__device__ __forceinline__ float2 kc2(float v) { return make_float2(v, v); }
+// e^x - 1 of two values, |x| <= KC_CARRY / 2^(8 - D) or so: the Taylor series
+// through x^D / D!, whose truncation x^D / (D + 1)! is below 3e-9 of the value
+// for D = 8 and |x| <= 1/2, D = 7 and 1/4, D = 6 and 1/8, D = 5 and 1/16.
+template <int D>
+__device__ __forceinline__ float2 kc_expm1(float2 x) {
+    constexpr float F[9] = {1.f, 1.f, 1.f / 2.f, 1.f / 6.f, 1.f / 24.f, 1.f / 120.f, 1.f / 720.f, 1.f / 5040.f,
+                            1.f / 40320.f};
+    float2 p = kc2(F[D]);
+#pragma unroll
+    for (int i = D - 1; i >= 1; --i) p = __ffma2_rn(p, x, kc2(F[i]));
+    return __fmul2_rn(p, x);
+}
+
+// A slot's values v[w][h] = (cell (w, h), cell (w, h + NG/2)) to the band: its
+// own slot; position 0 leaves the cells w < g to the previous pair (pair 0:
+// zeros); position TperR is the pair's tail (w < g), in slot 0 of the next
+// pair (after the last pair the slot has no owner and its other cells are
+// zeroed).
+template <int NG>
+__device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs, int TperR, int pos, int l,
+                                         const float2 (&v)[NG][NG / 2]) {
+    constexpr int SLOT = NG * NG, NH = NG / 2;
+    float *dst = band + band_row(k * TperR + pos, l, NG);   // (the tail: the next pair's slot 0)
+    if (pos > 0 && pos < TperR) {
+#pragma unroll
+        for (int i = 0; i < SLOT / 4; ++i) {
+            const float2 u = v[2 * i / NH][2 * i % NH], t = v[(2 * i + 1) / NH][(2 * i + 1) % NH];
+            *reinterpret_cast<float4 *>(dst + band_off(4 * i)) = make_float4(u.x, u.y, t.x, t.y);
+        }
+        return;
+    }
+    const bool tail = pos == TperR;
+    const bool zero = tail ? k == n_pairs - 1 : k == 0;
+#pragma unroll
+    for (int w = 0; w < NG; ++w)
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            const float c = g < NH ? v[w][g % NH].x : v[w][g % NH].y;
+            const int at = band_off(w * NG + 2 * (g % NH) + g / NH);
+            if (tail ? w < g : w >= g) dst[at] = c;
+            else if (zero) dst[at] = 0.f;
+        }
+}
+
+// The slot's cells one by one from the points (RBF lift), stored as kc_store does.
+template <int NG>
+__device__ __noinline__ void kc_slot_direct(const KcArgs &a, int64_t k, int64_t row0, int64_t col0, int pos, int l) {
+    constexpr int SLOT = NG * NG;
+    const int64_t d = a.src.d;
+    const int ny = (int)a.src.Lb - 1;
+    const bool tail = pos == a.TperR;
+    float *dst = a.band + band_row(k * a.TperR + pos, l, NG);   // tail: slot 0 of the next pair
+    for (int e = 0; e < SLOT; ++e) {
+        const int w = e / NG, g = e - w * NG;
+        const bool other = tail ? w >= g : (pos == 0 && w < g);   // the neighbour pair's cell
+        if (other && k != (tail ? a.n_pairs - 1 : 0)) continue;
+        const int p = l * NG + g - a.vrows, q = pos * NG + w - g - a.NQV;
+        float c = 0.f;
+        if (!other && p >= 0 && q >= 0 && q < ny) {
+            const float *x = (const float *)a.src.A + (row0 + p) * d, *y = (const float *)a.src.B + (col0 + q) * d;
+            float uu = 0.f, ux = 0.f, uy = 0.f, xy = 0.f, xx = 0.f, yy = 0.f;
+            for (int64_t i = 0; i < d; ++i) {
+                const float u = x[i] - y[i], dx = x[i + d] - x[i], dy = y[i + d] - y[i];
+                uu = fmaf(u, u, uu); ux = fmaf(u, dx, ux); uy = fmaf(u, dy, uy);
+                xy = fmaf(dx, dy, xy); xx = fmaf(dx, dx, xx); yy = fmaf(dy, dy, yy);
+            }
+            c = scheme_coef(rbf_second_difference(uu, ux, uy, xy, xx, yy, a.s) * a.scale, a.src.scheme);
+        }
+        dst[band_off(w * NG + 2 * (g % (NG / 2)) + g / (NG / 2))] = c;
+    }
+}
+
+// A slot's sums <dx,dy> into its coefficients (RBF lift).  Everything is done
+// for rows h and h + NG/2 at once; at window w row g is one column ahead of row
+// g + 1, so a(g + 1) of the next window is a(g) + (1 + a(g)) e(g) of this one.
+// The slot's first cells: rows h, h + NG/2 at entry NG - 1 - h of the column
+// pairs, and row 0 in windows NG/2 + i and i at entry NG + NG/2 - 1 + i.  Their
+// sums come from the staged channels, or (more channels than are staged at
+// once) from the points.  False where the slot was formed cell by cell.
+template <int NG>
+__device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcArgs &a, int64_t k, const PairRef &pr,
+                                        int pos, int l, const float *xi, const float *xp, const float *xx,
+                                        const float2 *yi, const float *yp, const float *yy, int YS) {
+    constexpr int NH = NG / 2, XS = kc_xs<NG>();
+    const float s = a.s, s2 = 2.f * s;
+    const float2 minus = kc2(-1.f);
+    float2 uu[NH], ux[NH], uy[NH], ur[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) uu[h] = ux[h] = uy[h] = ur[h] = kc2(0.f);
+    if (a.src.d <= KC_CH) {
+#pragma unroll 1
+        for (int c = 0; c < (int)a.src.d; ++c) {
+            float2 xv[NH], dv[NH];
+            kc_rows<NG>(xv, xp + c * XS, l);
+            kc_rows<NG>(dv, xi + c * XS, l);
+            const float *q = yp + c * YS * kc_pp<NG>();
+            const float2 *e = yi + c * YS;
+            auto pts = [&](int j) {
+                if constexpr (kc_pp<NG>() == 2) return reinterpret_cast<const float2 *>(q)[j];
+                else return make_float2(q[j], q[j - NH]);
+            };
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const float2 u = __ffma2_rn(pts(NG - 1 - h), minus, xv[h]);
+                uu[h] = __ffma2_rn(u, u, uu[h]);
+                ux[h] = __ffma2_rn(u, dv[h], ux[h]);
+                uy[h] = __ffma2_rn(u, e[NG - 1 - h], uy[h]);
+                const float2 t = __ffma2_rn(pts(NG + NH - 1 + h), minus, kc2(xv[0].x));
+                ur[h] = __ffma2_rn(t, e[NG + NH - 1 + h], ur[h]);
+            }
+        }
+    } else {
+        const int64_t d = a.src.d;
+        const int ny = (int)a.src.Lb - 1, P0 = l * NG - a.vrows, Q0 = pos * NG - (NG - 1) - a.NQV;
+        auto row = [&](int g) { return (const float *)a.src.A + (pr.a_row0 + (P0 + g < 0 ? 0 : P0 + g)) * d; };
+        auto col = [&](int j) {
+            const int q = Q0 + j;
+            return (const float *)a.src.B + (pr.b_row0 + (q < 0 ? 0 : q > ny ? ny : q)) * d;
+        };
+#pragma unroll 1
+        for (int64_t c = 0; c < d; ++c) {
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const int ja = NG - 1 - h, jb = NH - 1 - h, jr = NG + NH - 1 + h, js = NG - 1 + h;
+                const float *ra = row(h), *rb = row(h + NH);
+                const float2 x = make_float2(ra[c], rb[c]);
+                const float2 dx = make_float2(P0 + h < 0 ? 0.f : ra[d + c] - x.x, P0 + h + NH < 0 ? 0.f : rb[d + c] - x.y);
+                const float2 y = make_float2(col(ja)[c], col(jb)[c]), z = make_float2(col(jr)[c], col(js)[c]);
+                const float2 dy = make_float2(col(ja + 1)[c] - y.x, col(jb + 1)[c] - y.y);
+                const float2 dz = make_float2(col(jr + 1)[c] - z.x, col(js + 1)[c] - z.y);
+                const float2 u = __ffma2_rn(y, minus, x), t = __ffma2_rn(z, minus, kc2(row(0)[c]));
+                uu[h] = __ffma2_rn(u, u, uu[h]);
+                ux[h] = __ffma2_rn(u, dx, ux[h]);
+                uy[h] = __ffma2_rn(u, dy, uy[h]);
+                ur[h] = __ffma2_rn(t, dz, ur[h]);
+            }
+        }
+    }
+    float far = 0.f;
+#pragma unroll
+    for (int w = 0; w < NG; ++w)
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            acc[w][h] = __fmul2_rn(acc[w][h], kc2(s2));   // C
+            far = fmaxf(far, fmaxf(fabsf(acc[w][h].x), fabsf(acc[w][h].y)));
+        }
+    far *= NG;
+    float2 av[NH], bv[NH], kap[NH], top[NH], sq[NH];
+    kc_rows<NG>(sq, xx, l);
+    auto arg = [&](float2 sum, float2 sqr, float sign) {   // sign s (2 sum + sign' square), its size noted
+        const float2 v = __fmul2_rn(kc2(sign * s), __ffma2_rn(kc2(2.f), sum, __fmul2_rn(kc2(-sign), sqr)));
+        far = fmaxf(far, fmaxf(fabsf(v.x), fabsf(v.y)));
+        return v;
+    };
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+        av[h] = arg(uy[h], make_float2(yy[NG - 1 - h], yy[NH - 1 - h]), 1.f);
+        top[h] = arg(ur[h], make_float2(yy[NG + NH - 1 + h], yy[NG - 1 + h]), 1.f);
+        bv[h] = arg(ux[h], sq[h], -1.f);
+    }
+    if (far > KC_CARRY) {
+        kc_slot_direct<NG>(a, k, pr.a_row0, pr.b_row0, pos, l);
+        return false;
+    }
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+        av[h] = kc_expm1<8>(av[h]);
+        bv[h] = kc_expm1<8>(bv[h]);
+        top[h] = kc_expm1<8>(top[h]);
+        kap[h] = make_float2(a.scale * __expf(-s * uu[h].x), a.scale * __expf(-s * uu[h].y));
+    }
+#pragma unroll
+    for (int w = 0; w < NG; ++w) {
+        float2 an[NH];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const float2 e = kc_expm1<NG == 8 ? 5 : NG == 4 ? 6 : 7>(acc[w][h]);
+            const float2 ea = __ffma2_rn(av[h], e, e), eb = __ffma2_rn(bv[h], e, e);
+            acc[w][h] = __fmul2_rn(kap[h], __ffma2_rn(av[h], bv[h], __ffma2_rn(bv[h], ea, ea)));
+            kap[h] = __ffma2_rn(kap[h], av[h], kap[h]);
+            an[h] = __fadd2_rn(av[h], ea);
+            bv[h] = __fadd2_rn(bv[h], eb);
+        }
+        // row g + 1 takes row g's; row 0 its own of the next column
+#pragma unroll
+        for (int h = NH - 1; h >= 1; --h) av[h] = an[h - 1];
+        av[0] = make_float2(w + 1 < NH ? top[w + 1].y : w + 1 < NG ? top[w + 1 - NH].x : 0.f, an[NH - 1].x);
+    }
+    return true;
+}
+
+template <int NG, bool RBF>
+__global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>::MINB) band_coef_kernel(KcArgs a) {
+    extern __shared__ __align__(16) float kc_sm[];
+    constexpr int NPP = 32 * NG, XS = kc_xs<NG>(), NP = KcShape<NG, RBF>::NP, NH = NG / 2;
+    using Sh = KcShape<NG, RBF>;
+    const int nt = blockDim.x, tid = threadIdx.x, warp = tid >> 5;
+    const int lw = tid & (Sh::LW - 1), jw = (tid & 31) / Sh::LW;   // lane and position in the warp's item
+    const int64_t d = a.src.d;
+    const int nch = d < KC_CH ? (int)d : KC_CH, YS = kc_ys(a.tp, NG);
+    float *xi = kc_sm;                                            // row increments (linear: scaled)
+    float *y0 = xi + nch * XS;                                    // the next unit's column points
+    float2 *yi = reinterpret_cast<float2 *>(y0 + nch * YS);       // pairs of column increments
+    float *yp = reinterpret_cast<float *>(yi + nch * YS);         // RBF: this unit's column points,
+    float *xp = yp + nch * YS * kc_pp<NG>();                      // row points, and the squared
+    float *xx = xp + nch * XS, *yy = xx + XS;                     // increments of rows and columns
+    const int64_t units = a.n_pairs * a.tiles, per = (units + gridDim.x - 1) / gridDim.x;
+    const int64_t ubeg = (int64_t)blockIdx.x * per;
+    const int64_t uend = ubeg + per < units ? ubeg + per : units;
+    if (ubeg >= uend) return;
+    const int ny = (int)a.src.Lb - 1;
+    const bool once = d <= KC_CH;   // all channels staged at once
+
+    auto stage_x = [&](int64_t row0, int64_t c0, int nc) {
+        const float *x = (const float *)a.src.A + row0 * d + c0;
+        const int gs = kc_group(nc), c = tid & (gs - 1);
+        if (c < nc)
+            for (int P = tid / gs; P < NPP; P += nt / gs) {
+                const int p = P - a.vrows;
+                const float *r = x + (int64_t)(p < 0 ? 0 : p) * d + c;
+                const float e = p >= 0 ? __ldg(r + d) - __ldg(r) : 0.f;
+                xi[c * XS + kc_xpos<NG>(P)] = RBF ? e : e * a.scale;
+                if (RBF) xp[c * XS + kc_xpos<NG>(P)] = __ldg(r);
+            }
+    };
+    // tile t's column points, ends repeated, into y0[c][iq], Q = t tp NG + iq - (NG - 1)
+    auto fetch_y = [&](int64_t row0, int t, int64_t c0, int nc) {
+        const float *y = (const float *)a.src.B + row0 * d + c0;
+        const int gs = kc_group(nc), c = tid & (gs - 1), Q0 = t * a.tp * NG - (NG - 1) - a.NQV;
+        if (c < nc)
+            for (int iq = tid / gs; iq < YS; iq += nt / gs) {
+                int q = Q0 + iq;
+                q = q < 0 ? 0 : (q > ny ? ny : q);
+                kc_cp4(y0 + c * YS + iq, y + (int64_t)q * d + c);
+            }
+        kc_commit();
+    };
+    // the pairs (column iq, column iq - NG/2) from the fetched points; RBF: and the
+    // squared increments, over the channels so far (rows' where they were staged)
+    auto pair_y = [&](int64_t c0, int nc, bool rows) {
+        for (int iq = tid; iq < YS; iq += nt) {
+            float sq = RBF && c0 > 0 ? yy[iq] : 0.f;
+            const int ib = iq >= NH ? iq - NH : 0, hi = iq + 1 < YS ? 1 : 0;
+            for (int c = 0; c < nc; ++c) {
+                const float *y = y0 + c * YS;
+                const float ya = y[iq], yb = y[ib];
+                const float2 e = make_float2(y[iq + hi] - ya, y[ib + 1] - yb);
+                yi[c * YS + iq] = e;
+                if (RBF) {
+                    if constexpr (kc_pp<NG>() == 2)
+                        reinterpret_cast<float2 *>(yp)[c * YS + iq] = make_float2(ya, yb);
+                    else
+                        yp[c * YS + iq] = ya;
+                    sq = fmaf(e.x, e.x, sq);
+                }
+            }
+            if (RBF) yy[iq] = sq;
+        }
+        if (RBF && rows)
+            for (int P = tid; P < NPP; P += nt) {
+                float sq = c0 > 0 ? xx[P] : 0.f;
+                for (int c = 0; c < nc; ++c) sq = fmaf(xi[c * XS + P], xi[c * XS + P], sq);
+                xx[P] = sq;   // in the staged order, as xi
+            }
+    };
+
+    int64_t kn = ubeg / a.tiles;          // the next unit's pair and tile
+    int tn = (int)(ubeg - kn * a.tiles);
+    PairRef pr = pair_ref(a.src, kn);
+    int64_t staged = -1;   // the row path whose values xi (and xp) hold
+    if (once) fetch_y(pr.b_row0, tn, 0, (int)d);
+    for (int64_t u = ubeg; u < uend; ++u) {
+        const PairRef cur = pr;
+        const int64_t k = kn;
+        const int t = tn;
+        const bool more = u + 1 < uend;
+        if (more && ++tn == a.tiles) {
+            tn = 0;
+            pr = pair_ref(a.src, ++kn);
+        }
+        if (once) {
+            kc_wait();
+            __syncthreads();   // this unit's columns are here, and the last unit's readers are done
+            const bool fresh = staged != cur.a_row0;
+            if (fresh) {
+                stage_x(cur.a_row0, 0, (int)d);
+                staged = cur.a_row0;
+                if (RBF) __syncthreads();
+            }
+            pair_y(0, (int)d, fresh);
+            __syncthreads();
+            if (more) fetch_y(pr.b_row0, tn, 0, (int)d);
+        }
+        for (int pass = 0; pass < a.passes; ++pass) {
+            // the warp's item: a block of lanes and a group of positions
+            const int item = pass * (nt >> 5) + warp, l = item % (32 / Sh::LW) * Sh::LW + lw;
+            const int first = item / (32 / Sh::LW) * Sh::GP + jw * NP;
+            const bool live = first < a.tp && t * a.tp + first <= a.TperR;
+            const int rel = live ? first : 0, pos = t * a.tp + rel;
+            float2 acc[NP][NG][NH];
+#pragma unroll
+            for (int n = 0; n < NP; ++n)
+#pragma unroll
+                for (int w = 0; w < NG; ++w)
+#pragma unroll
+                    for (int h = 0; h < NH; ++h) acc[n][w][h] = make_float2(0.f, 0.f);
+            for (int64_t c0 = 0; c0 < d; c0 += KC_CH) {
+                const int nc = d - c0 < KC_CH ? (int)(d - c0) : KC_CH;
+                if (!once) {
+                    __syncthreads();
+                    stage_x(cur.a_row0, c0, nc);
+                    fetch_y(cur.b_row0, t, c0, nc);
+                    kc_wait();
+                    __syncthreads();
+                    pair_y(c0, nc, true);
+                    __syncthreads();
+                }
+                const float2 *yr = yi + rel * NG;   // entry j: columns Q = pos NG - (NG - 1) + j and Q - NG/2
+#pragma unroll 2
+                for (int c = 0; c < nc; ++c) {
+                    float2 xv[NH], yv[(NP + 1) * NG - NH];
+                    kc_rows<NG>(xv, xi + c * XS, l);
+                    kc_cols<NG>(yv, yr + c * YS + NH);
+#pragma unroll
+                    for (int n = 0; n < NP; ++n)
+#pragma unroll
+                        for (int w = 0; w < NG; ++w)
+#pragma unroll
+                            for (int h = 0; h < NH; ++h)
+                                acc[n][w][h] = __ffma2_rn(xv[h], yv[n * NG + w - h + NG - 1 - NH], acc[n][w][h]);
+                }
+            }
+            if (!live) continue;
+#pragma unroll
+            for (int n = 0; n < NP; ++n) {
+                if (n > 0 && (rel + n >= a.tp || pos + n > a.TperR)) break;
+                if constexpr (RBF)
+                    if (!kc_lift<NG>(acc[n], a, k, cur, pos + n, l, xi, xp, xx, yi + (rel + n) * NG,
+                                     yp + (rel + n) * NG * kc_pp<NG>(), yy + (rel + n) * NG, YS))
+                        continue;
+                if (a.src.scheme != SIGK_SCHEME_EXPLICIT) {
+#pragma unroll
+                    for (int w = 0; w < NG; ++w)
+#pragma unroll
+                        for (int h = 0; h < NH; ++h)
+                            acc[n][w][h] = make_float2(scheme_coef(acc[n][w][h].x, a.src.scheme),
+                                                       scheme_coef(acc[n][w][h].y, a.src.scheme));
+                }
+                kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos + n, l, acc[n]);
+            }
+        }
+    }
+}
+
+template <int NG, bool RBF>
+cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
+    KcArgs a = a0;
+    const int npos = a.TperR + 1;
+    using Sh = KcShape<NG, RBF>;
+    a.tiles = (npos + Sh::TILE - 1) / Sh::TILE;
+    a.tp = ((npos + a.tiles - 1) / a.tiles + Sh::NP - 1) / Sh::NP * Sh::NP;
+    const int items = (a.tp + Sh::GP - 1) / Sh::GP * (32 / Sh::LW);
+    a.passes = (items + Sh::WARPS - 1) / Sh::WARPS;
+    const int warps = (items + a.passes - 1) / a.passes;
+    const int smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, (int)(a.src.d < KC_CH ? a.src.d : KC_CH));
+    auto kern = band_coef_kernel<NG, RBF>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem)) != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    int64_t grid = (int64_t)sms * per_sm;
+    if (grid > a.n_pairs * a.tiles) grid = a.n_pairs * a.tiles;
+    kern<<<(int)grid, warps * 32, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_band_coefs(const PairSrc &src, const BandPlan &p, int64_t n_pairs, float *band, int sms,
+                              cudaStream_t st) {
+    KcArgs a;
+    a.src = src;
+    a.band = band;
+    a.n_pairs = n_pairs;
+    a.TperR = p.TperR;
+    a.NQV = p.NQV;
+    a.vrows = p.vrows;
+    a.tiles = a.tp = a.passes = 1;
+    a.scale = 0.5f / (float)(1 << (2 * p.lam));
+    a.s = (float)(0.5 / (src.sigma * src.sigma));
+    const bool rbf = src.kernel == SIGK_KERNEL_RBF;
+    if (p.NG == 8) return rbf ? launch<8, true>(a, sms, st) : launch<8, false>(a, sms, st);
+    if (p.NG == 4) return rbf ? launch<4, true>(a, sms, st) : launch<4, false>(a, sms, st);
+    return rbf ? launch<2, true>(a, sms, st) : launch<2, false>(a, sms, st);
+}
+
+}  // namespace sigk

@@ -97,12 +97,21 @@ struct PairRef {
     int64_t out0, out1;     // output slots (out1 = -1 when only one)
 };
 
-// Upper-triangle enumeration (i <= j) of an n x n symmetric Gram matrix.
+// Upper-triangle enumeration (i <= j) of an n x n symmetric Gram matrix.  The
+// row is estimated from the inverse of its offset and corrected to the exact
+// one: in FP32 for n <= 4096 (there the estimate is off by a few rows at most;
+// an FP64 instruction takes a warp 64 cycles here, and every pair of the FP32
+// sweeps asks for its row), in FP64 beyond.
 __host__ __device__ inline void sym_index(int64_t k, int64_t n, int64_t &i, int64_t &j) {
     // row i holds n - i entries, starting at off(i) = i*n - i*(i-1)/2
-    double nn = (double)n;
-    double disc = (2.0 * nn + 1.0) * (2.0 * nn + 1.0) - 8.0 * (double)k;
-    int64_t ii = (int64_t)((2.0 * nn + 1.0 - sqrt(disc > 0 ? disc : 0.0)) * 0.5);
+    int64_t ii;
+    if (n <= 4096) {
+        const int m = 2 * (int)n + 1, disc = m * m - 8 * (int)k;   // below 2^27
+        ii = (int64_t)(((float)m - sqrtf(disc > 0 ? (float)disc : 0.f)) * 0.5f);
+    } else {
+        const double nn = (double)n, disc = (2.0 * nn + 1.0) * (2.0 * nn + 1.0) - 8.0 * (double)k;
+        ii = (int64_t)((2.0 * nn + 1.0 - sqrt(disc > 0 ? disc : 0.0)) * 0.5);
+    }
     if (ii < 0) ii = 0;
     if (ii > n - 1) ii = n - 1;
     while (ii > 0 && ii * n - ii * (ii - 1) / 2 > k) --ii;
@@ -172,13 +181,29 @@ struct BandPlan {
     int NQ, NQV, vrows;     // padded coarse columns, virtual columns, virtual coarse rows
     int64_t slot_floats;    // floats per (pair, position) slot row: 32 lanes x NG x NG
 };
+// The coefficient band: slot (pair k, position pos) of lane l, NG x NG floats,
+// element i = window NG + place in the window.  The slots of a launch's pairs
+// follow one another (linear position s = k TperR + pos), and lane l's slot s is
+// in row s + l: the row that holds what the 32 lanes of a sweep warp, one
+// position apart, read in one macro-step, four floats of a lane at a time next
+// to the neighbour lanes' (a window is one or two 512-byte runs; slots kept
+// whole per lane cost a sweep load or a producer store 32 cache lines instead).
+__host__ __device__ inline int64_t band_row(int64_t s, int l, int NG) {
+    return (s + l) * (32 * NG * NG) + 4 * l;
+}
+// offset of element i in it
+__host__ __device__ constexpr int band_off(int i) { return (i / 4) * 128 + i % 4; }
 // Geometry only (no device query); false when the band form has no instance.
 bool band_geometry(int64_t La, int64_t Lb, int lam, int rows_per_lane, BandPlan &p);
 int64_t band_bytes(const BandPlan &p, int64_t n_pairs);
 // with the solution surface: the band, then the surface values in the band layout
 int64_t band_surface_offset(const BandPlan &p, int64_t n_pairs);
 int64_t band_surface_bytes(const BandPlan &p, int64_t n_pairs);
-// coef_path 3: coefficients on tcgen05 (d <= 64); otherwise the FMA contraction
+// The coefficients of n_pairs pairs into the band (band_coef.cu): every slot of
+// the launch's pairs and the tail slot after the last is written.
+cudaError_t launch_band_coefs(const PairSrc &src, const BandPlan &p, int64_t n_pairs, float *band, int sms,
+                              cudaStream_t st);
+// coef_path 3: coefficients on tcgen05 (d <= 64); otherwise the FP32 kernel
 // surf (optional): the solution surface, node (i, j) of pair k (of the call)
 // at surf[k s_pair + i s_a + j s_b]; nodes on row or column 0 are not written.
 // It needs band_surface_bytes of workspace instead of band_bytes.
