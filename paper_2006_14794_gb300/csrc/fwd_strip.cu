@@ -35,6 +35,7 @@
 #include "rbf.cuh"
 #include "sigk_internal.cuh"
 #include "tc5.cuh"
+#include "tile_gemm.cuh"
 
 namespace sigk {
 
@@ -63,8 +64,11 @@ struct PairPlan {
     int nw;                  // windows (coefficient diagonals) per strip
     int swap;                // 1: the rows refine the B path (src.B), columns the A path
     int64_t s_off;           // backward: start of its checkpoints of the forward state
-    int64_t g_off;           // backward: start of its dense dk/dG [nx][ny]
+    int64_t g_off;           // backward: start of its dense dk/dG [nx][gbar_ld(ny)]
 };
+
+// dk/dG's row stride: rows start on 16 bytes
+__host__ __device__ inline int gbar_ld(int ny) { return (ny + 3) / 4 * 4; }
 
 // totals[]: the sums of the coefficient, boundary-row, strip, sums and dk/dG
 // sizes over all pairs
@@ -104,7 +108,7 @@ __global__ void plan_kernel(PairSrc src, int64_t n, PairPlan *plan, int64_t *tot
         p.bnd_off = p.ns > 0 ? (int64_t)(ck ? p.ns : p.ns - 1) * p.nj * 2 : 0;
         p.strip_base = p.ns;
         p.s_off = ck ? (int64_t)p.ns * ((p.nj + TH - 1 + ck - 1) / ck) * TH * 2 : 0;
-        p.g_off = (int64_t)p.nx * p.ny;
+        p.g_off = (int64_t)p.nx * gbar_ld(p.ny);
         plan[k] = p;
     }
     __syncthreads();
@@ -930,7 +934,7 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_adj_kernel(AdjArgs<T> 
             for (int g = 0; g < NG; ++g) {
                 const int p = prow0 + NG * lane + g, q = w - NG * lane - g;
                 if (p >= 0 && p < pp.nx && q >= 0 && q < pp.ny)
-                    a.gbar[pp.g_off + (int64_t)p * pp.ny + q] =
+                    a.gbar[pp.g_off + (int64_t)p * gbar_ld(pp.ny) + q] =
                         a.scheme != SIGK_SCHEME_EXPLICIT ? gN[g] * scheme_dcoef(cn[g], a.scheme) : gN[g];
                 gN[g] = gO[g];
                 gO[g] = 0;
@@ -940,6 +944,7 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_adj_kernel(AdjArgs<T> 
     }
 }
 
+// (FP64; FP32 takes grad_chain_tile_kernel below)
 // Chain rule through G(p,q) = <dx_p, dy_q>: dk/d dx_p = f sum_q Gbar(p,q) dy_q,
 // dk/d dy_q = f sum_p Gbar(p,q) dx_p (f = incoming gradient x 1/2 4^-lambda),
 // then to the points, atomically (a path appears in many pairs).  Both
@@ -971,6 +976,7 @@ __global__ void __launch_bounds__(256) grad_chain_kernel(PairSrc src, const Pair
         if (pp.ns == 0) continue;
         const T f = gout[pp.out0] * scale;
         const T *G = gbar + pp.g_off;
+        const int64_t ld = gbar_ld(pp.ny);
         const V4 *xi = reinterpret_cast<const V4 *>(pp.swap ? incB : incA) + pp.a_row0 * D4;
         const V4 *yi = reinterpret_cast<const V4 *>(pp.swap ? incA : incB) + pp.b_row0 * D4;
         T *gx = pp.swap ? dB : dA;
@@ -1000,7 +1006,7 @@ __global__ void __launch_bounds__(256) grad_chain_kernel(PairSrc src, const Pair
                             const int orow = r0 + i, red = k0 + j;
                             T v = 0;
                             if (orow < nrow && red < nred)
-                                v = pass == 0 ? G[(int64_t)orow * pp.ny + red] : G[(int64_t)red * pp.ny + orow];
+                                v = pass == 0 ? G[(int64_t)orow * ld + red] : G[(int64_t)red * ld + orow];
                             Gs[i][j] = v;
                         }
                         for (int u = threadIdx.x; u < CT * 8; u += blockDim.x) {
@@ -1035,6 +1041,99 @@ __global__ void __launch_bounds__(256) grad_chain_kernel(PairSrc src, const Pair
                             atomicAdd(&gout_pts[(int64_t)(orow + 1) * d + c], v);
                             atomicAdd(&gout_pts[(int64_t)orow * d + c], -v);
                         }
+                    }
+                }
+            }
+        }
+    }
+}
+
+// The same chain rule in FP32, on the tiles of tile_gemm.cuh: 128 rows of dk/d dx
+// (or dk/d dy) by NT channels a block, blockIdx.x over (contraction, row tile,
+// channel block, share of the reduction), blockIdx.y over the pairs.  ksplit
+// shares only where the tiles alone leave SMs idle.  64 pairs of 4096 points, d
+// = 64: 15.7 ms on the 64 x 64 tiles above, 5.7 here (3.4 at the FP32 pipe's peak).
+template <int NT>
+__global__ void __launch_bounds__(TG_THREADS, 2) grad_chain_tile_kernel(const PairPlan *plan, int64_t n_pairs,
+                                                                        int64_t d, const float *gbar,
+                                                                        const float *incA, const float *incB,
+                                                                        const float *gout, float *dA, float *dB,
+                                                                        float scale, int ksplit) {
+    using Tile = TileGemm<NT>;
+    __shared__ __align__(16) typename Tile::Shared sh;
+    const int64_t D4 = (d + 3) / 4;
+    const int ncb = (int)((d + NT - 1) / NT);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t k = blockIdx.y; k < n_pairs; k += gridDim.y) {
+        const PairPlan pp = plan[k];
+        if (pp.ns == 0) continue;
+        const int tx = (pp.nx + TG_M - 1) / TG_M, ty = (pp.ny + TG_M - 1) / TG_M;
+        const int ld = gbar_ld(pp.ny);
+        const float f = gout[pp.out0] * scale;
+        const float *G = gbar + pp.g_off;
+        for (int64_t wi = blockIdx.x; wi < (int64_t)(tx + ty) * ncb * ksplit; wi += gridDim.x) {
+            const int tile = (int)(wi / (ncb * ksplit)), rem = (int)(wi - (int64_t)tile * ncb * ksplit);
+            const bool rows = tile < tx;   // rows p of dk/d dx over q; else rows q of dk/d dy over p
+            const bool onA = rows != (pp.swap != 0);
+            float *pts = onA ? dA : dB;
+            if (!pts) continue;
+            pts += (rows ? pp.a_row0 : pp.b_row0) * d;
+            const float4 *other = reinterpret_cast<const float4 *>(onA ? incB : incA) +
+                                  (rows ? pp.b_row0 : pp.a_row0) * D4;
+            const int r0 = (rows ? tile : tile - tx) * TG_M, cb = rem / ksplit * (NT / 4);
+            const int nrow = rows ? pp.nx : pp.ny, nred = rows ? pp.ny : pp.nx;
+            const int nsl = (nred + TG_K - 1) / TG_K, ks = rem % ksplit;
+            const int s0 = (int)((int64_t)nsl * ks / ksplit), s1 = (int)((int64_t)nsl * (ks + 1) / ksplit);
+            Tile t;
+            t.clear();
+            auto load_b = [&](int i, float4 (&v)[NT / 32]) {
+#pragma unroll
+                for (int u = 0; u < NT / 32; ++u) {
+                    const int kk = (s0 + i) * TG_K + Tile::b_line(u), c4 = cb + Tile::b_quad(u);
+                    v[u] = kk < nred && c4 < D4 ? __ldg(other + (int64_t)kk * D4 + c4) : zero;
+                }
+            };
+            if (rows) {
+                t.template run<true>(sh, s1 - s0, [&](int i, float4 (&v)[4]) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int p = r0 + Tile::template line<true>(u);
+                        const int q = (s0 + i) * TG_K + 4 * Tile::template quad<true>(u);
+                        v[u] = zero;
+                        if (p < nrow && q < nred) {
+                            v[u] = __ldcs(reinterpret_cast<const float4 *>(G + (int64_t)p * ld + q));
+                            // the row's padding is unwritten
+                            if (q + 1 >= nred) v[u].y = 0.f;
+                            if (q + 2 >= nred) v[u].z = 0.f;
+                            if (q + 3 >= nred) v[u].w = 0.f;
+                        }
+                    }
+                }, load_b);
+            } else {
+                t.template run<false>(sh, s1 - s0, [&](int i, float4 (&v)[4]) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int p = (s0 + i) * TG_K + Tile::template line<false>(u);
+                        const int q = r0 + 4 * Tile::template quad<false>(u);
+                        v[u] = p < nred && q < nrow ? __ldcs(reinterpret_cast<const float4 *>(G + (int64_t)p * ld + q))
+                                                    : zero;
+                    }
+                }, load_b);
+            }
+            // dk/dx_i = dk/d dx_{i-1} - dk/d dx_i, the thread's eight rows at once
+            const int rb = r0 + 8 * (threadIdx.x >> 4);
+#pragma unroll
+            for (int n = 0; n < Tile::TN; ++n) {
+                const int c = cb * 4 + Tile::TN * (threadIdx.x & 15) + n;
+                float prev = 0.f;
+                if (c < d && rb < nrow) {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        if (rb + r >= nrow) break;
+                        const float v = t.out(r, n) * f;
+                        atomicAdd(pts + (int64_t)(rb + r) * d + c, prev - v);
+                        prev = v;
+                        if (r == 7 || rb + r + 1 == nrow) atomicAdd(pts + (int64_t)(rb + r + 1) * d + c, v);
                     }
                 }
             }
@@ -1495,7 +1594,7 @@ static StripLayout strip_layout_bwd(int64_t n, int64_t max_la, int64_t max_lb, i
     L.ckpt = off;
     off += al256(n * ns * ((nj + TH - 1 + ck - 1) / ck) * TH * 2 * es);
     L.gbar = off;
-    off += al256(n * nx * ny * es);
+    off += al256(n * nx * gbar_ld((int)ny) * es);
     L.total = off;
     return L;
 }
@@ -1786,12 +1885,30 @@ static cudaError_t launch_strip_bwd_t(const PairSrc &src, int64_t n, void *ws, c
     }
     const T scale = (T)0.5 / (T)(1LL << (2 * LAM));
     {
-        // tiles of the longest pair in x, pairs in y
-        const int64_t lx = max_la > max_lb ? max_la : max_lb;
-        const int64_t tiles = 2 * ((lx - 1 + CT - 1) / CT) * ((D4 + 7) / 8);
-        const dim3 grid((unsigned)(tiles < 1 ? 1 : tiles), (unsigned)(n < 65535 ? n : 65535));
-        grad_chain_kernel<T><<<grid, 256, 0, st>>>(src, plan, n, (const T *)(w + L.gbar), incA, incB, gout, dA,
-                                                   dB, scale);
+        const int64_t lx = max_la > max_lb ? max_la : max_lb, ly = max_la > max_lb ? max_lb : max_la;
+        const unsigned gy = (unsigned)(n < 65535 ? n : 65535);
+        if constexpr (sizeof(T) == 4) {
+            const int nt = src.d > 32 ? 64 : 32;
+            const int64_t tiles = ((lx - 1 + TG_M - 1) / TG_M + (ly - 1 + TG_M - 1) / TG_M) * ((src.d + nt - 1) / nt);
+            // shares of the reduction (at least four slices each) until two blocks an SM have work
+            int64_t ks = (2 * (int64_t)sms + tiles * n - 1) / (tiles * n);
+            const int64_t most = (ly - 1 + 4 * TG_K - 1) / (4 * TG_K);
+            if (ks > most) ks = most;
+            if (ks < 1) ks = 1;
+            const dim3 grid((unsigned)(tiles * ks), gy);
+            if (nt == 64)
+                grad_chain_tile_kernel<64><<<grid, TG_THREADS, 0, st>>>(plan, n, src.d, (const float *)(w + L.gbar),
+                                                                       incA, incB, gout, dA, dB, scale, (int)ks);
+            else
+                grad_chain_tile_kernel<32><<<grid, TG_THREADS, 0, st>>>(plan, n, src.d, (const float *)(w + L.gbar),
+                                                                       incA, incB, gout, dA, dB, scale, (int)ks);
+        } else {
+            // tiles of the longest pair in x, pairs in y
+            const int64_t tiles = 2 * ((lx - 1 + CT - 1) / CT) * ((D4 + 7) / 8);
+            const dim3 grid((unsigned)(tiles < 1 ? 1 : tiles), gy);
+            grad_chain_kernel<T><<<grid, 256, 0, st>>>(src, plan, n, (const T *)(w + L.gbar), incA, incB, gout, dA,
+                                                       dB, scale);
+        }
     }
     return cudaGetLastError();
 }
