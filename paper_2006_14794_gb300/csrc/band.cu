@@ -23,6 +23,7 @@
 
 #include "sigk_internal.cuh"
 #include "tc5.cuh"
+#include "tile_gemm.cuh"
 
 namespace sigk {
 
@@ -98,6 +99,28 @@ __device__ __forceinline__ void store_window(float *dst, const float2 (&v)[NG / 
     }
 }
 
+// Macro-steps of coefficients in flight per warp, by cp.async into shared memory,
+// where a macro-step is too short (R < 16 steps) for a load issued one ahead
+// to arrive in time: 32 steps' worth.  0: registers, refilled window by window
+// a macro-step ahead (R = 16, and the 8 KB slots of R = NG = 8).  24 x 17 paths of
+// 50 and 71 points, order 1 (R = 4): the checkpointing sweep 90 -> 18 us, the
+// adjoint 72 -> 49 us.
+template <int R, int NG>
+__host__ __device__ constexpr int band_ring() { return R < 16 && NG <= 4 ? 32 / R : 0; }
+
+template <int NBYTES>
+__device__ __forceinline__ void cp_async(void *dst, const void *src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (NBYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(NBYTES) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // The sweep: fwd_chain.cu's chain_f32_kernel with its staging and dot
 // products replaced by one coefficient vector per window, prefetched one
 // macro-step ahead into the registers the window has just consumed.
@@ -141,18 +164,34 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
     for (int g = 0; g < NH; ++g) { CN[g] = make_float2(0.f, 0.f); CO[g] = CN[g]; }
     float pK = 1.f, pQ = 0.f;
 
-    // slot of local pair kk at position pp, or null outside the chain (its
-    // first pair's rows before they start, and after the last pair except the
-    // slot that holds that pair's tail)
-    auto slot = [&](int kk, int pp) -> const float * {
-        if (kk < 0 || kk > np || (kk == np && pp != 0)) return nullptr;
-        return a.band + band_row((k0 + kk) * TperR + pp, lane, NG);
+    // the lane's slot in macro-step m (linear position m - lane of the chain), or
+    // null outside the chain (its first pair's rows before they start, and after
+    // the last pair except the slot that holds that pair's tail)
+    const float *band0 = a.band + band_row(k0 * TperR - lane, lane, NG);
+    auto slot = [&](int64_t m) -> const float * {
+        return m >= lane && m - lane <= (int64_t)np * TperR ? band0 + m * (32 * SLOT) : nullptr;
+    };
+    constexpr int D = band_ring<R, NG>();
+    __shared__ __align__(16) float ring[D ? BAND_WARPS * D * 32 * SLOT : 1];
+    float *rw = ring + (D ? warp * D * 32 * SLOT : 0) + 4 * lane;
+    auto fetch = [&](int64_t m) {   // into the ring, quads of a lane 128 floats apart as in the band
+        const float *p = slot(m);
+        float *dst = rw + (int)(m % (D ? D : 1)) * 32 * SLOT;
+#pragma unroll
+        for (int i = 0; i < SLOT; i += 4) {
+            if (p) cp_async<16>(dst + band_off(i), p + band_off(i));
+            else *reinterpret_cast<float4 *>(dst + band_off(i)) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        cp_commit();
     };
 
     int kl = (lane == 0) ? 0 : -((lane + TperR - 1) / TperR);
     int pos = -lane - kl * TperR;
-    {
-        const float *p0 = slot(kl, pos);
+    if constexpr (D > 0) {
+#pragma unroll
+        for (int m = 0; m < D - 1; ++m) fetch(m);
+    } else {
+        const float *p0 = slot(0);
 #pragma unroll
         for (int w = 0; w < NG; ++w) {
             if (p0) load_window<NG>(cb[w], p0, w);
@@ -167,7 +206,22 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
 
     for (int64_t m = 0; m < total_m; ++m) {
         const bool trans = (pos == 0);
-        const float *pn = (pos + 1 == TperR) ? slot(kl + 1, 0) : slot(kl, pos + 1);
+        const float *pn = nullptr;
+        if constexpr (D > 0) {
+            fetch(m + D - 1);
+            cp_wait<D - 1>();   // macro-step m's have landed
+            const float *src = rw + (int)(m % D) * 32 * SLOT;
+#pragma unroll
+            for (int i = 0; i < SLOT; i += 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(src + band_off(i));
+                cb[i / NG][i % NG] = v.x;
+                cb[(i + 1) / NG][(i + 1) % NG] = v.y;
+                cb[(i + 2) / NG][(i + 2) % NG] = v.z;
+                cb[(i + 3) / NG][(i + 3) % NG] = v.w;
+            }
+        } else {
+            pn = slot(m + 1);
+        }
         // exit states go to the pair the rows leave (kl - 1), when it is one of the chain's
         float *ex = (SAVE && trans && kl >= 1 && kl <= np)
                         ? a.exitk + ((k0 + kl - 1) * 32 + lane) * (int64_t)R : nullptr;
@@ -179,10 +233,12 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
                 CO[g] = CN[g];
                 CN[g] = make_float2(cb[w][2 * g], cb[w][2 * g + 1]);   // groups g, g + NH
             }
-            if (pn) load_window<NG>(cb[w], pn, w);
-            else
+            if constexpr (D == 0) {
+                if (pn) load_window<NG>(cb[w], pn, w);
+                else
 #pragma unroll
-                for (int g = 0; g < NG; ++g) cb[w][g] = 0.f;
+                    for (int g = 0; g < NG; ++g) cb[w][g] = 0.f;
+            }
 #pragma unroll
             for (int jj = 0; jj < S; ++jj) {
                 const int j = w * S + jj;
@@ -260,6 +316,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
             ++kl;
         }
     }
+    if constexpr (D > 0) cp_wait<0>();
 }
 
 // The band's coefficients on the fifth-generation tensor cores (tcgen05), for d <= 64.
@@ -504,18 +561,6 @@ struct BandAdjArgs {
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-template <int NBYTES>
-__device__ __forceinline__ void cp_async(void *dst, const void *src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (NBYTES == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(NBYTES) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // dk/dc from the adjoint's band layout into the dense Gbar the chain-rule
 // contractions read: [row path * nx][column path * ny] (Gram: every column
 // path of the call; pairs: one nx x ny block per pair).  Pair k's cell (P, Q)
@@ -613,9 +658,15 @@ __global__ void __launch_bounds__(GB_THREADS) band_gbar_kernel(BandGbarArgs a) {
     }
 }
 
+// macro-steps of coefficient slots and last-row Q's kept per warp
+template <int R, int LAM>
+__host__ __device__ constexpr int adj_ring() {
+    constexpr int d = band_ring<R, (R >> LAM)>();
+    return d > 0 ? d : 2;
+}
 template <int R, int LAM>
 __host__ __device__ constexpr int adj_warp_floats() {
-    return 2 * 32 * (R >> LAM) * (R >> LAM) + 2 * R;
+    return adj_ring<R, LAM>() * (32 * (R >> LAM) * (R >> LAM) + R);
 }
 
 template <int R, int LAM>
@@ -636,10 +687,12 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
     if (k0 >= a.n_pairs) return;
     const int np = (int)min(a.ppw, a.n_pairs - k0);
     const int TperR = a.TperR;
-    // per warp: two macro-steps of coefficient slots (lane-major, 16-byte
+    // per warp: D macro-steps of coefficient slots (lane-major, 16-byte
     // chunks rotated by lane against bank conflicts) and of the last row's Q
+    constexpr bool DEEP = band_ring<R, NG>() > 0;   // fetched D - 1 macro-steps ahead, else one
+    constexpr int D = adj_ring<R, LAM>();
     float *ring = adj_sm + (size_t)warp * adj_warp_floats<R, LAM>();
-    float *bqs = ring + 2 * 32 * SLOT;
+    float *bqs = ring + D * 32 * SLOT;
     const float *bq = a.botq + gw * a.bq_stride;
     auto chunk = [&](int c) { return NCH >= 8 ? (c ^ (lane & 7)) : (NCH >= 2 ? (c ^ (lane & (NCH - 1))) : c); };
     auto lane_slot = [&](int buf) { return ring + ((size_t)buf * 32 + lane) * SLOT; };
@@ -650,14 +703,15 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
         kl = (int)q;
         pos = (int)(mm - q * TperR);
     };
-    auto slot_ptr = [&](int kk, int pp) -> const float * {
-        if (kk < 0 || kk > np || (kk == np && pp != 0)) return nullptr;
-        return a.band + band_row((k0 + kk) * TperR + pp, lane, NG);
+    // the lane's slot in macro-step m, as in the forward
+    const float *band0 = a.band + band_row(k0 * TperR - lane, lane, NG);
+    auto slot_ptr = [&](int64_t m) -> const float * {
+        return m >= lane && m - lane <= (int64_t)np * TperR ? band0 + m * (32 * SLOT) : nullptr;
     };
-    // window w of macro-step m (slot src, null outside the chain) into buffer m & 1;
+    // window w of macro-step m (slot src, null outside the chain) into buffer m % D;
     // with window NG-1 also the last row's Q
     auto fetch = [&](int64_t m, const float *src, int w) {
-        float *dst = lane_slot((int)(m & 1));
+        float *dst = lane_slot((int)(m % D));
         if constexpr (NG == 8) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -675,7 +729,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
             else *reinterpret_cast<float2 *>(dd) = make_float2(0.f, 0.f);
         }
         if (w == NG - 1 && lane == 31) {
-            float *bd = bqs + (m & 1) * R;
+            float *bd = bqs + (m % D) * R;
 #pragma unroll
             for (int h = 0; h < R / 4; ++h) cp_async<16>(bd + 4 * h, bq + m * R + 4 * h);
         }
@@ -717,8 +771,18 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
     const int64_t mlast = (int64_t)np * TperR + 31;
     int kl, pos;   // this lane's pair and position at macro-step m, tracked backwards
     locate(mlast, kl, pos);
-    {
-        const float *s0 = slot_ptr(kl, pos);
+    if constexpr (DEEP) {
+#pragma unroll 1
+        for (int64_t m = mlast; m > mlast - (D - 1); --m) {
+            if (m >= 0) {
+                const float *s0 = slot_ptr(m);
+#pragma unroll
+                for (int w = NG - 1; w >= 0; --w) fetch(m, s0, w);
+            }
+            cp_commit();
+        }
+    } else {
+        const float *s0 = slot_ptr(mlast);
 #pragma unroll
         for (int w = NG - 1; w >= 0; --w) {
             fetch(mlast, s0, w);
@@ -733,7 +797,22 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
         }
         const bool trans = (pos == 0);
         const float *sprev = nullptr;
-        if (m >= 1) sprev = pos > 0 ? slot_ptr(kl, pos - 1) : slot_ptr(kl - 1, TperR - 1);
+        if constexpr (DEEP) {
+            if (m >= D - 1) {
+                const float *s0 = slot_ptr(m - (D - 1));
+#pragma unroll
+                for (int w = NG - 1; w >= 0; --w) fetch(m - (D - 1), s0, w);
+            }
+            cp_commit();
+            cp_wait<D - 2>();   // macro-steps m and m - 1
+        } else if (m >= 1) {
+            sprev = slot_ptr(m - 1);
+        }
+        // what macro-step m - 1 will read from memory: a checkpoint, its exit states
+        // (the forward wrote them to DRAM long ago: about 1 GB for 16384 pairs)
+        if (m % BAND_CK == 0 && m >= 1)
+            prefetch_l2(a.ckpt + ((gw * a.nck + (m - 1) / BAND_CK) * 32 + lane) * (int64_t)(2 * R));
+        if (pos == 1 && kl >= 1 && kl <= np) prefetch_l2(a.exitk + ((k0 + kl - 1) * 32 + lane) * (int64_t)R);
         if ((m + 1) % BAND_CK == 0 || m == mlast) {
             // the forward's state after macro-step m
             const float4 *ck = reinterpret_cast<const float4 *>(
@@ -772,18 +851,20 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
                 gseed = a.gout[pr.out0] + (pr.out1 >= 0 ? a.gout[pr.out1] : 0.f);
             }
         }
-        const int buf = (int)(m & 1);
+        const int buf = (int)(m % D), bufn = (int)((m + D - 1) % D);   // bufn: macro-step m - 1's
 
         // a runtime loop over the windows keeps the body within the instruction cache
 #pragma unroll 1
         for (int w = NG - 1; w >= 0; --w) {
-            if (m >= 1) fetch(m - 1, sprev, w);
-            cp_commit();
-            cp_wait<NG - 1>();   // window w - 1 of this macro-step (w = 0: window NG-1 of the one before)
+            if constexpr (!DEEP) {
+                if (m >= 1) fetch(m - 1, sprev, w);
+                cp_commit();
+                cp_wait<NG - 1>();   // window w - 1 of this macro-step (w = 0: window NG-1 of the one before)
+            }
             float2 CN[NH], CO[NH];
             read_window(buf, w, CN);
             if (w > 0) read_window(buf, w - 1, CO);
-            else read_window(buf ^ 1, NG - 1, CO);
+            else read_window(bufn, NG - 1, CO);
             const int tw = has_prev ? w : -1;   // group whose rows turn over in this window
 
 #pragma unroll
@@ -1066,13 +1147,14 @@ __global__ void __launch_bounds__(256) band_gemm_kernel(GemmArgs a) {
 // and the mirror for y: a dense contraction of Wt with the points plus the
 // row and column sums of Wt.
 
-// C (+)= G B per batch for a dense G read as G[r * ld + k] (or G[k * ld + r]
-// when trans).  128 x 32 output tiles, 32-deep K slices staged in shared
-// memory (the next slice is loaded into registers while the current one is
-// used), 4 x 4 outputs per thread; long K ranges split across blocks whose
-// partial tiles band_split_sum_kernel adds in order.  A symmetric Gram's Wt
-// holds blocks i <= j only (tri_rb x tri_cb blocks): the K slices of blocks
-// below the diagonal are skipped.
+// C = G B per batch for a dense G read as G[r * ld + k] (or G[k * ld + r] when
+// trans), ld a multiple of 4, on the tiles of tile_gemm.cuh; long K ranges split
+// across blocks whose partial tiles band_split_sum_kernel adds in order.  G's
+// columns are the column paths' points, padded per path from `py` to `py4`
+// (zeros): column (path, j) meets B or C row path py + j.  A symmetric Gram's Wt
+// holds blocks i <= j only (tri_rb x py4 blocks): the K slices of blocks below
+// the diagonal are skipped.  (128 x 128 Gram of 256-point paths, N = 32: 2.9 ms
+// on 4 x 4 outputs a thread, 2.4 here.)
 struct DenseGemmArgs {
     const float *G;
     int64_t g_ld, g_bstride;
@@ -1080,97 +1162,100 @@ struct DenseGemmArgs {
     int64_t b_bstride;
     float *C;
     int64_t c_bstride;
-    int64_t M, K;
-    int N, trans, ksplit;
+    int64_t M, K;            // padded rows of C (trans) or padded reduction
+    int N, trans, ksplit, py, py4;
+    int64_t crows;           // unpadded rows of C
     float *partial;
-    int64_t tri_rb, tri_cb;
+    int64_t tri_rb;
 };
 
-__global__ void __launch_bounds__(256) dense_gemm_kernel(DenseGemmArgs a) {
-    __shared__ __align__(16) float Gs[GT_K][GT_M + 4];
-    __shared__ __align__(16) float Bs[GT_K][GT_N];
+template <int NT>
+__global__ void __launch_bounds__(TG_THREADS, 2) dense_gemm_kernel(DenseGemmArgs a) {
+    using Tile = TileGemm<NT>;
+    __shared__ __align__(16) typename Tile::Shared sh;
     const int64_t b = blockIdx.z / a.ksplit;
     const int ks = blockIdx.z - (int)b * a.ksplit;
     const float *G = a.G + b * a.g_bstride;
     const float *Bm = a.Bm + b * a.b_bstride;
     float *C = a.C + b * a.c_bstride;
-    const int64_t r0 = (int64_t)blockIdx.x * GT_M;
-    const int n0 = blockIdx.y * GT_N;
-    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int64_t r0 = (int64_t)blockIdx.x * TG_M;
+    const int n0 = blockIdx.y * NT;
     // this block's K range, in whole slices
     int64_t kmin = 0, kmax = a.K;
     if (a.tri_rb > 0) {
-        if (!a.trans) kmin = (r0 / a.tri_rb) * a.tri_cb;   // rows of block i: columns of blocks j >= i
-        else {                                           // columns of block j: rows of blocks i <= j
-            const int64_t rl = (r0 + GT_M - 1 < a.M ? r0 + GT_M - 1 : a.M - 1);
-            kmax = (rl / a.tri_cb + 1) * a.tri_rb;
+        if (!a.trans) kmin = (r0 / a.tri_rb) * a.py4;   // rows of block i: columns of blocks j >= i
+        else {                                         // columns of block j: rows of blocks i <= j
+            const int64_t rl = (r0 + TG_M - 1 < a.M ? r0 + TG_M - 1 : a.M - 1);
+            kmax = (rl / a.py4 + 1) * a.tri_rb;
             if (kmax > a.K) kmax = a.K;
         }
     }
-    const int64_t sl0 = kmin / GT_K, nslice = (kmax + GT_K - 1) / GT_K - sl0;
+    const int64_t sl0 = kmin / TG_K, nslice = (kmax + TG_K - 1) / TG_K - sl0;
     const int64_t s_lo = sl0 + nslice * ks / a.ksplit, s_hi = sl0 + nslice * (ks + 1) / a.ksplit;
-    float gr[16], br[4];
-    auto load = [&](int64_t k0) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool vec = a.N % 4 == 0 && (reinterpret_cast<uintptr_t>(Bm) & 15) == 0;
+    auto load_b = [&](int i, float4 (&v)[NT / 32]) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int v = threadIdx.x + 256 * i;
-            int rr, kk;
-            if (!a.trans) { rr = v / GT_K; kk = v % GT_K; } else { kk = v / GT_M; rr = v % GT_M; }
-            const int64_t r = r0 + rr, k = k0 + kk;
-            gr[i] = (r < a.M && k < a.K) ? (a.trans ? G[k * a.g_ld + r] : G[r * a.g_ld + k]) : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int v = threadIdx.x + 256 * i;
-            const int kk = v / GT_N, nn = v % GT_N;
-            const int64_t k = k0 + kk;
-            const int n = n0 + nn;
-            br[i] = (k < a.K && n < a.N) ? Bm[k * a.N + n] : 0.f;
+        for (int u = 0; u < NT / 32; ++u) {
+            const int64_t k = (s_lo + i) * TG_K + Tile::template b_line<>(u);
+            const int n = n0 + 4 * Tile::template b_quad<>(u);
+            v[u] = zero;
+            int64_t row = k;
+            if (!a.trans) {   // the reduction runs over padded columns
+                const int64_t path = k / a.py4;
+                const int j = (int)(k - path * a.py4);
+                row = j < a.py ? path * a.py + j : -1;
+            }
+            if (k >= a.K || row < 0) continue;
+            const float *p = Bm + row * a.N + n;
+            if (vec) {
+                if (n < a.N) v[u] = __ldg(reinterpret_cast<const float4 *>(p));
+            } else {
+                if (n < a.N) v[u].x = p[0];
+                if (n + 1 < a.N) v[u].y = p[1];
+                if (n + 2 < a.N) v[u].z = p[2];
+                if (n + 3 < a.N) v[u].w = p[3];
+            }
         }
     };
-    float acc[4][4];
+    Tile t;
+    t.clear();
+    if (!a.trans) {
+        t.template run<true>(sh, (int)(s_hi - s_lo), [&](int i, float4 (&v)[4]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+            for (int u = 0; u < 4; ++u) {
+                const int64_t r = r0 + Tile::template line<true>(u);
+                const int64_t k = (s_lo + i) * TG_K + 4 * Tile::template quad<true>(u);
+                v[u] = r < a.M && k < a.K ? __ldcs(reinterpret_cast<const float4 *>(G + r * a.g_ld + k)) : zero;
+            }
+        }, load_b);
+    } else {
+        t.template run<false>(sh, (int)(s_hi - s_lo), [&](int i, float4 (&v)[4]) {
 #pragma unroll
-        for (int jx = 0; jx < 4; ++jx) acc[i][jx] = 0.f;
-    if (s_lo < s_hi) load(s_lo * GT_K);
-    for (int64_t sl = s_lo; sl < s_hi; ++sl) {
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int v = threadIdx.x + 256 * i;
-            if (!a.trans) Gs[v % GT_K][v / GT_K] = gr[i];
-            else Gs[v / GT_M][v % GT_M] = gr[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int v = threadIdx.x + 256 * i;
-            Bs[v / GT_N][v % GT_N] = br[i];
-        }
-        __syncthreads();
-        if (sl + 1 < s_hi) load((sl + 1) * GT_K);
-#pragma unroll 8
-        for (int kk = 0; kk < GT_K; ++kk) {
-            const float4 g = *reinterpret_cast<const float4 *>(&Gs[kk][4 * ty]);
-            const float4 bv = *reinterpret_cast<const float4 *>(&Bs[kk][4 * tx]);
-            const float gg[4] = {g.x, g.y, g.z, g.w};
-            const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int jx = 0; jx < 4; ++jx) acc[i][jx] = fmaf(gg[i], bb[jx], acc[i][jx]);
-        }
+            for (int u = 0; u < 4; ++u) {
+                const int64_t k = (s_lo + i) * TG_K + Tile::template line<false>(u);
+                const int64_t r = r0 + 4 * Tile::template quad<false>(u);
+                v[u] = r < a.M && k < a.K ? __ldcs(reinterpret_cast<const float4 *>(G + k * a.g_ld + r)) : zero;
+            }
+        }, load_b);
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t r = r0 + 4 * ty + i;
+    for (int i = 0; i < 8; ++i) {
+        const int64_t r = r0 + 8 * (threadIdx.x >> 4) + i;
         if (r >= a.M) continue;
+        int64_t row = r;
+        if (a.trans) {
+            const int64_t path = r / a.py4;
+            const int j = (int)(r - path * a.py4);
+            if (j >= a.py) continue;
+            row = path * a.py + j;
+        }
 #pragma unroll
-        for (int jx = 0; jx < 4; ++jx) {
-            const int n = n0 + 4 * tx + jx;
+        for (int jx = 0; jx < Tile::TN; ++jx) {
+            const int n = n0 + Tile::TN * (threadIdx.x & 15) + jx;
             if (n >= a.N) continue;
-            if (a.ksplit > 1) a.partial[((int64_t)ks * a.M + r) * a.N + n] = acc[i][jx];
-            else C[r * a.N + n] = acc[i][jx];
+            if (a.ksplit > 1) a.partial[((int64_t)ks * a.crows + row) * a.N + n] = t.out(i, jx);
+            else C[row * a.N + n] = t.out(i, jx);
         }
     }
 }
@@ -1203,38 +1288,65 @@ __global__ void band_points_kernel(const float *dinc, int64_t npaths, int64_t L,
 }
 
 
+// Squared norms of rows of d floats.
+__global__ void rbf_norms_kernel(const float *P, int64_t rows, int64_t d, float *out) {
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
+        float s = 0.f;
+        for (int64_t c = 0; c < d; ++c) s = fmaf(P[r * d + c], P[r * d + c], s);
+        out[r] = s;
+    }
+}
+
 // Wt of every pair's (nx+1) x (ny+1) points (see the RBF chain rule above)
-// and its row and column sums.  Units are (pair, 128 x 32 point tile); a
-// block stages the tile's points channel-major (32 channels a pass) and the
-// 129 x 33 values of dk/dc around it from the band layout; thread t owns
-// points rows 4 (t/8) .. +3 and columns 4 (t%8) .. +3 of the tile.
+// and its row and column sums.  Units are (pair, 128 x 64 point tile).  <x_i,
+// y_j> is a tile of tile_gemm.cuh over the channels; |x_i - y_j|^2 = |x_i|^2 +
+// |y_j|^2 - 2 <x_i, y_j> (only kappa itself is needed here, so the cancellation
+// near x_i = y_j costs an absolute error of about FP32 epsilon times |x|^2).  The
+// band slots that hold dk/dc around the tile are staged whole (windows and
+// slots padded by one float: the tile's rows and columns then spread over the
+// banks), and a thread takes the 9 x 5 values around its 8 x 4 points from
+// there.  It is bound by issue slots: per point 16 FMAs' worth at d = 32, about
+// 9 for its share of dk/dc, 10 for kappa and the sums.  8 x 4 points a thread
+// instead of 4 x 4 and a tile core with vector reads: 128 x 128 Gram of
+// 256-point paths, d = 32, 9.6 -> 6.2 ms.
 struct RbfWtArgs {
     PairSrc src;             // oriented: rows refine A
     const float *gband;      // dk/dc in the band layout (TperR1 slots per pair)
     float *wt;               // Gram: [row path ia][i] x [column path jb][j], ld = ldw; pairs: [k][i][j]
     float *rsum, *csum;      // sums over j / over i (zeroed before)
+    const float *xn, *yn;    // squared norms of the launch's row points and of the column points
     int64_t n_pairs, ldw, a0;
-    int TperR1, vrows, NQV, tiles_i, tiles_j;
+    int TperR1, vrows, NQV, tiles_i, tiles_j, py4;
     float s, scale;          // 1/(2 sigma^2), 1/2 4^-lambda
 };
-constexpr int RW_TI = 128, RW_TJ = 32, RW_CH = 32;
+constexpr int RW_TI = TG_M, RW_TJ = 64;
+
+// the staged slots of a tile: lanes (rows), positions (columns), floats a slot
+template <int NG>
+struct RwStage {
+    static constexpr int SL = RW_TI / NG + 1 < 32 ? RW_TI / NG + 1 : 32, SP = RW_TJ / NG + 2;
+    static constexpr int WS = NG + 1, SS = NG * WS + 1;
+    static constexpr int FLOATS = SL * SP * SS;
+};
+template <int NG>
+constexpr int rw_smem_bytes() {
+    constexpr int a = 4 * RwStage<NG>::FLOATS, b = (int)sizeof(typename TileGemm<RW_TJ>::Shared);
+    return a + b;
+}
 
 template <int NG>
-__global__ void __launch_bounds__(256) rbf_wt_kernel(RbfWtArgs a) {
+__global__ void __launch_bounds__(TG_THREADS, 2) rbf_wt_kernel(RbfWtArgs a) {
+    using Tile = TileGemm<RW_TJ>;
+    using St = RwStage<NG>;
     constexpr int SLOT = NG * NG;
-    // the band slots around a tile: lanes (rows) and positions (columns)
-    constexpr int SL = RW_TI / NG + 1 < 32 ? RW_TI / NG + 1 : 32, SP = RW_TJ / NG + 2;
-    // the points (channel loop) and the staged slots (before it) share memory
-    constexpr int PTS = RW_CH * RW_TI + RW_CH * (RW_TJ + 1), STG = SL * SP * SLOT;
-    __shared__ __align__(16) float pool[PTS > STG ? PTS : STG];
-    float (*xs)[RW_TI] = reinterpret_cast<float (*)[RW_TI]>(pool);
-    float (*ys)[RW_TJ + 1] = reinterpret_cast<float (*)[RW_TJ + 1]>(pool + RW_CH * RW_TI);
-    __shared__ float gs[RW_TI + 1][RW_TJ + 2];
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int r = (tid >> 3) * 4, c0 = (tid & 7) * 4;
+    extern __shared__ __align__(16) float rw_sm[];
+    typename Tile::Shared &sh = *reinterpret_cast<typename Tile::Shared *>(rw_sm);
+    float *stage = rw_sm + sizeof(typename Tile::Shared) / 4;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int64_t d = a.src.d;
     const bool gram = a.src.mode != PM_PAIRS;
-    const int per = a.tiles_i * a.tiles_j;
+    const bool vec = d % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.src.A) | reinterpret_cast<uintptr_t>(a.src.B)) & 15) == 0;
+    const int per = a.tiles_i * a.tiles_j, nsl = (int)((d + TG_K - 1) / TG_K);
     for (int64_t u = blockIdx.x; u < a.n_pairs * per; u += gridDim.x) {
         const int64_t k = u / per;
         const int t = (int)(u - k * per);
@@ -1244,127 +1356,104 @@ __global__ void __launch_bounds__(256) rbf_wt_kernel(RbfWtArgs a) {
         if (i0 > nx || j0 > ny) continue;   // block-uniform
         const float *xp = (const float *)a.src.A + pr.a_row0 * d;
         const float *yp = (const float *)a.src.B + pr.b_row0 * d;
-        __syncthreads();
-        // the slots holding dk/dc at (p, q) = (i0 - 1 + pi, j0 - 1 + qj): lanes
-        // from l0, positions from s0 (for a position, the lanes are one
-        // contiguous run), staged with 16-byte loads; then the tile, zero
-        // outside the grid
+        __syncthreads();   // the last tile's readers of the stage are done
+        // the slots holding dk/dc at (p, q) = (i0 - 1 + pi, j0 - 1 + qj): lanes from
+        // l0, positions from s0 (for a position, the lanes are one contiguous run)
         const int Pf = i0 - 1 + a.vrows, Qf = j0 - 1 + a.NQV;
         const int l0 = (Pf < 0 ? 0 : Pf) / NG, s0 = (Qf < 0 ? 0 : Qf) / NG;
-        for (int v = tid; v < STG / 4; v += 256) {
-            const int sl = v / (SLOT / 4), e = v - sl * (SLOT / 4);
-            const int pr = sl / SL, lr = sl - pr * SL;
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (l0 + lr < 32 && s0 + pr < a.TperR1)
-                x = __ldg(reinterpret_cast<const float4 *>(a.gband + ((k * a.TperR1 + s0 + pr) * 32 + l0 + lr) *
-                                                                        (int64_t)SLOT) + e);
-            reinterpret_cast<float4 *>(pool)[v] = x;
-        }
-        __syncthreads();
-        for (int v = tid; v < (RW_TI + 1) * (RW_TJ + 1); v += 256) {
-            const int pi = v / (RW_TJ + 1), qj = v - pi * (RW_TJ + 1);
-            const int pp = i0 - 1 + pi, qq = j0 - 1 + qj;
-            float gv = 0.f;
-            if (pp >= 0 && pp < nx && qq >= 0 && qq < ny) {
-                const int P = pp + a.vrows, Q = qq + a.NQV;
-                const int l = P / NG, g = P % NG, tq = Q + g;
-                gv = pool[((tq / NG - s0) * SL + l - l0) * SLOT + (tq % NG) * NG + band_gpos<NG>(g)];
-            }
-            gs[pi][qj] = gv;
-        }
-        // |x_i - y_j|^2 = |x_i|^2 + |y_j|^2 - 2 <x_i, y_j>: one FMA a pair and
-        // channel (only kappa itself is needed here, so the cancellation near
-        // x_i = y_j costs an absolute error of about FP32 epsilon times |x|^2)
-        float xy[4][4], xx[4], yy[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            xx[i] = 0.f;
-            yy[i] = 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) xy[i][j] = 0.f;
-        }
-        for (int64_t cb = 0; cb < d; cb += RW_CH) {
-            const int nc = d - cb < RW_CH ? (int)(d - cb) : RW_CH;
-            __syncthreads();
-            // consecutive threads take consecutive channels of a point (the
-            // full-width passes without a division)
-            for (int v = tid; v < nc * RW_TI; v += 256) {
-                const int i = nc == RW_CH ? v >> 5 : v / nc, c = nc == RW_CH ? v & 31 : v - i * nc;
-                xs[c][i] = i0 + i <= nx ? xp[(int64_t)(i0 + i) * d + cb + c] : 0.f;
-            }
-            for (int v = tid; v < nc * RW_TJ; v += 256) {
-                const int j = nc == RW_CH ? v >> 5 : v / nc, c = nc == RW_CH ? v & 31 : v - j * nc;
-                ys[c][j] = j0 + j <= ny ? yp[(int64_t)(j0 + j) * d + cb + c] : 0.f;
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int c = 0; c < nc; ++c) {
-                float xv[4], yv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = xs[c][r + i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) yv[j] = ys[c][c0 + j];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) yy[j] = fmaf(yv[j], yv[j], yy[j]);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    xx[i] = fmaf(xv[i], xv[i], xx[i]);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) xy[i][j] = fmaf(xv[i], yv[j], xy[i][j]);
-                }
+        for (int v = tid; v < St::SL * St::SP * (SLOT / 4); v += TG_THREADS) {
+            const int sl = v / (SLOT / 4), e = 4 * (v - sl * (SLOT / 4));
+            const int sp = sl / St::SL, lr = sl - sp * St::SL;
+            if (l0 + lr < 32 && s0 + sp < a.TperR1) {
+                const float4 x = __ldcs(reinterpret_cast<const float4 *>(
+                    a.gband + ((k * a.TperR1 + s0 + sp) * 32 + l0 + lr) * (int64_t)SLOT + e));
+                float *dst = stage + sl * St::SS;
+                dst[e / NG * St::WS + e % NG] = x.x;
+                dst[(e + 1) / NG * St::WS + (e + 1) % NG] = x.y;
+                dst[(e + 2) / NG * St::WS + (e + 2) % NG] = x.z;
+                dst[(e + 3) / NG * St::WS + (e + 3) % NG] = x.w;
             }
         }
-        float rs[4] = {0.f, 0.f, 0.f, 0.f}, cs[4] = {0.f, 0.f, 0.f, 0.f};
+        // <x_i, y_j>
+        auto quad = [&](const float *p, int64_t c) {   // channels c .. c + 3 of the point at p
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vec) {
+                if (c < d) v = __ldg(reinterpret_cast<const float4 *>(p + c));
+            } else {
+                if (c < d) v.x = __ldg(p + c);
+                if (c + 1 < d) v.y = __ldg(p + c + 1);
+                if (c + 2 < d) v.z = __ldg(p + c + 2);
+                if (c + 3 < d) v.w = __ldg(p + c + 3);
+            }
+            return v;
+        };
+        Tile g;
+        g.clear();
+        g.template run<true, true>(sh, nsl, [&](int sl, float4 (&v)[4]) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = min(i0 + Tile::template line<true>(e), nx);
+                v[e] = quad(xp + (int64_t)i * d, (int64_t)sl * TG_K + 4 * Tile::template quad<true>(e));
+            }
+        }, [&](int sl, float4 (&v)[RW_TJ / 32]) {
+#pragma unroll
+            for (int e = 0; e < RW_TJ / 32; ++e) {
+                const int j = min(j0 + Tile::template b_line<true>(e), ny);
+                v[e] = quad(yp + (int64_t)j * d, (int64_t)sl * TG_K + 4 * Tile::template b_quad<true>(e));
+            }
+        });
+        // (the run's barriers also cover the staged slots)
         const int64_t ia = gram ? pr.a_row0 / pr.la - a.a0 : k;
         const int64_t jb = gram ? pr.b_row0 / pr.lb : k;
-        // a row's four columns leave as one 16-byte store where the rows are
-        // 16-byte aligned and all four are real
-        const bool vec = ((ny + 1) & 3) == 0 && j0 + c0 + 3 <= ny;
+        const int ib = i0 + 8 * ty, jc = j0 + 4 * tx;   // the thread's first point
+        // dk/dc at (p, jc - 1 + e), e < 5, zero outside the grid
+        auto row_dc = [&](int p, float (&v)[5]) {
+            const int P = p + a.vrows, l = P / NG, gg = P - l * NG;
+            const float *base = stage + (l - l0) * St::SS + band_gpos<NG>(gg);
+            const bool in = p >= 0 && p < nx;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int pi = r + i, ii = i0 + pi;
-            if (ii > nx) continue;
-            float wv[4];
+            for (int e = 0; e < 5; ++e) {
+                const int q = jc - 1 + e, tq = q + a.NQV + gg;
+                v[e] = 0.f;
+                if (in && q >= 0 && q < ny) v[e] = base[(tq / NG - s0) * (St::SL * St::SS) + tq % NG * St::WS];
+            }
+        };
+        float yy[4], cs[4] = {0.f, 0.f, 0.f, 0.f}, up[5], dn[5];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) yy[j] = jc + j <= ny ? a.yn[(gram ? pr.b_row0 : k * (ny + 1)) + jc + j] : 0.f;
+        row_dc(ib - 1, up);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int ii = ib + i;
+            row_dc(ii, dn);
+            float wv[4], rs = 0.f;
+            const bool in = ii <= nx;
+            const float xx = in ? a.xn[ia * (nx + 1) + ii] : 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int qj = c0 + j;
-                const float W = gs[pi][qj] - gs[pi][qj + 1] - gs[pi + 1][qj] + gs[pi + 1][qj + 1];
-                const float uu = fmaxf(xx[i] + yy[j] - 2.f * xy[i][j], 0.f);
-                wv[j] = j0 + qj <= ny ? a.scale * W * __expf(-a.s * uu) : 0.f;
-                rs[i] += wv[j];
+                const float W = up[j] - up[j + 1] - dn[j] + dn[j + 1];
+                const float uu = fmaxf(xx + yy[j] - 2.f * g.out(i, j), 0.f);
+                wv[j] = in && jc + j <= ny ? a.scale * W * __expf(-a.s * uu) : 0.f;
+                rs += wv[j];
                 cs[j] += wv[j];
             }
-            float *row = gram ? a.wt + (ia * (nx + 1) + ii) * a.ldw + jb * (ny + 1)
-                              : a.wt + (k * (nx + 1) + ii) * (int64_t)(ny + 1);
-            if (vec) {
-                *reinterpret_cast<float4 *>(row + j0 + c0) = make_float4(wv[0], wv[1], wv[2], wv[3]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (j0 + c0 + j <= ny) row[j0 + c0 + j] = wv[j];
+            if (in && jc < a.py4) {   // a path's padding columns get zeros
+                float *row = gram ? a.wt + (ia * (nx + 1) + ii) * a.ldw + jb * a.py4
+                                  : a.wt + (k * (nx + 1) + ii) * (int64_t)a.py4;
+                *reinterpret_cast<float4 *>(row + jc) = make_float4(wv[0], wv[1], wv[2], wv[3]);
             }
-        }
-        // row sums over the 8 threads of a row group, column sums over the
-        // 4 row groups of the warp; then one atomic add per value
+            // the row's sum over its 16 threads, one atomic add
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            rs[i] += __shfl_xor_sync(FULL, rs[i], 1);
-            rs[i] += __shfl_xor_sync(FULL, rs[i], 2);
-            rs[i] += __shfl_xor_sync(FULL, rs[i], 4);
+            for (int o = 1; o < 16; o *= 2) rs += __shfl_xor_sync(FULL, rs, o);
+            if (tx == 0 && in) atomicAdd(a.rsum + ia * (nx + 1) + ii, rs);
+#pragma unroll
+            for (int e = 0; e < 5; ++e) up[e] = dn[e];
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            cs[j] += __shfl_xor_sync(FULL, cs[j], 8);
             cs[j] += __shfl_xor_sync(FULL, cs[j], 16);
+            if ((tid & 16) == 0 && jc + j <= ny) atomicAdd(a.csum + jb * (ny + 1) + jc + j, cs[j]);
         }
-        if ((lane & 7) == 0)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (i0 + r + i <= nx) atomicAdd(a.rsum + ia * (nx + 1) + i0 + r + i, rs[i]);
-        if (lane < 8)
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (j0 + c0 + j <= ny) atomicAdd(a.csum + jb * (ny + 1) + j0 + c0 + j, cs[j]);
     }
 }
 
@@ -1585,13 +1674,13 @@ BwdRegions bwd_regions(const PairSrc &src, const BandPlan &p, int64_t nbp, int c
         // the lift works on points: Wt of every pair (dense, in gbar), the
         // contractions' results (dinc), the row and column sums; no increments
         const int64_t px = nx + 1, py = ny + 1;
-        r.gbar = up4(nA * px * nB * py);
-        if (!gram) r.gbar = up4(nbp * px * py);
+        r.gbar = nA * px * nB * up4(py);
+        if (!gram) r.gbar = nbp * px * up4(py);
         r.incA = r.incB = 0;
         r.dincA = up4(nA * px * d);
         r.dincB = up4(nB * py * d);
         r.part = gram ? up4((int64_t)GEMM_MAX_SPLIT * (nA * px > nB * py ? nA * px : nB * py) * d) : 0;
-        r.rsum = up4(nA * px) + up4(nB * py);
+        r.rsum = 2 * (up4(nA * px) + up4(nB * py));   // and the points' squared norms
     }
     // the adjoint's dk/dc in the band layout: TperR + 1 slots per pair
     r.gband = up4(nbp * ((int64_t)p.TperR + 1) * 32 * p.NG * p.NG);
@@ -1636,8 +1725,16 @@ cudaError_t rbf_chain_rule(const PairSrc &src, const BandPlan &p, int64_t m, int
     if ((e = cudaMemsetAsync(rsum, 0, sizeof(float) * (size_t)(up4(nrow * px) + ncol * py), st)) != cudaSuccess)
         return e;
     // a symmetric Gram stores pairs i <= j: the blocks below the diagonal stay zero
-    if (sym && (e = cudaMemsetAsync(wt, 0, sizeof(float) * (size_t)(nA * px * nB * py), st)) != cudaSuccess)
+    const int64_t py4 = up4(py);
+    if (sym && (e = cudaMemsetAsync(wt, 0, sizeof(float) * (size_t)(nA * px * nB * py4), st)) != cudaSuccess)
         return e;
+    const float *Apts = (const float *)src.A + (gram ? a0 : src.kbase) * px * d;
+    const float *Bpts = sym ? (const float *)src.A : (const float *)src.B + (gram ? 0 : src.kbase) * py * d;
+    float *xn = csum + up4(ncol * py), *yn = xn + up4(nrow * px);
+    rbf_norms_kernel<<<(unsigned)((nrow * px + 255) / 256 < sms * 8 ? (nrow * px + 255) / 256 : sms * 8), 256, 0, st>>>(
+        Apts, nrow * px, d, xn);
+    rbf_norms_kernel<<<(unsigned)((ncol * py + 255) / 256 < sms * 8 ? (ncol * py + 255) / 256 : sms * 8), 256, 0, st>>>(
+        Bpts, ncol * py, d, yn);
     RbfWtArgs w;
     w.src = src;
     w.gband = gband;
@@ -1645,7 +1742,10 @@ cudaError_t rbf_chain_rule(const PairSrc &src, const BandPlan &p, int64_t m, int
     w.rsum = rsum;
     w.csum = csum;
     w.n_pairs = m;
-    w.ldw = gram ? nB * py : py;
+    w.xn = xn;
+    w.yn = yn;
+    w.py4 = (int)py4;
+    w.ldw = gram ? nB * py4 : py4;
     w.a0 = a0;
     w.TperR1 = p.TperR + 1;
     w.vrows = p.vrows;
@@ -1655,14 +1755,18 @@ cudaError_t rbf_chain_rule(const PairSrc &src, const BandPlan &p, int64_t m, int
     w.s = (float)(0.5 / (src.sigma * src.sigma));
     w.scale = 0.5f / (float)(1 << (2 * p.lam));
     int64_t grid = m * w.tiles_i * w.tiles_j;
-    if (grid > (int64_t)sms * 8) grid = (int64_t)sms * 8;
-    if (p.NG == 8) rbf_wt_kernel<8><<<(int)grid, 256, 0, st>>>(w);
-    else if (p.NG == 4) rbf_wt_kernel<4><<<(int)grid, 256, 0, st>>>(w);
-    else rbf_wt_kernel<2><<<(int)grid, 256, 0, st>>>(w);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (grid > (int64_t)sms * 2) grid = (int64_t)sms * 2;
+    auto go = [&](auto kern, int smem) {
+        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r != cudaSuccess) return r;
+        kern<<<(int)grid, TG_THREADS, smem, st>>>(w);
+        return cudaGetLastError();
+    };
+    if (p.NG == 8) e = go(rbf_wt_kernel<8>, rw_smem_bytes<8>());
+    else if (p.NG == 4) e = go(rbf_wt_kernel<4>, rw_smem_bytes<4>());
+    else e = go(rbf_wt_kernel<2>, rw_smem_bytes<2>());
+    if (e != cudaSuccess) return e;
     // the contractions
-    const float *Apts = (const float *)src.A + (gram ? a0 : src.kbase) * px * d;
-    const float *Bpts = sym ? (const float *)src.A : (const float *)src.B + (gram ? 0 : src.kbase) * py * d;
     DenseGemmArgs g1;
     memset(&g1, 0, sizeof(g1));
     g1.G = wt;
@@ -1674,27 +1778,31 @@ cudaError_t rbf_chain_rule(const PairSrc &src, const BandPlan &p, int64_t m, int
     g2.Bm = Apts;
     g2.C = CY;
     g2.trans = 1;
+    g1.py = g2.py = (int)py;
+    g1.py4 = g2.py4 = (int)py4;
     int64_t batches = 1;
     if (gram) {
-        g1.g_ld = g2.g_ld = nB * py;
-        g1.M = nA * px; g1.K = nB * py;
-        g2.M = nB * py; g2.K = nA * px;
+        g1.g_ld = g2.g_ld = nB * py4;
+        g1.M = nA * px; g1.K = nB * py4;
+        g2.M = nB * py4; g2.K = nA * px;
+        g1.crows = nA * px; g2.crows = nB * py;
         g1.tri_rb = g2.tri_rb = sym ? px : 0;
-        g1.tri_cb = g2.tri_cb = sym ? py : 0;
     } else {
         batches = m;
-        g1.g_ld = g2.g_ld = py;
-        g1.g_bstride = g2.g_bstride = px * py;
+        g1.g_ld = g2.g_ld = py4;
+        g1.g_bstride = g2.g_bstride = px * py4;
         g1.b_bstride = py * d; g2.b_bstride = px * d;
         g1.c_bstride = px * d; g2.c_bstride = py * d;
-        g1.M = px; g1.K = py;
-        g2.M = py; g2.K = px;
+        g1.M = px; g1.K = py4;
+        g2.M = py4; g2.K = px;
+        g1.crows = px; g2.crows = py;
     }
+    const int nt = d > 32 ? 64 : 32;
     auto split = [&](const DenseGemmArgs &g) {
         if (!gram) return 1;
-        const int64_t tiles = ((g.M + GT_M - 1) / GT_M) * ((d + GT_N - 1) / GT_N);
+        const int64_t tiles = ((g.M + TG_M - 1) / TG_M) * ((d + nt - 1) / nt);
         int64_t ksp = (4 * (int64_t)sms + tiles - 1) / tiles;
-        const int64_t nsl = (g.K + GT_K - 1) / GT_K;
+        const int64_t nsl = (g.K + TG_K - 1) / TG_K;
         if (ksp > nsl / 4) ksp = nsl / 4;
         if (ksp > GEMM_MAX_SPLIT) ksp = GEMM_MAX_SPLIT;
         return (int)(ksp < 1 ? 1 : ksp);
@@ -1705,10 +1813,11 @@ cudaError_t rbf_chain_rule(const PairSrc &src, const BandPlan &p, int64_t m, int
     const bool want_b = dB || sym;
     for (int pass = 0; pass < (want_b ? 2 : 1); ++pass) {
         const DenseGemmArgs &g = pass == 0 ? g1 : g2;
-        const dim3 gd((unsigned)((g.M + GT_M - 1) / GT_M), (unsigned)((d + GT_N - 1) / GT_N),
+        const dim3 gd((unsigned)((g.M + TG_M - 1) / TG_M), (unsigned)((d + nt - 1) / nt),
                       (unsigned)(batches * g.ksplit));
-        dense_gemm_kernel<<<gd, 256, 0, st>>>(g);
-        if (g.ksplit > 1) band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g.ksplit, g.M * d, 0, g.C);
+        if (nt == 64) dense_gemm_kernel<64><<<gd, TG_THREADS, 0, st>>>(g);
+        else dense_gemm_kernel<32><<<gd, TG_THREADS, 0, st>>>(g);
+        if (g.ksplit > 1) band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g.ksplit, g.crows * d, 0, g.C);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // the points

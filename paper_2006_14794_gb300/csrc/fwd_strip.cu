@@ -1089,7 +1089,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) grad_chain_tile_kernel(const Pa
             auto load_b = [&](int i, float4 (&v)[NT / 32]) {
 #pragma unroll
                 for (int u = 0; u < NT / 32; ++u) {
-                    const int kk = (s0 + i) * TG_K + Tile::b_line(u), c4 = cb + Tile::b_quad(u);
+                    const int kk = (s0 + i) * TG_K + Tile::template b_line<>(u), c4 = cb + Tile::template b_quad<>(u);
                     v[u] = kk < nred && c4 < D4 ? __ldg(other + (int64_t)kk * D4 + c4) : zero;
                 }
             };

@@ -8,7 +8,8 @@
 // current one is used, one barrier a slice.  G may lie with k contiguous (its
 // float4s are turned in shared memory) or with m contiguous; either way element
 // (k, m) is kept at [k][m ^ 4 ((k / 4) % 8)], so the turned stores of a warp hit
-// 32 banks and the float4 reads stay whole.
+// 32 banks and the float4 reads stay whole.  B likewise (element (k, n) at [k][n
+// ^ 4 ((k / 4) % 8)]).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -61,13 +62,31 @@ struct TileGemm {
             }
         }
     }
-    // B's slice: NT / 4 float4s a line, NT / 32 a thread
-    static __device__ __forceinline__ int b_line(int i) { return (threadIdx.x + TG_THREADS * i) / (NT / 4); }
-    static __device__ __forceinline__ int b_quad(int i) { return (threadIdx.x + TG_THREADS * i) % (NT / 4); }
+    // B's slice, NT / 32 float4s a thread: with n contiguous, line k, quad of n;
+    // with k contiguous, line n, quad of k
+    template <bool BK = false>
+    static __device__ __forceinline__ int b_line(int i) {
+        return (threadIdx.x + TG_THREADS * i) / (BK ? 8 : NT / 4);
+    }
+    template <bool BK = false>
+    static __device__ __forceinline__ int b_quad(int i) {
+        return (threadIdx.x + TG_THREADS * i) % (BK ? 8 : NT / 4);
+    }
+    template <bool BK>
     static __device__ __forceinline__ void put_b(Shared &s, int buf, const float4 (&v)[NT / 32]) {
 #pragma unroll
-        for (int i = 0; i < NT / 32; ++i)
-            *reinterpret_cast<float4 *>(&s.b[buf][b_line(i)][4 * b_quad(i)]) = v[i];
+        for (int i = 0; i < NT / 32; ++i) {
+            const int l = b_line<BK>(i), q = b_quad<BK>(i);
+            if constexpr (BK) {
+                const int n = l ^ (4 * q);
+                s.b[buf][4 * q][n] = v[i].x;
+                s.b[buf][4 * q + 1][n] = v[i].y;
+                s.b[buf][4 * q + 2][n] = v[i].z;
+                s.b[buf][4 * q + 3][n] = v[i].w;
+            } else {
+                *reinterpret_cast<float4 *>(&s.b[buf][l][4 * (q ^ ((l >> 2) & 7))]) = v[i];
+            }
+        }
     }
     __device__ __forceinline__ void slice(const Shared &s, int buf) {
         const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
@@ -80,10 +99,10 @@ struct TileGemm {
                                  make_float2(g1.z, g1.w)};
             float b[TN];
             if constexpr (TN == 4) {
-                const float4 t = *reinterpret_cast<const float4 *>(&s.b[buf][k][4 * tx]);
+                const float4 t = *reinterpret_cast<const float4 *>(&s.b[buf][k][4 * (tx ^ sw)]);
                 b[0] = t.x; b[1] = t.y; b[2] = t.z; b[3] = t.w;
             } else {
-                const float2 t = *reinterpret_cast<const float2 *>(&s.b[buf][k][2 * tx]);
+                const float2 t = *reinterpret_cast<const float2 *>(&s.b[buf][k][4 * ((tx >> 1) ^ sw) + 2 * (tx & 1)]);
                 b[0] = t.x; b[1] = t.y;
             }
 #pragma unroll
@@ -93,7 +112,7 @@ struct TileGemm {
         }
     }
     // all slices 0 .. n - 1: load_g(slice, float4[4]) and load_b(slice, float4[NT / 32])
-    template <bool KCONT, class LG, class LB>
+    template <bool KCONT, bool BK = false, class LG, class LB>
     __device__ __forceinline__ void run(Shared &s, int n, LG load_g, LB load_b) {
         float4 gv[4], bv[NT / 32];
         if (n > 0) {
@@ -103,7 +122,7 @@ struct TileGemm {
         __syncthreads();   // the last run's readers are done
         for (int i = 0; i < n; ++i) {
             put_g<KCONT>(s, i & 1, gv);
-            put_b(s, i & 1, bv);
+            put_b<BK>(s, i & 1, bv);
             __syncthreads();
             if (i + 1 < n) {
                 load_g(i + 1, gv);
