@@ -49,6 +49,17 @@ constexpr int CW = 32;           // columns per published chunk of a bottom row
 template <typename T>
 __host__ __device__ constexpr int strip_ck() { return sizeof(T) == 4 ? 64 : 128; }
 inline int strip_ck_of(int64_t es) { return es == 4 ? 64 : 128; }
+// checkpoint slots of a strip of `tend` steps.  FP64: the state after step t is
+// in slot t / ck, for the last step of each slot's range and step tend - 1.
+// FP32: slot 0 is the state after step tend - 1, slot 1 + m that after step
+// adj_top - 64 m, where the adjoint's 32-step chunks begin.
+__host__ __device__ constexpr int64_t strip_ckpts(int64_t tend, int64_t ck) { return (tend + ck - 1) / ck + 1; }
+// the FP32 adjoint runs whole groups of four windows: its first step (maybe
+// past the sweep's last, tend - 1)
+__host__ __device__ constexpr int adj_top(int tend, int lam) {
+    const int w4 = 4 << lam;
+    return (tend + w4 - 1) / w4 * w4 - 1;
+}
 
 // ---- planning: per-pair sizes and offsets, computed on the device ----------
 
@@ -107,7 +118,7 @@ __global__ void plan_kernel(PairSrc src, int64_t n, PairPlan *plan, int64_t *tot
         p.c_off = (int64_t)p.ns * p.nw * CP;        // sizes for now, offsets after the scan
         p.bnd_off = p.ns > 0 ? (int64_t)(ck ? p.ns : p.ns - 1) * p.nj * 2 : 0;
         p.strip_base = p.ns;
-        p.s_off = ck ? (int64_t)p.ns * ((p.nj + TH - 1 + ck - 1) / ck) * TH * 2 : 0;
+        p.s_off = ck ? p.ns * strip_ckpts(p.nj + TH - 1, ck) * TH * 2 : 0;
         p.g_off = (int64_t)p.nx * gbar_ld(p.ny);
         plan[k] = p;
     }
@@ -342,7 +353,8 @@ struct StripArgs {
     T *out;
     long long wait_cycles;
     int fault_inject;   // 1: the first strip of the first pair never publishes
-    T *sums;            // backward: checkpoints of the state, [strip][step / ck][lane][K 0..R-1, Q 0..R-1]
+    T *sums;            // backward: checkpoints of the state (strip_ckpts), [strip][slot][lane][K of R rows, Q]
+                        // (FP32: rows i, i + R/2 side by side)
 };
 
 constexpr int NRING = 8;   // coefficient diagonals in flight per warp
@@ -590,15 +602,18 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_kernel(StripArgs<T> a)
                     }
                     if constexpr (SAVE) {
                         constexpr int CK = strip_ck<T>();
-                        if ((t + 1) % CK == 0 || t == tend - 1) {
-                            const int nck = (tend + CK - 1) / CK;
-                            T *dst = a.sums + pp.s_off + (((int64_t)s * nck + t / CK) * 32 + lane) * (2 * R);
+                        const int back = adj_top(tend, LAM) - t;   // steps from the adjoint's first
+                        auto save = [&](int64_t slot) {
+                            float4 *dst = reinterpret_cast<float4 *>(
+                                a.sums + pp.s_off + ((s * strip_ckpts(tend, CK) + slot) * 32 + lane) * (2 * R));
 #pragma unroll
-                            for (int i = 0; i < H; ++i) {
-                                dst[i] = KP[i].x; dst[i + H] = KP[i].y;
-                                dst[R + i] = QP[i].x; dst[R + i + H] = QP[i].y;
+                            for (int i = 0; i < H; i += 2) {
+                                dst[i / 2] = make_float4(KP[i].x, KP[i].y, KP[i + 1].x, KP[i + 1].y);
+                                dst[(H + i) / 2] = make_float4(QP[i].x, QP[i].y, QP[i + 1].x, QP[i + 1].y);
                             }
-                        }
+                        };
+                        if (back % CK == 0) save(1 + back / CK);
+                        if (t == tend - 1) save(0);
                     }
                 } else {
 #pragma unroll
@@ -622,8 +637,8 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_kernel(StripArgs<T> a)
                     if constexpr (SAVE) {
                         constexpr int CK = strip_ck<T>();
                         if ((t + 1) % CK == 0 || t == tend - 1) {
-                            const int nck = (tend + CK - 1) / CK;
-                            T *dst = a.sums + pp.s_off + (((int64_t)s * nck + t / CK) * 32 + lane) * (2 * R);
+                            const int64_t nck = strip_ckpts(tend, CK);
+                            T *dst = a.sums + pp.s_off + ((s * nck + t / CK) * 32 + lane) * (2 * R);
 #pragma unroll
                             for (int r = 0; r < R; ++r) { dst[r] = K[r]; dst[R + r] = Q[r]; }
                         }
@@ -684,7 +699,7 @@ struct AdjArgs {
     const int64_t *totals;
     int64_t n_pairs;
     const T *cbuf;
-    const T *ckpt;   // the forward's checkpoints: [strip][step / ck][lane][K 0..R-1, Q 0..R-1]
+    const T *ckpt;   // the forward's checkpoints (StripArgs::sums)
     const T *bnd;    // the forward's bottom rows (K, Q) per column, every strip
     T *vbuf;         // per pair, per strip boundary: V of the lower strip's first row [nj],
                      // filled with the all-ones pattern first
@@ -729,9 +744,9 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_adj_kernel(AdjArgs<T> 
         const int nj = pp.nj;
         const int tend = nj + TH - 1;
         const int nwin = (tend + S - 1) / S;
-        const int nck = (tend + CK - 1) / CK;
+        const int64_t nck = strip_ckpts(tend, CK);
         const T *blk = a.cbuf + pp.c_off + (int64_t)s * pp.nw * CP;
-        const T *ck = a.ckpt + pp.s_off + (int64_t)s * nck * TH * 2 + lane * (2 * R);
+        const T *ck = a.ckpt + pp.s_off + s * nck * TH * 2 + lane * (2 * R);
         const T *topb = s > 0 ? a.bnd + pp.bnd_off + (int64_t)(s - 1) * nj * 2 : nullptr;
         const T *botb = a.bnd + pp.bnd_off + (int64_t)s * nj * 2;
         const T *below = s < pp.ns - 1 ? a.vbuf + pp.bnd_off / 2 + (int64_t)s * nj : nullptr;
@@ -941,6 +956,251 @@ __global__ void __launch_bounds__(STRIP_WARPS * 32) strip_adj_kernel(AdjArgs<T> 
             }
         }
         ring_wait<0>();
+    }
+}
+
+// The FP32 adjoint: the same sweep with rows (i, i + H) of a lane in float2s, as
+// the forward (add2, fma2 undo a step and advance A and V for two rows at once,
+// the state kept as (K, -Q)), in groups of four windows of straight-line code.
+//  - What a step reads from outside the strip (the upper strip's K at its
+//    column for lane 0; the strip's own bottom row and the lower strip's V for
+//    lane 31) is taken 32 steps at a time: lane j of a chunk loads step j's four
+//    values, they go to shared memory as one float4 a step, and the steps read
+//    theirs with one broadcast load.  Chunks, checkpoints and groups all count
+//    from adj_top, so every such event is at a group's first step.
+//  - dk/dG leaves as float4s: group g's column at window w is q = w - NG lane -
+//    g, so with NG a multiple of 4 and four windows unrolled, the window that
+//    completes an aligned quad of columns is known when compiling; the values
+//    of its other windows wait in registers.  (Dyadic orders 2 and 3: NG = 4 in
+//    the same way, NG = 2 as single floats.)
+// The scalar form took about 330 instructions a step, a dozen branches and 8
+// scattered 4-byte stores a window.  64 pairs of 4096 points, order 1: 13.9 ->
+// 6.3 ms.
+struct AdjChunk { float4 v[32]; };   // (upper K, own K, own Q, lower V) of 32 steps
+
+template <int R, int LAM>
+__host__ __device__ constexpr int adjp_warp_floats() {
+    return NRING * 32 * (R >> LAM) + (int)(sizeof(AdjChunk) / 4);
+}
+
+template <int R, int LAM>
+__global__ void __launch_bounds__(STRIP_WARPS * 32) strip_adj_pack_kernel(AdjArgs<float> a) {
+    constexpr int S = 1 << LAM, NG = R / S, CP = 32 * NG, TH = 32 * R, H = R / 2, NH = NG / 2;
+    constexpr int CK = strip_ck<float>();
+    constexpr int GS = 4 * S;                    // steps a group
+    constexpr bool QUADS = NG % 4 == 0;
+    constexpr int AHEAD = GS <= 16 ? 16 : 32;    // steps before its first that a chunk is loaded
+    static_assert(NG % 2 == 0 && 32 % GS == 0 && CK % 32 == 0, "");
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *ringc = reinterpret_cast<float *>(adj_smem) + (size_t)warp * adjp_warp_floats<R, LAM>();
+    AdjChunk &cur = *reinterpret_cast<AdjChunk *>(ringc + NRING * CP);
+    const int64_t total_strips = a.totals[TOT_STRIPS];
+    auto add = [](float2 x, float2 y) { return __fadd2_rn(x, y); };
+    auto mad = [](float2 x, float2 y, float2 z) { return __ffma2_rn(x, y, z); };
+
+    for (;;) {
+        int64_t gs = 0;
+        if (lane == 0) gs = atomicAdd((unsigned long long *)a.counter, 1ULL);
+        gs = __shfl_sync(FULL, gs, 0);
+        if (gs >= total_strips) break;
+        int64_t lo = 0, hi = a.n_pairs - 1;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (a.plan[mid].strip_base <= gs) lo = mid; else hi = mid - 1;
+        }
+        const PairPlan pp = a.plan[lo];
+        const int s = pp.ns - 1 - (int)(gs - pp.strip_base);   // last strip first
+        const int nj = pp.nj, tend = nj + TH - 1, top = adj_top(tend, LAM);
+        const float *blk = a.cbuf + pp.c_off + (int64_t)s * pp.nw * CP + lane * NG;
+        const float4 *ck = reinterpret_cast<const float4 *>(a.ckpt + pp.s_off + s * strip_ckpts(tend, CK) * TH * 2 +
+                                                            lane * (2 * R));
+        const float *topb = s > 0 ? a.bnd + pp.bnd_off + (int64_t)(s - 1) * nj * 2 : nullptr;
+        const float *botb = a.bnd + pp.bnd_off + (int64_t)s * nj * 2;
+        const float *below = s < pp.ns - 1 ? a.vbuf + pp.bnd_off / 2 + (int64_t)s * nj : nullptr;
+        float *above = s > 0 ? a.vbuf + pp.bnd_off / 2 + (int64_t)(s - 1) * nj : nullptr;
+        const int prow = s * CP - (pp.pad >> LAM) + NG * lane;   // the lane's first coarse row
+        const int ld = gbar_ld(pp.ny);
+        float *gp = a.gbar + pp.g_off + (int64_t)prow * ld;
+
+        const float2 zero2 = make_float2(0.f, 0.f);
+        float2 KP[H], QN[H], A[H], V[H], CN[NH], CO[NH], CNP[NH], gN[NH], gO[NH];
+        float carry[QUADS ? NG : 1][3];   // dk/dG of the columns q0 + 3, q0 + 2, q0 + 1 of group g's open quad
+#pragma unroll
+        for (int i = 0; i < H; ++i) { A[i] = zero2; V[i] = zero2; }
+#pragma unroll
+        for (int g = 0; g < NH; ++g) { CN[g] = CO[g] = CNP[g] = gN[g] = gO[g] = zero2; }
+#pragma unroll
+        for (int g = 0; g < (QUADS ? NG : 1); ++g) carry[g][0] = carry[g][1] = carry[g][2] = 0.f;
+        auto restore = [&](int64_t slot) {   // the forward's state
+            const float4 *src = ck + slot * (TH * 2 / 4);
+#pragma unroll
+            for (int i = 0; i < H; i += 2) {
+                const float4 k = src[i / 2], q = src[(H + i) / 2];
+                KP[i] = make_float2(k.x, k.y);
+                KP[i + 1] = make_float2(k.z, k.w);
+                QN[i] = make_float2(-q.x, -q.y);
+                QN[i + 1] = make_float2(-q.z, -q.w);
+            }
+        };
+        restore(0);
+
+        // chunk c: lane j holds step t = top - 32 c - j
+        bool timed_out = false;
+        float4 nxt;
+        auto load_v = [&](int c) {   // the lower strip's V, or the seed V(Ni+1, Nj) = 1
+            const int col = top - 32 * c - lane - (TH - 1);
+            if (below) nxt.w = col >= 0 && col < nj ? ld_relaxed(below + col) : 0.f;
+            else nxt.w = col == nj - 1 ? 1.f : 0.f;
+        };
+        auto load_chunk = [&](int c) {
+            const int t = top - 32 * c - lane, bc = t - TH;   // bc: the last row's column before the step
+            nxt.x = topb && t >= 0 && t < nj ? topb[(int64_t)t * 2] : 1.f;
+            // beyond the grid's last column every value is virtual and meets only zero adjoints
+            const bool in = bc >= 0 && bc < nj;
+            nxt.y = in ? botb[(int64_t)bc * 2] : 1.f;
+            nxt.z = in ? -botb[(int64_t)bc * 2 + 1] : 0.f;
+            load_v(c);
+        };
+        auto wait_chunk = [&](int c) {
+            const long long t0 = clock64();
+            while (!timed_out && __any_sync(FULL, unwritten(nxt.w))) {
+                if (__any_sync(FULL, clock64() - t0 > a.wait_cycles)) {
+                    timed_out = true;
+                    if (lane == 0) atomicExch(a.status, (int)SIGK_ETIMEOUT);
+                    break;
+                }
+                __nanosleep(100);
+                load_v(c);
+            }
+        };
+        if (below) {   // start once chunks 0 and 1 are written
+            load_chunk(1);
+            wait_chunk(1);
+        }
+        load_chunk(0);
+
+        // coefficient diagonals, NRING - 1 windows ahead (those the buffer does not hold are zero)
+        const int wtop = (top + 1) / S - 1;
+        auto fetch = [&](int w) {
+            float *dst = ringc + (w & (NRING - 1)) * CP + lane * NG;
+            if (w >= 0 && w < pp.nw) {
+                ring_fetch<float, NG>(dst, blk + (int64_t)w * CP);
+            } else if (w >= 0) {
+#pragma unroll
+                for (int g = 0; g < NG; ++g) dst[g] = 0.f;
+            }
+            ring_commit();
+        };
+        auto read = [&](float2 (&c)[NH], int w) {
+            const float *cw = ringc + (w & (NRING - 1)) * CP + lane * NG;
+#pragma unroll
+            for (int g = 0; g < NH; ++g) c[g] = make_float2(cw[g], cw[g + NH]);
+        };
+#pragma unroll 1
+        for (int k = 0; k < NRING - 1; ++k) fetch(wtop - k);
+        ring_wait<NRING - 2>();
+        read(CO, wtop);
+
+        for (int wb = wtop - 3; wb >= 0; wb -= 4) {
+            const int u0 = top - (wb * S + GS - 1);   // the group's first step, counted from top
+            if (u0 % 32 == 0) {
+                const int c = u0 / 32;
+                wait_chunk(c);
+                __syncwarp();
+                cur.v[lane] = nxt;
+                __syncwarp();
+                if (AHEAD == 32) load_chunk(c + 1);
+                if (u0 % CK == 0 && u0 > 0) restore(1 + u0 / CK);
+            } else if (AHEAD == 16 && u0 % 32 == 16) {
+                load_chunk(u0 / 32 + 1);
+            }
+#pragma unroll
+            for (int w4 = 3; w4 >= 0; --w4) {
+                const int w = wb + w4;
+                // diagonal w - (NRING - 1) into the slot read last window; w - 1 has landed
+                fetch(w - (NRING - 1));
+                ring_wait<NRING - 2>();
+#pragma unroll
+                for (int g = 0; g < NH; ++g) { CNP[g] = CN[g]; CN[g] = CO[g]; }
+                if (w > 0) {
+                    read(CO, w - 1);
+                } else {
+#pragma unroll
+                    for (int g = 0; g < NH; ++g) CO[g] = zero2;
+                }
+#pragma unroll
+                for (int jj = S - 1; jj >= 0; --jj) {
+                    const int t = w * S + jj;
+                    if (t >= tend) continue;   // (warp-uniform, the first group only)
+                    const float4 ev = cur.v[(top - t) & 31];
+                    const float vH = V[0].y;
+                    float vd = __shfl_down_sync(FULL, V[0].x, 1);
+                    if (lane == 31) vd = ev.w;
+                    // undo step t: K before it, the cells' sums, -Q of the row above
+                    const float2 KlH = add(KP[H - 1], QN[H - 1]);
+                    float kup = __shfl_up_sync(FULL, KlH.y, 1);
+                    if (lane == 0) kup = ev.x;
+                    float2 kprev = make_float2(kup, KlH.x), t0 = zero2;
+#pragma unroll
+                    for (int i = 0; i < H; ++i) {
+                        const int g1 = i / S, s1 = i % S;   // row i; row i + H: group g1 + NH, same s1
+                        const float2 Kl = i == H - 1 ? KlH : add(KP[i], QN[i]);
+                        const float2 sum = add(Kl, kprev);
+                        const float2 c = jj >= s1 ? CN[g1] : CO[g1];
+                        const float2 tq = mad(c, sum, QN[i]);
+                        if (i == 0) t0 = tq;
+                        else QN[i - 1] = tq;
+                        KP[i] = Kl;
+                        kprev = Kl;
+                        const float2 vb = i < H - 1 ? V[i < H - 1 ? i + 1 : 0] : make_float2(vH, vd);
+                        // the row's coefficient one forward step later
+                        const float2 cp = jj < S - 1 ? (jj + 1 >= s1 ? CN[g1] : CO[g1]) : (s1 == 0 ? CNP[g1] : CN[g1]);
+                        const float2 P = mad(cp, A[i], vb);
+                        A[i] = add(A[i], P);
+                        V[i] = mad(c, A[i], P);
+                        if (jj >= s1) gN[g1] = mad(A[i], sum, gN[g1]);
+                        else gO[g1] = mad(A[i], sum, gO[g1]);
+                    }
+                    const float qd = __shfl_down_sync(FULL, t0.x, 1);
+                    // the strip's last row takes its own bottom row, kept by the forward
+                    QN[H - 1] = make_float2(t0.y, lane == 31 ? ev.z : qd);
+                    if (lane == 31) KP[H - 1].y = ev.y;
+                    // lane 0's first row is at column t: its V goes to the strip above
+                    if (above) st_boundary_if(above + t, V[0].x, lane == 0 && t < nj);
+                }
+                // diagonal w is complete
+                if (a.scheme != SIGK_SCHEME_EXPLICIT) {
+#pragma unroll
+                    for (int g = 0; g < NH; ++g) {
+                        gN[g].x *= scheme_dcoef(CN[g].x, a.scheme);
+                        gN[g].y *= scheme_dcoef(CN[g].y, a.scheme);
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    const float v = g < NH ? gN[g % NH].x : gN[g % NH].y;
+                    const int q = w - NG * lane - g;
+                    const bool row = prow + g >= 0 && prow + g < pp.nx;
+                    if constexpr (QUADS) {
+                        // q % 4 = (w4 - g) % 4: the quad's other columns came before
+                        const int m = (w4 - g) & 3;
+                        if (m > 0) {
+                            carry[g][3 - m] = v;
+                        } else if (row && q >= 0 && q < pp.ny) {
+                            *reinterpret_cast<float4 *>(gp + (int64_t)g * ld + q) =
+                                make_float4(v, carry[g][2], carry[g][1], carry[g][0]);
+                        }
+                    } else if (row && q >= 0 && q < pp.ny) {
+                        gp[(int64_t)g * ld + q] = v;
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < NH; ++g) { gN[g] = gO[g]; gO[g] = zero2; }
+            }
+        }
+        ring_wait<0>();
+        __syncwarp();
     }
 }
 
@@ -1592,7 +1852,7 @@ static StripLayout strip_layout_bwd(int64_t n, int64_t max_la, int64_t max_lb, i
     // checkpoints: (K, Q) of the strip's 32 R rows after every ck-th step
     const int64_t ck = strip_ck_of(es);
     L.ckpt = off;
-    off += al256(n * ns * ((nj + TH - 1 + ck - 1) / ck) * TH * 2 * es);
+    off += al256(n * ns * strip_ckpts(nj + TH - 1, ck) * TH * 2 * es);
     L.gbar = off;
     off += al256(n * nx * gbar_ld((int)ny) * es);
     L.total = off;
@@ -1873,15 +2133,22 @@ static cudaError_t launch_strip_bwd_t(const PairSrc &src, int64_t n, void *ws, c
         a.gbar = (T *)(w + L.gbar);
         a.wait_cycles = wait_cycles;
         a.scheme = src.scheme;
-        auto ak = strip_adj_kernel<T, R, LAM>;
-        const int asmem = STRIP_WARPS * adj_warp_elems<T, R, LAM>() * (int)sizeof(T);
-        if ((e = cudaFuncSetAttribute(ak, cudaFuncAttributeMaxDynamicSharedMemorySize, asmem)) != cudaSuccess)
-            return e;
-        int per_sm = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ak, STRIP_WARPS * 32, asmem)) != cudaSuccess)
-            return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        ak<<<strip_grid(L, sms, per_sm), STRIP_WARPS * 32, asmem, st>>>(a);
+        auto go = [&](auto ak, int asmem) {
+            cudaError_t r;
+            if ((r = cudaFuncSetAttribute(ak, cudaFuncAttributeMaxDynamicSharedMemorySize, asmem)) != cudaSuccess)
+                return r;
+            int per_sm = 0;
+            if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ak, STRIP_WARPS * 32, asmem)) != cudaSuccess)
+                return r;
+            if (per_sm < 1) return cudaErrorInvalidConfiguration;
+            ak<<<strip_grid(L, sms, per_sm), STRIP_WARPS * 32, asmem, st>>>(a);
+            return cudaGetLastError();
+        };
+        if constexpr (sizeof(T) == 4)
+            e = go(strip_adj_pack_kernel<R, LAM>, STRIP_WARPS * adjp_warp_floats<R, LAM>() * (int)sizeof(float));
+        else
+            e = go(strip_adj_kernel<T, R, LAM>, STRIP_WARPS * adj_warp_elems<T, R, LAM>() * (int)sizeof(T));
+        if (e != cudaSuccess) return e;
     }
     const T scale = (T)0.5 / (T)(1LL << (2 * LAM));
     {
