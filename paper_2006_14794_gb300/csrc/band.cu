@@ -21,6 +21,8 @@
 // each lane's kept whole ([pair][pos][lane][w][g]).
 #include <string.h>
 
+#include <type_traits>
+
 #include "sigk_internal.cuh"
 #include "tc5.cuh"
 #include "tile_gemm.cuh"
@@ -1136,6 +1138,182 @@ __global__ void __launch_bounds__(256) band_gemm_kernel(GemmArgs a) {
     }
 }
 
+// The same contraction with the row role's increments as output (not trans), for
+// lanes of 4 or 8 coarse rows: no tile is turned.  A thread owns the NG rows of a
+// lane and four channels (a block: 128 rows by 32 channels, as above), and takes
+// the lane's slots as they lie: window w holds the pairs (dk/dc of row h, of row
+// h + NG/2), which meet the columns j = NG - 1 + w - h and j - NG/2 of the
+// position; the column increments are kept in shared memory as those pairs, so
+// a window is NG/2 float2s of dk/dc, one new pair of column rows and 2 NG packed
+// FMAs with no moves, about half of the FP32 pipe's time in shared-memory
+// wavefronts.  POS positions (32 columns) a stage, double-buffered: slots by
+// cp.async, the columns through registers.  Each output adds the columns of its
+// share of the reduction in the same order as band_gemm_kernel, bit for bit (a
+// Gram's gradients are sums of 10^4 terms that cancel: another order moves them by
+// 1e-5).  128 x 128 Gram of 256-point paths, N = 32: 2.98 ms a launch through
+// turned tiles (which still take the transposed contraction and two rows a
+// lane), 2.3 here.
+template <int NG>
+struct GrStage {
+    static constexpr int LANES = 128 / NG, THREADS = 8 * LANES;
+    static constexpr int POS = 32 / NG, SLOT = NG * NG, SS = SLOT + 4;   // padded: 4 lanes, 4 bank quads
+    static constexpr int ROWS = (POS + 1) * NG;                          // column rows, from NG - 1 before the stage's first
+    float g[POS][LANES][SS];
+    float y[ROWS][2][8][4];   // row j: for channel quad c, halves of the pairs (y[j], y[j - NG/2]) of its 4 channels
+};
+
+template <int NG>
+__global__ void __launch_bounds__(GrStage<NG>::THREADS, 512 / GrStage<NG>::THREADS) band_rows_kernel(GemmArgs a) {
+    using St = GrStage<NG>;
+    constexpr int NH = NG / 2, POS = St::POS, SLOT = St::SLOT, ROWS = St::ROWS, NT = St::THREADS, LANES = St::LANES;
+    constexpr int YV = (ROWS * 32 + NT - 1) / NT;   // column values a thread stages
+    extern __shared__ __align__(16) float gr_sm[];
+    St *st = reinterpret_cast<St *>(gr_sm);         // two of them
+    const int tid = threadIdx.x, l = tid >> 3, cq = tid & 7;
+    const int64_t b = blockIdx.z / a.ksplit;
+    const int ks = blockIdx.z - (int)b * a.ksplit;
+    const float *Bm = a.Bm + b * a.b_bstride;
+    float *C = a.C + b * a.c_bstride;
+    constexpr int TPP = 32 / LANES;                 // blocks a path
+    const int64_t opath = blockIdx.x / TPP;
+    const int l0 = (int)(blockIdx.x - opath * TPP) * LANES;
+    const int n0 = blockIdx.y * 32;
+    // the share in slices of 32 columns; a slice is POS positions, and cells of
+    // its last columns lie in the position after it
+    const int TperR = a.TperR1 - 1, spp = (TperR + POS - 1) / POS;
+    const int64_t rlo = a.mode == PM_GRAM_SYM ? opath : 0;
+    const int64_t total = (a.nB - rlo) * spp;
+    const int64_t s_lo = total * ks / a.ksplit, s_hi = total * (ks + 1) / a.ksplit;
+
+    // a stage: positions p .. of path rp, which the share visits from pb to pe
+    struct Walk { int64_t rp; int p, pb, pe; };
+    auto open = [&](int64_t path, int slice) {
+        Walk w;
+        w.rp = path;
+        w.pb = w.p = slice * POS;
+        const int64_t left = s_hi - path * spp;   // slices of this path before the share's end
+        w.pe = left >= spp ? TperR : (int)left * POS;
+        return w;
+    };
+    auto next = [&](const Walk &w) {
+        if (w.p + POS <= w.pe) {
+            Walk n = w;
+            n.p += POS;
+            return n;
+        }
+        return open(w.rp + 1, 0);
+    };
+    auto ended = [&](const Walk &w) { return w.rp * spp >= s_hi; };
+
+    float yr[YV];
+    // a stage's slots into buffer buf (cp.async), its columns into registers
+    auto fetch = [&](const Walk &w, int buf) {
+        const int64_t k = gemm_pair(a, b, opath, rlo + w.rp);
+        const float *src = a.band + ((k * a.TperR1 + w.p) * 32 + l0) * (int64_t)SLOT;
+#pragma unroll
+        for (int i = 0; i < POS * LANES * (SLOT / 4) / NT; ++i) {
+            const int v = tid + NT * i, sl = v / (SLOT / 4), e = v - sl * (SLOT / 4), pr = sl / LANES, lr = sl % LANES;
+            float *dst = &st[buf].g[pr][lr][4 * e];
+            if (w.p + pr <= w.pe) cp_async<16>(dst, src + (pr * 32 + lr) * SLOT + 4 * e);
+        }
+        cp_commit();
+#pragma unroll
+        for (int i = 0; i < YV; ++i) {
+            const int v = tid + NT * i, j = v >> 5, n = n0 + (v & 31);
+            const int q = (w.p - 1) * NG + j + 1 - a.NQV;   // row j: Q = p NG - (NG - 1) + j
+            yr[i] = j < ROWS && q >= 0 && q < a.ny && n < a.N ? __ldg(Bm + ((rlo + w.rp) * a.ny + q) * a.N + n) : 0.f;
+        }
+    };
+    auto put_y = [&](int buf) {
+#pragma unroll
+        for (int i = 0; i < YV; ++i) {
+            const int v = tid + NT * i, j = v >> 5, c = v & 31;
+            if (j >= ROWS) continue;
+            // channel c of quad c / 4: pair c % 2 of half (c % 4) / 2
+            st[buf].y[j][(c & 3) >> 1][c >> 2][2 * (c & 1)] = yr[i];
+            if (j + NH < ROWS) st[buf].y[j + NH][(c & 3) >> 1][c >> 2][2 * (c & 1) + 1] = yr[i];
+        }
+    };
+    float2 acc[NH][4];
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[h][c] = make_float2(0.f, 0.f);
+
+    Walk wn = open(s_lo / spp, (int)(s_lo % spp));
+    if (s_lo < s_hi) fetch(wn, 0);
+    for (int buf = 0; s_lo < s_hi && !ended(wn); buf ^= 1) {
+        const Walk wk = wn;
+        wn = next(wk);
+        put_y(buf);
+        cp_wait<0>();
+        __syncthreads();   // the stage is complete, and the other buffer's readers are done
+        if (!ended(wn)) fetch(wn, buf ^ 1);
+        const St &S = st[buf];
+        // column pairs j in yv[j % NG]; a position's window 0 needs j = NH .. NG - 1
+        float2 yv[NG][4];
+        auto get_y = [&](int j, float2 (&v)[4]) {
+            const float4 u = *reinterpret_cast<const float4 *>(S.y[j][0][cq]);
+            const float4 w = *reinterpret_cast<const float4 *>(S.y[j][1][cq]);
+            v[0] = make_float2(u.x, u.y);
+            v[1] = make_float2(u.z, u.w);
+            v[2] = make_float2(w.x, w.y);
+            v[3] = make_float2(w.z, w.w);
+        };
+#pragma unroll
+        for (int j = NH; j < NG - 1; ++j) get_y(j, yv[j]);
+        // EDGE 1: the first position of a path's visit, whose cells w < g are
+        // columns before it (of another share, or of the previous pair); 2: the
+        // last, whose cells w >= g are columns after it.  They count as zero
+        // whatever the slots hold
+        auto position = [&](int pr, auto edge_tag) {
+            constexpr int EDGE = decltype(edge_tag)::value;
+            const float *sl = S.g[pr][l];
+#pragma unroll
+            for (int w = 0; w < NG; ++w) {
+                get_y(pr * NG + NG - 1 + w, yv[(NG - 1 + w) % NG]);
+                float2 g[NH];
+#pragma unroll
+                for (int h = 0; h < NH; h += 2) {
+                    const float4 v = *reinterpret_cast<const float4 *>(sl + w * NG + 2 * h);
+                    g[h] = make_float2(v.x, v.y);
+                    g[h + 1] = make_float2(v.z, v.w);
+                }
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    if (EDGE == 1 ? w < h : EDGE == 2 && w >= h) g[h].x = 0.f;
+                    if (EDGE == 1 ? w < h + NH : EDGE == 2 && w >= h + NH) g[h].y = 0.f;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        acc[h][c] = fma2(g[h], yv[(NG - 1 + w - h) % NG][c], acc[h][c]);
+                }
+            }
+        };
+#pragma unroll 1
+        for (int pr = 0; pr < POS; ++pr) {
+            const int pos = wk.p + pr;
+            if (pos > wk.pe) break;
+            if (pos == wk.pb) position(pr, std::integral_constant<int, 1>{});
+            else if (pos == wk.pe) position(pr, std::integral_constant<int, 2>{});
+            else position(pr, std::integral_constant<int, 0>{});
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        const int real = (l0 + l) * NG + g - a.vrows;
+        if (real < 0 || real >= a.nx) continue;
+        const int64_t r = opath * a.nx + real;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int n = n0 + 4 * cq + c;
+            if (n >= a.N) continue;
+            const float v = g < NH ? acc[g % NH][c].x : acc[g % NH][c].y;
+            if (a.ksplit > 1) a.partial[((int64_t)ks * a.M + r) * a.N + n] = v;
+            else C[r * a.N + n] = v;
+        }
+    }
+}
+
 // ---- the RBF lift's chain rule (Sec. 2.2) ---------------------------------
 // With c(p, q) = 1/2 4^-lambda (k(p+1,q+1) - k(p+1,q) - k(p,q+1) + k(p,q)),
 // k(i, j) = kappa(x_i, y_j) = exp(-|x_i - y_j|^2 / (2 sigma^2)), the adjoint's
@@ -2042,6 +2220,8 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             if (ksp > GEMM_MAX_SPLIT) ksp = GEMM_MAX_SPLIT;
             return (int)(ksp < 1 ? 1 : ksp);
         };
+        // the row role's contraction as the slots lie, for 4 and 8 rows a lane
+        const bool by_rows = p.NG >= 4;
         g1.ksplit = split(tiles1, nBall * ((NQc + GT_K - 1) / GT_K));
         g2.ksplit = split(tiles2, nA * (BHr / GT_K));
         g1.partial = g2.partial = part;
@@ -2086,7 +2266,18 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             if (tc) {
                 if ((e = launch_chain_gemm_tc5(as_chain(g1, 0), status, st)) != cudaSuccess) return e;
             } else {
-                gemm(gd1, g1);
+                if (by_rows) {
+                    auto go = [&](auto kern, int threads, int smem) {
+                        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                        if (r == cudaSuccess) kern<<<gd1, threads, smem, st>>>(g1);
+                        return r;
+                    };
+                    if (p.NG == 8) e = go(band_rows_kernel<8>, GrStage<8>::THREADS, 2 * (int)sizeof(GrStage<8>));
+                    else e = go(band_rows_kernel<4>, GrStage<4>::THREADS, 2 * (int)sizeof(GrStage<4>));
+                    if (e != cudaSuccess) return e;
+                } else {
+                    gemm(gd1, g1);
+                }
                 if (g1.ksplit > 1)
                     band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g1.ksplit, g1.M * d, 0, dincA);
             }
