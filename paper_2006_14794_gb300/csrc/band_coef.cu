@@ -52,7 +52,8 @@ template <int NG, bool RBF>
 struct KcShape {
     static constexpr int LW = NG == 8 ? 8 : 16, NP = NG == 8 ? 1 : NG == 4 ? 2 : 4;
     static constexpr int GP = 32 / LW * NP;   // positions a warp item
-    static constexpr int TILE = 36, WARPS = NG == 8 ? 12 : 9, MINB = NG == 8 ? 1 : 2;
+    static constexpr int TILE = 36, TILEC = 12;   // (TILEC: with more channels than are staged at once)
+    static constexpr int WARPS = NG == 8 ? 12 : 9, MINB = NG == 8 ? 1 : 2;
 };
 constexpr float KC_CARRY = 0.5f;   // see above: a, b <= e^1 - 1 along a slot
 
@@ -61,7 +62,8 @@ struct KcArgs {
     float *band;
     int64_t n_pairs;
     int TperR, NQV, vrows;
-    int tiles, tp, passes;   // units a pair, positions a unit, positions a warp
+    int tiles, tp, passes;   // units a pair, positions a unit, items a warp
+    int chunks, xch;         // channel chunks of a unit (more than one: one pass); row channels kept
     float scale, s;       // 1/2 4^-lambda, 1/(2 sigma^2)
 };
 
@@ -83,9 +85,9 @@ __host__ __device__ inline int kc_ys(int tp, int NG) { return (tp * NG + NG + 3)
 template <int NG>
 __host__ __device__ constexpr int kc_pp() { return NG == 8 ? 1 : 2; }
 template <int NG, bool RBF>
-__host__ __device__ inline int kc_smem_floats(int tp, int nch) {
+__host__ __device__ inline int kc_smem_floats(int tp, int nch, int xch) {
     const int ys = kc_ys(tp, NG), xs = kc_xs<NG>();
-    return RBF ? nch * ((3 + kc_pp<NG>()) * ys + 2 * xs) + ys + xs : nch * (3 * ys + xs);
+    return RBF ? nch * (3 + kc_pp<NG>()) * ys + 2 * xch * xs + ys + xs : nch * 3 * ys + xch * xs;
 }
 // threads that share a staged point's channels: the power of two at or above nc (32 at most)
 __device__ __forceinline__ int kc_group(int nc) { return nc > 16 ? 32 : nc > 8 ? 16 : nc > 4 ? 8 : 4; }
@@ -176,6 +178,34 @@ __device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs
         }
 }
 
+// kappa at the end of a step less kappa at its start, exponents E0 and E1 = E0 + x.
+__device__ __forceinline__ float kc_step(float E0, float E1, float x) {
+    return fabsf(x) <= 4.f ? __expf(E0) * expm1_taylor(x) : expf(E1) - expf(E0);
+}
+// The second difference of kappa over the cell of points x, x + d and y, y + d.
+// Where an exponent from corner (p, q) is above 4 in size (a jump of several
+// bandwidths: e^A overflows, or A cancels against |u|^2), it is the difference
+// of the two steps along the side with the smaller one, every corner from its
+// own distance.
+__device__ __forceinline__ float kc_second_difference(const float *x, const float *y, int64_t d, float s) {
+    float uu = 0.f, ux = 0.f, uy = 0.f, xy = 0.f, xx = 0.f, yy = 0.f;
+    for (int64_t i = 0; i < d; ++i) {
+        const float u = x[i] - y[i], dx = x[i + d] - x[i], dy = y[i + d] - y[i];
+        uu = fmaf(u, u, uu); ux = fmaf(u, dx, ux); uy = fmaf(u, dy, uy);
+        xy = fmaf(dx, dy, xy); xx = fmaf(dx, dx, xx); yy = fmaf(dy, dy, yy);
+    }
+    const float A = s * (2.f * uy - yy), B = -s * (2.f * ux + xx);
+    if (fmaxf(fabsf(A), fabsf(B)) <= 4.f) return rbf_second_difference(uu, ux, uy, xy, xx, yy, s);
+    float n01 = 0.f, n10 = 0.f, n11 = 0.f, ux1 = 0.f, uy1 = 0.f;
+    for (int64_t i = 0; i < d; ++i) {
+        const float u01 = x[i] - y[i + d], u10 = x[i + d] - y[i], u11 = x[i + d] - y[i + d];
+        n01 = fmaf(u01, u01, n01); n10 = fmaf(u10, u10, n10); n11 = fmaf(u11, u11, n11);
+        ux1 = fmaf(u01, x[i + d] - x[i], ux1); uy1 = fmaf(u10, y[i + d] - y[i], uy1);
+    }
+    return fabsf(A) >= fabsf(B) ? kc_step(-s * n01, -s * n11, -s * (2.f * ux1 + xx)) - kc_step(-s * uu, -s * n10, B)
+                                : kc_step(-s * n10, -s * n11, s * (2.f * uy1 - yy)) - kc_step(-s * uu, -s * n01, A);
+}
+
 // The slot's cells one by one from the points (RBF lift), stored as kc_store does.
 template <int NG>
 __device__ __noinline__ void kc_slot_direct(const KcArgs &a, int64_t k, int64_t row0, int64_t col0, int pos, int l) {
@@ -192,84 +222,55 @@ __device__ __noinline__ void kc_slot_direct(const KcArgs &a, int64_t k, int64_t 
         float c = 0.f;
         if (!other && p >= 0 && q >= 0 && q < ny) {
             const float *x = (const float *)a.src.A + (row0 + p) * d, *y = (const float *)a.src.B + (col0 + q) * d;
-            float uu = 0.f, ux = 0.f, uy = 0.f, xy = 0.f, xx = 0.f, yy = 0.f;
-            for (int64_t i = 0; i < d; ++i) {
-                const float u = x[i] - y[i], dx = x[i + d] - x[i], dy = y[i + d] - y[i];
-                uu = fmaf(u, u, uu); ux = fmaf(u, dx, ux); uy = fmaf(u, dy, uy);
-                xy = fmaf(dx, dy, xy); xx = fmaf(dx, dx, xx); yy = fmaf(dy, dy, yy);
-            }
-            c = scheme_coef(rbf_second_difference(uu, ux, uy, xy, xx, yy, a.s) * a.scale, a.src.scheme);
+            c = scheme_coef(kc_second_difference(x, y, d, a.s) * a.scale, a.src.scheme);
         }
         dst[band_off(w * NG + 2 * (g % (NG / 2)) + g / (NG / 2))] = c;
     }
 }
 
+// The sums of a slot's first cells (RBF lift): rows h, h + NG/2 at entry NG - 1 -
+// h of the column pairs (|u|^2, <u,dx>, <u,dy>), and row 0 in windows NG/2 + i and
+// i at entry NG + NG/2 - 1 + i (<u,dy>).
+template <int NG>
+struct KcFirst {
+    static constexpr int NH = NG / 2;
+    float2 uu[NH], ux[NH], uy[NH], ur[NH];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int h = 0; h < NH; ++h) uu[h] = ux[h] = uy[h] = ur[h] = kc2(0.f);
+    }
+    // channel c: the lane's row points and increments, the columns' increments and points
+    __device__ __forceinline__ void add(const float *xp, const float *xi, const float2 *e, const float *q, int l) {
+        const float2 minus = kc2(-1.f);
+        float2 xv[NH], dv[NH];
+        kc_rows<NG>(xv, xp, l);
+        kc_rows<NG>(dv, xi, l);
+        auto pts = [&](int j) {
+            if constexpr (kc_pp<NG>() == 2) return reinterpret_cast<const float2 *>(q)[j];
+            else return make_float2(q[j], q[j - NH]);
+        };
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const float2 u = __ffma2_rn(pts(NG - 1 - h), minus, xv[h]);
+            uu[h] = __ffma2_rn(u, u, uu[h]);
+            ux[h] = __ffma2_rn(u, dv[h], ux[h]);
+            uy[h] = __ffma2_rn(u, e[NG - 1 - h], uy[h]);
+            const float2 t = __ffma2_rn(pts(NG + NH - 1 + h), minus, kc2(xv[0].x));
+            ur[h] = __ffma2_rn(t, e[NG + NH - 1 + h], ur[h]);
+        }
+    }
+};
+
 // A slot's sums <dx,dy> into its coefficients (RBF lift).  Everything is done
 // for rows h and h + NG/2 at once; at window w row g is one column ahead of row
 // g + 1, so a(g + 1) of the next window is a(g) + (1 + a(g)) e(g) of this one.
-// The slot's first cells: rows h, h + NG/2 at entry NG - 1 - h of the column
-// pairs, and row 0 in windows NG/2 + i and i at entry NG + NG/2 - 1 + i.  Their
-// sums come from the staged channels, or (more channels than are staged at
-// once) from the points.  False where the slot was formed cell by cell.
+// False where the slot was formed cell by cell.
 template <int NG>
-__device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcArgs &a, int64_t k, const PairRef &pr,
-                                        int pos, int l, const float *xi, const float *xp, const float *xx,
-                                        const float2 *yi, const float *yp, const float *yy, int YS) {
-    constexpr int NH = NG / 2, XS = kc_xs<NG>();
+__device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcFirst<NG> &first, const KcArgs &a,
+                                        int64_t k, const PairRef &pr, int pos, int l, const float *xx,
+                                        const float *yy) {
+    constexpr int NH = NG / 2;
     const float s = a.s, s2 = 2.f * s;
-    const float2 minus = kc2(-1.f);
-    float2 uu[NH], ux[NH], uy[NH], ur[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) uu[h] = ux[h] = uy[h] = ur[h] = kc2(0.f);
-    if (a.src.d <= KC_CH) {
-#pragma unroll 1
-        for (int c = 0; c < (int)a.src.d; ++c) {
-            float2 xv[NH], dv[NH];
-            kc_rows<NG>(xv, xp + c * XS, l);
-            kc_rows<NG>(dv, xi + c * XS, l);
-            const float *q = yp + c * YS * kc_pp<NG>();
-            const float2 *e = yi + c * YS;
-            auto pts = [&](int j) {
-                if constexpr (kc_pp<NG>() == 2) return reinterpret_cast<const float2 *>(q)[j];
-                else return make_float2(q[j], q[j - NH]);
-            };
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                const float2 u = __ffma2_rn(pts(NG - 1 - h), minus, xv[h]);
-                uu[h] = __ffma2_rn(u, u, uu[h]);
-                ux[h] = __ffma2_rn(u, dv[h], ux[h]);
-                uy[h] = __ffma2_rn(u, e[NG - 1 - h], uy[h]);
-                const float2 t = __ffma2_rn(pts(NG + NH - 1 + h), minus, kc2(xv[0].x));
-                ur[h] = __ffma2_rn(t, e[NG + NH - 1 + h], ur[h]);
-            }
-        }
-    } else {
-        const int64_t d = a.src.d;
-        const int ny = (int)a.src.Lb - 1, P0 = l * NG - a.vrows, Q0 = pos * NG - (NG - 1) - a.NQV;
-        auto row = [&](int g) { return (const float *)a.src.A + (pr.a_row0 + (P0 + g < 0 ? 0 : P0 + g)) * d; };
-        auto col = [&](int j) {
-            const int q = Q0 + j;
-            return (const float *)a.src.B + (pr.b_row0 + (q < 0 ? 0 : q > ny ? ny : q)) * d;
-        };
-#pragma unroll 1
-        for (int64_t c = 0; c < d; ++c) {
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                const int ja = NG - 1 - h, jb = NH - 1 - h, jr = NG + NH - 1 + h, js = NG - 1 + h;
-                const float *ra = row(h), *rb = row(h + NH);
-                const float2 x = make_float2(ra[c], rb[c]);
-                const float2 dx = make_float2(P0 + h < 0 ? 0.f : ra[d + c] - x.x, P0 + h + NH < 0 ? 0.f : rb[d + c] - x.y);
-                const float2 y = make_float2(col(ja)[c], col(jb)[c]), z = make_float2(col(jr)[c], col(js)[c]);
-                const float2 dy = make_float2(col(ja + 1)[c] - y.x, col(jb + 1)[c] - y.y);
-                const float2 dz = make_float2(col(jr + 1)[c] - z.x, col(js + 1)[c] - z.y);
-                const float2 u = __ffma2_rn(y, minus, x), t = __ffma2_rn(z, minus, kc2(row(0)[c]));
-                uu[h] = __ffma2_rn(u, u, uu[h]);
-                ux[h] = __ffma2_rn(u, dx, ux[h]);
-                uy[h] = __ffma2_rn(u, dy, uy[h]);
-                ur[h] = __ffma2_rn(t, dz, ur[h]);
-            }
-        }
-    }
     float far = 0.f;
 #pragma unroll
     for (int w = 0; w < NG; ++w)
@@ -288,9 +289,9 @@ __device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcArgs 
     };
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
-        av[h] = arg(uy[h], make_float2(yy[NG - 1 - h], yy[NH - 1 - h]), 1.f);
-        top[h] = arg(ur[h], make_float2(yy[NG + NH - 1 + h], yy[NG - 1 + h]), 1.f);
-        bv[h] = arg(ux[h], sq[h], -1.f);
+        av[h] = arg(first.uy[h], make_float2(yy[NG - 1 - h], yy[NH - 1 - h]), 1.f);
+        top[h] = arg(first.ur[h], make_float2(yy[NG + NH - 1 + h], yy[NG - 1 + h]), 1.f);
+        bv[h] = arg(first.ux[h], sq[h], -1.f);
     }
     if (far > KC_CARRY) {
         kc_slot_direct<NG>(a, k, pr.a_row0, pr.b_row0, pos, l);
@@ -301,7 +302,7 @@ __device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcArgs 
         av[h] = kc_expm1<8>(av[h]);
         bv[h] = kc_expm1<8>(bv[h]);
         top[h] = kc_expm1<8>(top[h]);
-        kap[h] = make_float2(a.scale * __expf(-s * uu[h].x), a.scale * __expf(-s * uu[h].y));
+        kap[h] = make_float2(a.scale * __expf(-s * first.uu[h].x), a.scale * __expf(-s * first.uu[h].y));
     }
 #pragma unroll
     for (int w = 0; w < NG; ++w) {
@@ -323,7 +324,9 @@ __device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcArgs 
     return true;
 }
 
-template <int NG, bool RBF>
+// MULTI: more channels than are staged at once (one pass; sums kept over the
+// chunks, in more registers than the common case needs)
+template <int NG, bool RBF, bool MULTI>
 __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>::MINB) band_coef_kernel(KcArgs a) {
     extern __shared__ __align__(16) float kc_sm[];
     constexpr int NPP = 32 * NG, XS = kc_xs<NG>(), NP = KcShape<NG, RBF>::NP, NH = NG / 2;
@@ -333,19 +336,21 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
     const int64_t d = a.src.d;
     const int nch = d < KC_CH ? (int)d : KC_CH, YS = kc_ys(a.tp, NG);
     float *xi = kc_sm;                                            // row increments (linear: scaled)
-    float *y0 = xi + nch * XS;                                    // the next unit's column points
+    float *y0 = xi + a.xch * XS;                                  // the next step's column points
     float2 *yi = reinterpret_cast<float2 *>(y0 + nch * YS);       // pairs of column increments
-    float *yp = reinterpret_cast<float *>(yi + nch * YS);         // RBF: this unit's column points,
+    float *yp = reinterpret_cast<float *>(yi + nch * YS);         // RBF: this step's column points,
     float *xp = yp + nch * YS * kc_pp<NG>();                      // row points, and the squared
-    float *xx = xp + nch * XS, *yy = xx + XS;                     // increments of rows and columns
+    float *xx = xp + a.xch * XS, *yy = xx + XS;                   // increments of rows and columns
     const int64_t units = a.n_pairs * a.tiles, per = (units + gridDim.x - 1) / gridDim.x;
     const int64_t ubeg = (int64_t)blockIdx.x * per;
     const int64_t uend = ubeg + per < units ? ubeg + per : units;
     if (ubeg >= uend) return;
     const int ny = (int)a.src.Lb - 1;
-    const bool once = d <= KC_CH;   // all channels staged at once
+    const bool keep = !MULTI || a.xch == (int)d;   // all of a row path's channels stay
+    const int chunks = MULTI ? a.chunks : 1, passes = MULTI ? 1 : a.passes;
 
-    auto stage_x = [&](int64_t row0, int64_t c0, int nc) {
+    // channels c0 .. c0 + nc - 1 of the row path's increments (and points) from xi[at XS] on
+    auto stage_x = [&](int64_t row0, int64_t c0, int nc, int at) {
         const float *x = (const float *)a.src.A + row0 * d + c0;
         const int gs = kc_group(nc), c = tid & (gs - 1);
         if (c < nc)
@@ -353,8 +358,8 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
                 const int p = P - a.vrows;
                 const float *r = x + (int64_t)(p < 0 ? 0 : p) * d + c;
                 const float e = p >= 0 ? __ldg(r + d) - __ldg(r) : 0.f;
-                xi[c * XS + kc_xpos<NG>(P)] = RBF ? e : e * a.scale;
-                if (RBF) xp[c * XS + kc_xpos<NG>(P)] = __ldg(r);
+                xi[(at + c) * XS + kc_xpos<NG>(P)] = RBF ? e : e * a.scale;
+                if (RBF) xp[(at + c) * XS + kc_xpos<NG>(P)] = __ldg(r);
             }
     };
     // tile t's column points, ends repeated, into y0[c][iq], Q = t tp NG + iq - (NG - 1)
@@ -370,8 +375,8 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
         kc_commit();
     };
     // the pairs (column iq, column iq - NG/2) from the fetched points; RBF: and the
-    // squared increments, over the channels so far (rows' where they were staged)
-    auto pair_y = [&](int64_t c0, int nc, bool rows) {
+    // squared increments, over the channels so far (rows': of the xc staged from c0)
+    auto pair_y = [&](int64_t c0, int nc, int xc) {
         for (int iq = tid; iq < YS; iq += nt) {
             float sq = RBF && c0 > 0 ? yy[iq] : 0.f;
             const int ib = iq >= NH ? iq - NH : 0, hi = iq + 1 < YS ? 1 : 0;
@@ -390,19 +395,21 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
             }
             if (RBF) yy[iq] = sq;
         }
-        if (RBF && rows)
+        if (RBF && xc > 0)
             for (int P = tid; P < NPP; P += nt) {
                 float sq = c0 > 0 ? xx[P] : 0.f;
-                for (int c = 0; c < nc; ++c) sq = fmaf(xi[c * XS + P], xi[c * XS + P], sq);
+                for (int c = 0; c < xc; ++c) sq = fmaf(xi[c * XS + P], xi[c * XS + P], sq);
                 xx[P] = sq;   // in the staged order, as xi
             }
     };
 
-    int64_t kn = ubeg / a.tiles;          // the next unit's pair and tile
+    int64_t kn = ubeg / a.tiles;          // the next step's pair and tile
     int tn = (int)(ubeg - kn * a.tiles);
     PairRef pr = pair_ref(a.src, kn);
     int64_t staged = -1;   // the row path whose values xi (and xp) hold
-    if (once) fetch_y(pr.b_row0, tn, 0, (int)d);
+    fetch_y(pr.b_row0, tn, 0, nch);
+    float2 acc[NP][NG][NH];
+    KcFirst<NG> first[RBF && MULTI ? NP : 1];
     for (int64_t u = ubeg; u < uend; ++u) {
         const PairRef cur = pr;
         const int64_t k = kn;
@@ -412,48 +419,49 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
             tn = 0;
             pr = pair_ref(a.src, ++kn);
         }
-        if (once) {
+        for (int ch = 0; ch < chunks; ++ch) {
+            const int64_t c0 = (int64_t)ch * KC_CH;
+            const int nc = d - c0 < KC_CH ? (int)(d - c0) : KC_CH;
             kc_wait();
-            __syncthreads();   // this unit's columns are here, and the last unit's readers are done
-            const bool fresh = staged != cur.a_row0;
+            __syncthreads();   // this step's columns are here, and the last step's readers are done
+            const bool fresh = !keep || staged != cur.a_row0;
             if (fresh) {
-                stage_x(cur.a_row0, 0, (int)d);
+                if (keep)
+                    for (int64_t c = 0; c < d; c += KC_CH)
+                        stage_x(cur.a_row0, c, d - c < KC_CH ? (int)(d - c) : KC_CH, (int)c);
+                else
+                    stage_x(cur.a_row0, c0, nc, 0);
                 staged = cur.a_row0;
                 if (RBF) __syncthreads();
             }
-            pair_y(0, (int)d, fresh);
+            pair_y(c0, nc, !fresh ? 0 : keep ? (int)d : nc);
             __syncthreads();
-            if (more) fetch_y(pr.b_row0, tn, 0, (int)d);
-        }
-        for (int pass = 0; pass < a.passes; ++pass) {
-            // the warp's item: a block of lanes and a group of positions
-            const int item = pass * (nt >> 5) + warp, l = item % (32 / Sh::LW) * Sh::LW + lw;
-            const int first = item / (32 / Sh::LW) * Sh::GP + jw * NP;
-            const bool live = first < a.tp && t * a.tp + first <= a.TperR;
-            const int rel = live ? first : 0, pos = t * a.tp + rel;
-            float2 acc[NP][NG][NH];
+            if (ch + 1 < chunks) fetch_y(cur.b_row0, t, c0 + KC_CH, d - c0 - KC_CH < KC_CH ? (int)(d - c0 - KC_CH) : KC_CH);
+            else if (more) fetch_y(pr.b_row0, tn, 0, nch);
+            const float *xc = xi + (keep ? (int)c0 * XS : 0), *xq = xp + (keep ? (int)c0 * XS : 0);
+            for (int pass = 0; pass < passes; ++pass) {
+                // the warp's item: a block of lanes and a group of positions
+                const int item = pass * (nt >> 5) + warp, l = item % (32 / Sh::LW) * Sh::LW + lw;
+                const int off = item / (32 / Sh::LW) * Sh::GP + jw * NP;
+                const bool live = off < a.tp && t * a.tp + off <= a.TperR;
+                const int rel = live ? off : 0, pos = t * a.tp + rel;
+                if (ch == 0) {
 #pragma unroll
-            for (int n = 0; n < NP; ++n)
+                    for (int n = 0; n < NP; ++n)
 #pragma unroll
-                for (int w = 0; w < NG; ++w)
+                        for (int w = 0; w < NG; ++w)
 #pragma unroll
-                    for (int h = 0; h < NH; ++h) acc[n][w][h] = make_float2(0.f, 0.f);
-            for (int64_t c0 = 0; c0 < d; c0 += KC_CH) {
-                const int nc = d - c0 < KC_CH ? (int)(d - c0) : KC_CH;
-                if (!once) {
-                    __syncthreads();
-                    stage_x(cur.a_row0, c0, nc);
-                    fetch_y(cur.b_row0, t, c0, nc);
-                    kc_wait();
-                    __syncthreads();
-                    pair_y(c0, nc, true);
-                    __syncthreads();
+                            for (int h = 0; h < NH; ++h) acc[n][w][h] = make_float2(0.f, 0.f);
+                    if constexpr (RBF && MULTI) {
+#pragma unroll
+                        for (int n = 0; n < NP; ++n) first[n].clear();
+                    }
                 }
                 const float2 *yr = yi + rel * NG;   // entry j: columns Q = pos NG - (NG - 1) + j and Q - NG/2
 #pragma unroll 2
                 for (int c = 0; c < nc; ++c) {
                     float2 xv[NH], yv[(NP + 1) * NG - NH];
-                    kc_rows<NG>(xv, xi + c * XS, l);
+                    kc_rows<NG>(xv, xc + c * XS, l);
                     kc_cols<NG>(yv, yr + c * YS + NH);
 #pragma unroll
                     for (int n = 0; n < NP; ++n)
@@ -463,24 +471,38 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
                             for (int h = 0; h < NH; ++h)
                                 acc[n][w][h] = __ffma2_rn(xv[h], yv[n * NG + w - h + NG - 1 - NH], acc[n][w][h]);
                 }
-            }
-            if (!live) continue;
+                auto add_first = [&](KcFirst<NG> &f, int n) {
+#pragma unroll 1
+                    for (int c = 0; c < nc; ++c)
+                        f.add(xq + c * XS, xc + c * XS, yr + c * YS + n * NG,
+                              yp + (c * YS + (rel + n) * NG) * kc_pp<NG>(), l);
+                };
+                if constexpr (RBF && MULTI) {
 #pragma unroll
-            for (int n = 0; n < NP; ++n) {
-                if (n > 0 && (rel + n >= a.tp || pos + n > a.TperR)) break;
-                if constexpr (RBF)
-                    if (!kc_lift<NG>(acc[n], a, k, cur, pos + n, l, xi, xp, xx, yi + (rel + n) * NG,
-                                     yp + (rel + n) * NG * kc_pp<NG>(), yy + (rel + n) * NG, YS))
-                        continue;
-                if (a.src.scheme != SIGK_SCHEME_EXPLICIT) {
-#pragma unroll
-                    for (int w = 0; w < NG; ++w)
-#pragma unroll
-                        for (int h = 0; h < NH; ++h)
-                            acc[n][w][h] = make_float2(scheme_coef(acc[n][w][h].x, a.src.scheme),
-                                                       scheme_coef(acc[n][w][h].y, a.src.scheme));
+                    for (int n = 0; n < NP; ++n) add_first(first[n], n);
                 }
-                kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos + n, l, acc[n]);
+                if (!live || ch + 1 < chunks) continue;
+#pragma unroll
+                for (int n = 0; n < NP; ++n) {
+                    if (n > 0 && (rel + n >= a.tp || pos + n > a.TperR)) break;
+                    if constexpr (RBF) {
+                        KcFirst<NG> &f = first[MULTI ? n : 0];
+                        if constexpr (!MULTI) {
+                            f.clear();
+                            add_first(f, n);
+                        }
+                        if (!kc_lift<NG>(acc[n], f, a, k, cur, pos + n, l, xx, yy + (rel + n) * NG)) continue;
+                    }
+                    if (a.src.scheme != SIGK_SCHEME_EXPLICIT) {
+#pragma unroll
+                        for (int w = 0; w < NG; ++w)
+#pragma unroll
+                            for (int h = 0; h < NH; ++h)
+                                acc[n][w][h] = make_float2(scheme_coef(acc[n][w][h].x, a.src.scheme),
+                                                           scheme_coef(acc[n][w][h].y, a.src.scheme));
+                    }
+                    kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos + n, l, acc[n]);
+                }
             }
         }
     }
@@ -491,22 +513,33 @@ cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
     KcArgs a = a0;
     const int npos = a.TperR + 1;
     using Sh = KcShape<NG, RBF>;
-    a.tiles = (npos + Sh::TILE - 1) / Sh::TILE;
+    const int d = (int)a.src.d, nch = d < KC_CH ? d : KC_CH;
+    a.chunks = (d + KC_CH - 1) / KC_CH;
+    const int most = a.chunks > 1 ? Sh::TILEC : Sh::TILE;
+    a.tiles = (npos + most - 1) / most;
     a.tp = ((npos + a.tiles - 1) / a.tiles + Sh::NP - 1) / Sh::NP * Sh::NP;
     const int items = (a.tp + Sh::GP - 1) / Sh::GP * (32 / Sh::LW);
-    a.passes = (items + Sh::WARPS - 1) / Sh::WARPS;
+    a.passes = a.chunks > 1 ? 1 : (items + Sh::WARPS - 1) / Sh::WARPS;
     const int warps = (items + a.passes - 1) / a.passes;
-    const int smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, (int)(a.src.d < KC_CH ? a.src.d : KC_CH));
-    auto kern = band_coef_kernel<NG, RBF>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem)) != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    int64_t grid = (int64_t)sms * per_sm;
-    if (grid > a.n_pairs * a.tiles) grid = a.n_pairs * a.tiles;
-    kern<<<(int)grid, warps * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    // a row path's channels all stay where they fit (two chunks do)
+    a.xch = d;
+    int smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch);
+    if (d <= 4 * KC_CH && (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d) <= 226 * 1024)
+        smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d);
+    else
+        a.xch = nch;
+    auto go = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem)) != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        int64_t grid = (int64_t)sms * per_sm;
+        if (grid > a.n_pairs * a.tiles) grid = a.n_pairs * a.tiles;
+        kern<<<(int)grid, warps * 32, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    return a.chunks > 1 ? go(band_coef_kernel<NG, RBF, true>) : go(band_coef_kernel<NG, RBF, false>);
 }
 
 }  // namespace
@@ -520,7 +553,7 @@ cudaError_t launch_band_coefs(const PairSrc &src, const BandPlan &p, int64_t n_p
     a.TperR = p.TperR;
     a.NQV = p.NQV;
     a.vrows = p.vrows;
-    a.tiles = a.tp = a.passes = 1;
+    a.tiles = a.tp = a.passes = a.chunks = a.xch = 1;
     a.scale = 0.5f / (float)(1 << (2 * p.lam));
     a.s = (float)(0.5 / (src.sigma * src.sigma));
     const bool rbf = src.kernel == SIGK_KERNEL_RBF;
