@@ -169,9 +169,10 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
     // the lane's slot in macro-step m (linear position m - lane of the chain), or
     // null outside the chain (its first pair's rows before they start, and after
     // the last pair except the slot that holds that pair's tail)
-    const float *band0 = a.band + band_row(k0 * TperR - lane, lane, NG);
+    const int64_t nslots = a.n_pairs * TperR + 1;
     auto slot = [&](int64_t m) -> const float * {
-        return m >= lane && m - lane <= (int64_t)np * TperR ? band0 + m * (32 * SLOT) : nullptr;
+        return m >= lane && m - lane <= (int64_t)np * TperR
+                   ? a.band + band_row(k0 * TperR + m - lane, lane, NG, nslots) : nullptr;
     };
     constexpr int D = band_ring<R, NG>();
     __shared__ __align__(16) float ring[D ? BAND_WARPS * D * 32 * SLOT : 1];
@@ -380,8 +381,8 @@ __global__ void __launch_bounds__(BT5_T, 1) band_coef_tc5_kernel(BandCoefArgs a,
             for (int v = tid; v < 32 * SLOT; v += BT5_T) {
                 const int l = v / SLOT, e = v - l * SLOT, w = e / NG, gp = e - w * NG;
                 const int g = (gp & 1) ? gp / 2 + NG / 2 : gp / 2;   // inverse of band_gpos
-                if (k == 0 && w < g) a.band[band_row(0, l, NG) + band_off(e)] = 0.f;
-                if (k == a.n_pairs - 1 && w >= g) a.band[band_row((k + 1) * TperR, l, NG) + band_off(e)] = 0.f;
+                if (k == 0 && w < g) a.band[band_row(0, l, NG, a.n_pairs * TperR + 1) + band_off(e)] = 0.f;
+                if (k == a.n_pairs - 1 && w >= g) a.band[band_row((k + 1) * TperR, l, NG, a.n_pairs * TperR + 1) + band_off(e)] = 0.f;
             }
         }
         for (int P0 = 0; P0 < NPP && !failed; P0 += BT5_M) {
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(BT5_T, 1) band_coef_tc5_kernel(BandCoefArgs a,
                     const float *srow = St + (P - P0) * BT5_SS;
                     // destination slot: the pair's own, or (the tail) the next pair's slot 0
                     const bool tail = pos == TperR;
-                    float *dst = a.band + band_row(tail ? (k + 1) * TperR : k * TperR + pos, l, NG);
+                    float *dst = a.band + band_row(tail ? (k + 1) * TperR : k * TperR + pos, l, NG, a.n_pairs * TperR + 1);
 #pragma unroll
                     for (int w = 0; w < NG; ++w) {
                         const int Q = pos * NG + w - g;
@@ -706,9 +707,10 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
         pos = (int)(mm - q * TperR);
     };
     // the lane's slot in macro-step m, as in the forward
-    const float *band0 = a.band + band_row(k0 * TperR - lane, lane, NG);
+    const int64_t nslots = a.n_pairs * TperR + 1;
     auto slot_ptr = [&](int64_t m) -> const float * {
-        return m >= lane && m - lane <= (int64_t)np * TperR ? band0 + m * (32 * SLOT) : nullptr;
+        return m >= lane && m - lane <= (int64_t)np * TperR
+                   ? a.band + band_row(k0 * TperR + m - lane, lane, NG, nslots) : nullptr;
     };
     // window w of macro-step m (slot src, null outside the chain) into buffer m % D;
     // with window NG-1 also the last row's Q
@@ -1678,13 +1680,13 @@ bool band_geometry(int64_t La, int64_t Lb, int lam, int rows_per_lane, BandPlan 
 
 // workspace: a 256-byte header (the status word of bounded waits), then the band
 int64_t band_bytes(const BandPlan &p, int64_t n_pairs) {
-    return 256 + (int64_t)sizeof(float) * (n_pairs * p.TperR + 32) * p.slot_floats;
+    return 256 + (int64_t)sizeof(float) * (n_pairs * p.TperR + 1) * p.slot_floats;
 }
 
 // The surface's band-layout values (TperR + 1 slots per pair) after the band:
 // their float offset from the band's start, and the whole workspace.
 int64_t band_surface_offset(const BandPlan &p, int64_t n_pairs) {
-    return ((n_pairs * p.TperR + 32) * p.slot_floats + 63) / 64 * 64;
+    return ((n_pairs * p.TperR + 1) * p.slot_floats + 63) / 64 * 64;
 }
 int64_t band_surface_bytes(const BandPlan &p, int64_t n_pairs) {
     return 256 + (int64_t)sizeof(float) *

@@ -156,7 +156,7 @@ template <int NG>
 __device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs, int TperR, int pos, int l,
                                          const float2 (&v)[NG][NG / 2]) {
     constexpr int SLOT = NG * NG, NH = NG / 2;
-    float *dst = band + band_row(k * TperR + pos, l, NG);   // (the tail: the next pair's slot 0)
+    float *dst = band + band_row(k * TperR + pos, l, NG, n_pairs * TperR + 1);   // (the tail: the next pair's slot 0)
     if (pos > 0 && pos < TperR) {
 #pragma unroll
         for (int i = 0; i < SLOT / 4; ++i) {
@@ -213,7 +213,7 @@ __device__ __noinline__ void kc_slot_direct(const KcArgs &a, int64_t k, int64_t 
     const int64_t d = a.src.d;
     const int ny = (int)a.src.Lb - 1;
     const bool tail = pos == a.TperR;
-    float *dst = a.band + band_row(k * a.TperR + pos, l, NG);   // tail: slot 0 of the next pair
+    float *dst = a.band + band_row(k * a.TperR + pos, l, NG, a.n_pairs * a.TperR + 1);   // tail: slot 0 of the next pair
     for (int e = 0; e < SLOT; ++e) {
         const int w = e / NG, g = e - w * NG;
         const bool other = tail ? w >= g : (pos == 0 && w < g);   // the neighbour pair's cell

@@ -183,13 +183,16 @@ struct BandPlan {
 };
 // The coefficient band: slot (pair k, position pos) of lane l, NG x NG floats,
 // element i = window NG + place in the window.  The slots of a launch's pairs
-// follow one another (linear position s = k TperR + pos), and lane l's slot s is
-// in row s + l: the row that holds what the 32 lanes of a sweep warp, one
-// position apart, read in one macro-step, four floats of a lane at a time next
-// to the neighbour lanes' (a window is one or two 512-byte runs; slots kept
-// whole per lane cost a sweep load or a producer store 32 cache lines instead).
-__host__ __device__ inline int64_t band_row(int64_t s, int l, int NG) {
-    return (s + l) * (32 * NG * NG) + 4 * l;
+// follow one another (linear position s = k TperR + pos, S = n TperR + 1 in all),
+// and lane l's slot s is in row (s + l) mod S: the row that holds what the 32
+// lanes of a sweep warp, one position apart, read in one macro-step, four floats
+// of a lane at a time next to the neighbour lanes' (a window is one or two
+// 512-byte runs; slots kept whole per lane cost a sweep load or a producer store
+// 32 cache lines instead).
+__host__ __device__ inline int64_t band_row(int64_t s, int l, int NG, int64_t S) {
+    s += l;
+    while (s >= S) s -= S;   // once, unless there are fewer slots than lanes
+    return s * (32 * NG * NG) + 4 * l;
 }
 // offset of element i in it
 __host__ __device__ constexpr int band_off(int i) { return (i / 4) * 128 + i % 4; }
