@@ -53,12 +53,13 @@ __host__ __device__ constexpr int vb_lane_stride(int NG) { return NG >= 8 ? NG +
 struct VbPair {
     int64_t r_row0, c_row0;    // first point rows of the row (shorter) and column paths
     int lr, lc;                // their lengths
-    int swapped;               // rows come from src.B (the Y paths)
     int cls;                   // band class; -1: a path with one point (k = 1)
     int T;                     // macro-steps
     int vrows, nqv;            // virtual coarse rows (top) and columns (left)
-    int first, last;           // first / last pair of its chain
-    int64_t base;              // float offset of the pair's slot 0 in the band
+    int s0, slots;             // the pair's first slot in its chain, the chain's slots
+    int8_t swapped;            // rows come from src.B (the Y paths)
+    int8_t first, last;        // first / last pair of its chain
+    int64_t base;              // float offset of the chain's band
     int64_t out0;              // output slot
 };
 
@@ -217,21 +218,23 @@ __global__ void __launch_bounds__(VB_PT) vb_plan_kernel(VbArgs a) {
         int c = 0;
         while (gc >= sChain0[c + 1]) ++c;
         const int ch = gc - sChain0[c], W = sW[c], cnt = a.cinfo[c].count, st = a.cinfo[c].start;
-        const int ng = vb_ng(a, c);
-        const int64_t slot = 32LL * ng * ng;
         const int np = vb_chain_len(ch, W, cnt);
-        int64_t base = a.scan[gc];
+        const int64_t base = a.scan[gc];
         a.chain_base[gc] = base;
         const int off = a.chain_off[gc];
+        int slots = 1, s0 = 0;
+        for (int j = 0; j < np; ++j) slots += a.plan[a.order[st + vb_snake(j, ch, W)]].T;
         for (int j = 0; j < np; ++j) {
             const int pid = a.order[st + vb_snake(j, ch, W)];
             VbPair &p = a.plan[pid];
             p.base = base;
+            p.s0 = s0;
+            p.slots = slots;
             p.first = j == 0;
             p.last = j == np - 1;
             a.cpid[off + j] = pid;
             a.cT[off + j] = p.T;
-            base += (int64_t)p.T * slot;
+            s0 += p.T;
         }
     }
 }
@@ -240,10 +243,32 @@ __global__ void __launch_bounds__(VB_PT) vb_plan_kernel(VbArgs a) {
 // band.  A thread computes WQ windows x NG groups of one slot (lane l,
 // position pos), each cell a d-term dot product of increments staged
 // channel-major in shared memory (as band_coef_kernel, with each pair's own
-// geometry).  Threads are numbered lane-fastest: the 32 threads of a warp are
-// the 32 lanes of one (position, window quarter), so they read the same
-// column increments (a broadcast) and their own row increments (rows padded
-// to a conflict-free stride, vb_lane_stride).
+// geometry).  The band of a chain is laid out as the uniform one (band_row:
+// slot s of lane l in row (s + l) mod the chain's slots), so that what a sweep
+// warp reads in a macro-step, its lanes one slot apart, is one row.  A warp
+// covers 8 lanes by 4 positions: a 16-byte store meets 11 rows, where the 32
+// lanes of one position (slots whole per lane) met 32 lines, which took the L1
+// twice the time of the operand reads; those are a broadcast over the
+// positions (rows, padded to a conflict-free stride, vb_lane_stride) or over
+// the lanes (columns).  4096 pairs of 16..512 points, d = 16, order 1: the call
+// 1.74 -> 1.41 ms, outputs bit for bit.
+// The unit (lane, position, part of a slot) of thread u of a pair, parts slowest
+// within a group of four positions.
+struct VbUnit {
+    int l, pos, part;
+};
+template <int PARTS>
+__device__ __forceinline__ VbUnit vb_unit(int u) {
+    const int i = u >> 5, q = i >> 2;   // warp item: lane block i & 3, then part, then positions
+    VbUnit v;
+    v.l = (i & 3) * 8 + (u & 7);
+    v.part = q % PARTS;
+    v.pos = q / PARTS * 4 + ((u >> 3) & 3);
+    return v;
+}
+template <int PARTS>
+__device__ __forceinline__ int vb_units(int T) { return 128 * ((T + 4) / 4) * PARTS; }   // T + 1 positions
+
 // Channel strides of the staged increments: multiples of 4 floats (16-byte
 // rows) that are 4 (mod 32), so the 8 channels a staging thread group writes
 // land in 8 bank quads.
@@ -290,7 +315,7 @@ __device__ __forceinline__ void vb_inc4(float (&e)[4], const float *x, int64_t d
 template <int NG, int WQ>
 __global__ void __launch_bounds__(VB_CT) vb_coef_kernel(VbArgs a, int cls, int dc) {
     extern __shared__ __align__(16) float vcs[];
-    constexpr int NPP = 32 * NG, XL = vb_lane_stride(NG), XS = vb_xstride<NG>(), SLOT = NG * NG;
+    constexpr int NPP = 32 * NG, XL = vb_lane_stride(NG), XS = vb_xstride<NG>();
     constexpr int NQW = NG / WQ;
     constexpr int YN = WQ + NG - 1, YL = (YN + 3) / 4 * 4;   // column increments a thread reads
     static_assert(NG == 2 ? WQ == 2 : WQ % 4 == 0, "vector loads of the column increments");
@@ -305,11 +330,12 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_kernel(VbArgs a, int cls, int d
         const float *cols = (const float *)(p.swapped ? a.src.A : a.src.B) + p.c_row0 * d;
         const int nx = p.lr - 1, ny = p.lc - 1, T = p.T, NQ = T * NG;
         const int YS = vb_ystride(T, NG);
-        const int nthr = 32 * (T + 1) * NQW;
+        const int nthr = vb_units<NQW>(T);
         for (int b0 = 0; b0 < nthr; b0 += VB_CT) {
             const int u = b0 + (int)threadIdx.x;
-            const int l = u & 31, pq = u >> 5;
-            const int pos = pq / NQW, w0 = (pq - pos * NQW) * WQ;
+            const VbUnit un = vb_unit<NQW>(u);
+            const bool live = u < nthr && un.pos <= T;
+            const int l = un.l, pos = live ? un.pos : 0, w0 = un.part * WQ;
             float acc[WQ][NG];
 #pragma unroll
             for (int w = 0; w < WQ; ++w)
@@ -364,23 +390,19 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_kernel(VbArgs a, int cls, int d
                     }
                 }
             }
-            if (u >= nthr) continue;
-            float *dst = a.band + p.base + ((int64_t)pos * 32 + l) * SLOT;   // pos = T: the next slot 0
+            if (!live) continue;
+            float *dst = a.band + p.base + band_row(p.s0 + pos, l, NG, p.slots);   // pos = T: the next slot 0
             if (pos > 0 && pos < T) {
+                float o[WQ * NG];
 #pragma unroll
-                for (int w = 0; w < WQ; ++w) {
-                    float o[NG];
+                for (int w = 0; w < WQ; ++w)
 #pragma unroll
-                    for (int g = 0; g < NG; ++g) o[vb_gpos<NG>(g)] = scheme_coef(acc[w][g] * a.scale, a.src.scheme);
-                    if constexpr (NG % 4 == 0) {
+                    for (int g = 0; g < NG; ++g)
+                        o[w * NG + vb_gpos<NG>(g)] = scheme_coef(acc[w][g] * a.scale, a.src.scheme);
 #pragma unroll
-                        for (int h = 0; h < NG / 4; ++h)
-                            reinterpret_cast<float4 *>(dst + (w0 + w) * NG)[h] =
-                                make_float4(o[4 * h], o[4 * h + 1], o[4 * h + 2], o[4 * h + 3]);
-                    } else {
-                        reinterpret_cast<float2 *>(dst + (w0 + w) * NG)[0] = make_float2(o[0], o[1]);
-                    }
-                }
+                for (int h = 0; h < WQ * NG; h += 4)
+                    *reinterpret_cast<float4 *>(dst + band_off(w0 * NG + h)) =
+                        make_float4(o[h], o[h + 1], o[h + 2], o[h + 3]);
                 continue;
             }
 #pragma unroll
@@ -389,7 +411,7 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_kernel(VbArgs a, int cls, int d
                 for (int g = 0; g < NG; ++g) {
                     const int ww = w0 + w;
                     const float v = scheme_coef(acc[w][g] * a.scale, a.src.scheme);
-                    float *o = dst + ww * NG + vb_gpos<NG>(g);
+                    float *o = dst + band_off(ww * NG + vb_gpos<NG>(g));
                     if (pos == 0) {
                         // the pair's own cells; the previous pair of the chain
                         // writes the cells w < g of this slot (its tail)
@@ -408,6 +430,7 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_kernel(VbArgs a, int cls, int d
 }
 
 // ---- the sweep ----------------------------------------------------------------
+// A lane's coefficients of one window: 16-byte pieces of a band row, 32 lanes side by side.
 template <int NG>
 __device__ __forceinline__ void vb_fetch(float *dst, const float *src) {
     constexpr int BYTES = NG * 4;
@@ -415,7 +438,7 @@ __device__ __forceinline__ void vb_fetch(float *dst, const float *src) {
     if constexpr (BYTES >= 16) {
 #pragma unroll
         for (int o = 0; o < BYTES; o += 16)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s + o), "l"((const char *)src + o)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s + o), "l"(src + band_off(o / 4))
                          : "memory");
     } else {
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(src), "n"(BYTES) : "memory");
@@ -427,10 +450,9 @@ __device__ __forceinline__ void vb_wait() { asm volatile("cp.async.wait_group %0
 
 // A lane's position in its chain: pair j (j = np: past the last pair), macro-
 // step pos of it (negative before the lane enters the chain), the pair's
-// macro-step count and the float offset of its slot 0.
+// macro-step count.
 struct VbCursor {
     int j, pos, T, nextT;
-    int64_t cur;
 };
 
 template <int R, int LAM, int MINB>
@@ -441,7 +463,7 @@ __global__ void __launch_bounds__(VB_WARPS * 32, MINB) vband_sweep_kernel(VbArgs
     constexpr int NH = NG / 2;
     constexpr int JOUT = R - 2;
     constexpr int SLOT = NG * NG;
-    constexpr int64_t PSTR = 32LL * SLOT;   // floats per slot (all lanes)
+    constexpr int64_t PSTR = 32LL * SLOT;   // floats per row (all lanes)
     static_assert(R % S == 0 && NG % 2 == 0 && NG <= 16, "2 to 16 coarse rows per lane, even");
     extern __shared__ __align__(16) float vring[];
 
@@ -465,29 +487,28 @@ __global__ void __launch_bounds__(VB_WARPS * 32, MINB) vband_sweep_kernel(VbArgs
     for (int o = 16; o > 0; o >>= 1) tsum += __shfl_xor_sync(FULL, tsum, o);
     const int total_m = tsum + 32;
 
-    // consumer (the sweep) and fetcher (VB_RING - 1 windows ahead) cursors
-    VbCursor cc, fc;
+    // consumer (the sweep) cursor
+    VbCursor cc;
     cc.j = 0;
     cc.pos = -lane;
     cc.T = cT[0];
     cc.nextT = np > 1 ? cT[1] : 1;
-    cc.cur = a.chain_base[gc];
-    fc = cc;
-    int fw = 0;   // window of the fetcher within its macro-step
     auto advance = [&](VbCursor &q) {
         if (++q.pos == q.T && q.j < np) {
             q.pos = 0;
-            q.cur += (int64_t)q.T * PSTR;
             ++q.j;
             q.T = q.nextT;
             q.nextT = q.j + 1 < np ? cT[q.j + 1] : 1;
         }
     };
+    // fetcher (VB_RING - 1 windows ahead): lane l takes its slot fs in row fs + l,
+    // every lane's the same, counted modulo the chain's slots
+    const float *const cband = a.band + a.chain_base[gc] + 4 * lane, *frow = cband;
+    int fs = -lane, fr = 0, fw = 0;   // slot, row, window within the macro-step
     auto fetch = [&](int e) {
         float *dst = ring + e * 32 * LS;
-        const bool live = fc.pos >= 0 && (fc.j < np || (fc.j == np && fc.pos == 0));
-        if (live) {
-            vb_fetch<NG>(dst, a.band + fc.cur + ((int64_t)fc.pos * 32 + lane) * SLOT + fw * NG);
+        if (fs >= 0 && fs <= tsum) {
+            vb_fetch<NG>(dst, frow + band_off(fw * NG));
         } else {
 #pragma unroll
             for (int g = 0; g < NG; g += 2) *reinterpret_cast<float2 *>(dst + g) = make_float2(0.f, 0.f);
@@ -495,7 +516,12 @@ __global__ void __launch_bounds__(VB_WARPS * 32, MINB) vband_sweep_kernel(VbArgs
         vb_commit();
         if (++fw == NG) {
             fw = 0;
-            advance(fc);
+            ++fs;
+            frow += PSTR;
+            if (++fr > tsum) {
+                fr = 0;
+                frow = cband;
+            }
         }
     };
 #pragma unroll
@@ -612,7 +638,7 @@ cudaError_t vb_launch_sweep(const VbArgs &a, int cls, int grid, cudaStream_t st)
 template <int NG, int WQ, int HB>
 __global__ void __launch_bounds__(VB_CT) vb_coef_pair_kernel(VbArgs a, int cls, int dc) {
     extern __shared__ __align__(16) float vcs[];
-    constexpr int NPP = 32 * NG, XL = vb_lane_stride(NG), XS = vb_xstride<NG>(), SLOT = NG * NG;
+    constexpr int NPP = 32 * NG, XL = vb_lane_stride(NG), XS = vb_xstride<NG>();
     constexpr int NH = NG / 2, NHB = NH / HB, NQW = NG / WQ;
     constexpr int YN = WQ + NH + HB - 1, YL = (YN + 3) / 4 * 4;
     static_assert(NH % HB == 0 && HB % 4 == 0 && WQ % 4 == 0 && (NH - HB) % 4 == 0, "aligned vector loads");
@@ -627,12 +653,12 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_pair_kernel(VbArgs a, int cls, 
         const float *cols = (const float *)(p.swapped ? a.src.A : a.src.B) + p.c_row0 * d;
         const int nx = p.lr - 1, ny = p.lc - 1, T = p.T, NQ = T * NG;
         const int YS = vb_ystride(T, NG);
-        const int nthr = 32 * (T + 1) * NQW * NHB;
+        const int nthr = vb_units<NQW * NHB>(T);
         for (int b0 = 0; b0 < nthr; b0 += VB_CT) {
             const int u = b0 + (int)threadIdx.x;
-            const int l = u & 31, pq = u >> 5;
-            const int hb = pq % NHB, pq2 = pq / NHB;
-            const int pos = pq2 / NQW, w0 = (pq2 - pos * NQW) * WQ, h0 = hb * HB;
+            const VbUnit un = vb_unit<NQW * NHB>(u);
+            const bool live = u < nthr && un.pos <= T;
+            const int l = un.l, pos = live ? un.pos : 0, w0 = un.part / NHB * WQ, h0 = un.part % NHB * HB;
             float acc[WQ][2 * HB];   // [w][2k]: group h0 + k, [w][2k + 1]: group h0 + k + NH
 #pragma unroll
             for (int w = 0; w < WQ; ++w)
@@ -681,18 +707,18 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_pair_kernel(VbArgs a, int cls, 
                     }
                 }
             }
-            if (u >= nthr) continue;
+            if (!live) continue;
 #pragma unroll
             for (int w = 0; w < WQ; ++w)
 #pragma unroll
                 for (int k = 0; k < 2 * HB; ++k) acc[w][k] = scheme_coef(acc[w][k] * a.scale, a.src.scheme);
-            float *dst = a.band + p.base + ((int64_t)pos * 32 + l) * SLOT;   // pos = T: the next slot 0
+            float *dst = a.band + p.base + band_row(p.s0 + pos, l, NG, p.slots);   // pos = T: the next slot 0
             if (pos > 0 && pos < T) {
 #pragma unroll
                 for (int w = 0; w < WQ; ++w)
 #pragma unroll
                     for (int k = 0; k < 2 * HB; k += 4)
-                        *reinterpret_cast<float4 *>(dst + (w0 + w) * NG + 2 * h0 + k) =
+                        *reinterpret_cast<float4 *>(dst + band_off((w0 + w) * NG + 2 * h0 + k)) =
                             make_float4(acc[w][k], acc[w][k + 1], acc[w][k + 2], acc[w][k + 3]);
                 continue;
             }
@@ -702,7 +728,7 @@ __global__ void __launch_bounds__(VB_CT) vb_coef_pair_kernel(VbArgs a, int cls, 
                 for (int k = 0; k < 2 * HB; ++k) {
                     const int g = (k & 1) ? h0 + (k >> 1) + NH : h0 + (k >> 1);
                     const int ww = w0 + w;
-                    float *o = dst + ww * NG + 2 * h0 + k;   // vb_gpos(g)
+                    float *o = dst + band_off(ww * NG + 2 * h0 + k);   // vb_gpos(g)
                     if (pos == 0) {
                         if (ww >= g) *o = acc[w][k];
                         else if (p.first) *o = 0.f;
