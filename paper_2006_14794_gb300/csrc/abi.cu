@@ -369,13 +369,15 @@ int run_backward(PairSrc src, int64_t n_pairs, int lam, int dtype, const sigk_op
     // every path below adds into zeroed outputs (atomics), except the band
     // form, whose last kernel writes each output once (and adds on request)
     const bool acc = accumulate_of(opts);
-    if (!acc && dX && cudaMemsetAsync(dX, 0, (size_t)(nX * es), st) != cudaSuccess) return SIGK_ECUDA;
-    if (!acc && dY && cudaMemsetAsync(dY, 0, (size_t)(nY * es), st) != cudaSuccess) return SIGK_ECUDA;
-    if (n_pairs == 0 || src.La < 2 || src.Lb < 2 || (!dX && !dY)) return SIGK_OK;
     const int rec = rec_of(opts);
-    if (rec == SIGK_REC_STRIP && !strip_supported(lam, src.d, dtype)) return SIGK_EUNSUPPORTED;
+    const bool none = n_pairs == 0 || src.La < 2 || src.Lb < 2;
     BandPlan bp;
-    if (bwd_uses_band(src, lam, dtype, rec, rows_of(opts), bp)) {
+    const bool band = !none && bwd_uses_band(src, lam, dtype, rec, rows_of(opts), bp);
+    if (!acc && !band && dX && cudaMemsetAsync(dX, 0, (size_t)(nX * es), st) != cudaSuccess) return SIGK_ECUDA;
+    if (!acc && !band && dY && cudaMemsetAsync(dY, 0, (size_t)(nY * es), st) != cudaSuccess) return SIGK_ECUDA;
+    if (none || (!dX && !dY)) return SIGK_OK;
+    if (rec == SIGK_REC_STRIP && !strip_supported(lam, src.d, dtype)) return SIGK_EUNSUPPORTED;
+    if (band) {
         bool sw;
         const PairSrc o = band_orient(src, n_pairs, sw);
         int64_t bytes;

@@ -948,15 +948,26 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
     cp_wait<0>();
 }
 
-// Real (unpadded) increments of paths: inc[(path * (L - 1) + p) * d + c].
-__global__ void band_inc_kernel(const float *pts, int64_t npaths, int64_t L, int64_t d, float *inc) {
-    const int64_t total = npaths * (L - 1) * d;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < total;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = v % d, row = v / d;
-        const int64_t path = row / (L - 1), p = row - path * (L - 1);
-        const float *x = pts + (path * L + p) * d + c;
-        inc[v] = x[d] - x[0];
+// Real (unpadded) increments of paths: inc[(path * (L - 1) + p) * d + c], of the
+// row role's and the column role's paths in one launch (a small gradient step
+// is bound by its launches), which also clears the status word of the
+// workspace (null: left alone).
+struct IncJob {
+    const float *pts;
+    int64_t npaths, L;
+    float *inc;
+};
+__global__ void band_inc_kernel(IncJob ja, IncJob jb, int64_t d, int *status) {
+    if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+    const int64_t na = ja.npaths * (ja.L - 1) * d, total = na + jb.npaths * (jb.L - 1) * d;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const bool isb = u >= na;
+        const IncJob &j = isb ? jb : ja;
+        const int64_t v = isb ? u - na : u, c = v % d, row = v / d;
+        const int64_t path = row / (j.L - 1), p = row - path * (j.L - 1);
+        const float *x = j.pts + (path * j.L + p) * d + c;
+        j.inc[v] = x[d] - x[0];
     }
 }
 
@@ -1451,19 +1462,31 @@ __global__ void band_split_sum_kernel(const float *partial, int ksplit, int64_t 
 
 // Point gradients from increment gradients: x_p enters dx_{p-1} (+) and dx_p
 // (-), so dX[path][p] = scale (dinc[p-1] - dinc[p]) (terms outside 0..L-2
-// absent).  Overwrites dpts, or adds to it (add).
-__global__ void band_points_kernel(const float *dinc, int64_t npaths, int64_t L, int64_t d, float scale,
-                                   int add, float *dpts) {
-    const int64_t total = npaths * L * d;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < total;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = v % d, row = v / d;
-        const int64_t path = row / L, p = row - path * L;
-        const float *di = dinc + path * (L - 1) * d + c;
-        const float lo = p >= 1 ? di[(p - 1) * d] : 0.f;
-        const float hi = p < L - 1 ? di[p * d] : 0.f;
+// absent).  Overwrites dpts, or adds to it (add).  Both roles in one launch;
+// dinc may be the split partials of a contraction, `stride` floats apart, which
+// are then added in band_split_sum_kernel's order (one launch less, the same sums).
+struct PointsJob {
+    const float *dinc;
+    int64_t npaths, L, stride;
+    int ksplit;
+    float *dpts;
+};
+__global__ void band_points_kernel(PointsJob ja, PointsJob jb, int64_t d, float scale, int add) {
+    const int64_t na = ja.npaths * ja.L * d, total = na + jb.npaths * jb.L * d;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const bool isb = u >= na;
+        const PointsJob &j = isb ? jb : ja;
+        const int64_t v = isb ? u - na : u, c = v % d, row = v / d;
+        const int64_t path = row / j.L, p = row - path * j.L;
+        const float *di = j.dinc + path * (j.L - 1) * d + c;
+        float lo = 0.f, hi = 0.f;
+        for (int s = 0; s < j.ksplit; ++s, di += j.stride) {
+            if (p >= 1) lo += di[(p - 1) * d];
+            if (p < j.L - 1) hi += di[p * d];
+        }
         const float g = scale * (lo - hi);
-        dpts[v] = add ? dpts[v] + g : g;
+        j.dpts[v] = add ? j.dpts[v] + g : g;
     }
 }
 
@@ -2037,7 +2060,6 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
     int *status = (int *)ws;
     float *band = w + 64;   // after the 256-byte status header
     float *gbar = w + rg.band;
-    if ((e = cudaMemsetAsync(status, 0, sizeof(int), st)) != cudaSuccess) return e;
     float *ckpt = gbar + rg.gbar;
     float *exitk = ckpt + rg.ckpt;
     float *botq = exitk + rg.exitk;
@@ -2050,18 +2072,23 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
     float *rsum = gband + rg.gband;   // the RBF lift's row sums, then its column sums
     const bool rbf = src0.kernel == SIGK_KERNEL_RBF;
     const int64_t nBall = gram ? src0.nb : 0;
-    if (gram && !rbf) {
-        // every column path is used by every launch: increments once, gradients summed
-        band_inc_kernel<<<sms * 4, 256, 0, st>>>((const float *)src0.B, nBall, src0.Lb, d, incB);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    if (rbf && (e = cudaMemsetAsync(status, 0, sizeof(int), st)) != cudaSuccess) return e;
     for (int64_t kb = 0; kb < n; kb += nbp) {
         const int64_t m = n - kb < nbp ? n - kb : nbp;
         PairSrc src = src0;
         src.kbase = src0.kbase + kb;
         const int64_t a0 = sym ? 0 : gram ? src.kbase / src0.nb : src.kbase;   // first row path
         const int64_t nA = sym ? src0.nb : gram ? m / src0.nb : m;
-        // 1. coefficients
+        // 1. increments of this launch's paths (a Gram's column paths, which every
+        // launch uses, with the first one's; a symmetric one has no others), and coefficients
+        if (!rbf) {
+            const bool b = !sym && (!gram || kb == 0);
+            const IncJob ja = {(const float *)src.A + a0 * src.La * d, nA, src.La, incA};
+            const IncJob jb = {(const float *)src.B + (gram ? 0 : src.kbase * src.Lb * d), !b ? 0 : gram ? nBall : m,
+                               src.Lb, incB};
+            band_inc_kernel<<<sms * 4, 256, 0, st>>>(ja, jb, d, kb == 0 ? status : nullptr);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
         BandCoefArgs c;
         c.src = src;
         c.n_pairs = m;
@@ -2169,13 +2196,7 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             else band_gbar_kernel<2><<<ggrid, GB_THREADS, 0, st>>>(gb);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        // 4. increments of this launch's paths
-        band_inc_kernel<<<sms * 4, 256, 0, st>>>((const float *)src.A + a0 * src.La * d, nA, src.La, d, incA);
-        if (!gram)
-            band_inc_kernel<<<sms * 4, 256, 0, st>>>((const float *)src.B + src.kbase * src.Lb * d, m, src.Lb, d,
-                                                     incB);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        // 5. chain rule: dinc_A = gbar inc_B, dinc_B (+)= gbar^T inc_A
+        // 4. chain rule: dinc_A = gbar inc_B, dinc_B (+)= gbar^T inc_A
         GemmArgs g1;
         memset(&g1, 0, sizeof(g1));
         g1.G = gbar;
@@ -2289,23 +2310,31 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
                 if ((e = launch_chain_gemm_tc5(as_chain(g2, add_b ? 1 : 0), status, st)) != cudaSuccess) return e;
             } else {
                 gemm(gd2, g2);
-                if (g2.ksplit > 1)
-                    band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g2.ksplit, g2.M * d, add_b ? 1 : 0,
-                                                                   g2.C);
+                if (g2.ksplit > 1 && add_b)
+                    band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g2.ksplit, g2.M * d, 1, g2.C);
+                else if (g2.ksplit > 1 && kb + m < n)   // the last launch's are summed by the point gradients
+                    band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g2.ksplit, g2.M * d, 0, g2.C);
             }
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        // 6. point gradients
-        if (dA)
-            band_points_kernel<<<sms * 4, 256, 0, st>>>(dincA, nA, src.La, d, scale, add, dA + a0 * src.La * d);
-        if (dB && !gram)
-            band_points_kernel<<<sms * 4, 256, 0, st>>>(dincB, m, src.Lb, d, scale, add,
-                                                      dB + src.kbase * src.Lb * d);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (dB && gram && !rbf) {
-        band_points_kernel<<<sms * 4, 256, 0, st>>>(dincB, nBall, src0.Lb, d, scale, add, dB);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // 5. point gradients (a Gram's column paths' with the last launch's)
+        PointsJob ja = {dincA, dA ? nA : 0, src.La, 0, 1, dA ? dA + a0 * src.La * d : nullptr};
+        PointsJob jb = {dincB, 0, src.Lb, 0, 1, dB};
+        if (dB && !gram) {
+            jb.npaths = m;
+            jb.dpts = dB + src.kbase * src.Lb * d;
+        } else if (dB && kb + m >= n) {
+            jb.npaths = nBall;
+            if (!tc && !add_b && g2.ksplit > 1) {
+                jb.dinc = part;
+                jb.ksplit = g2.ksplit;
+                jb.stride = g2.M * d;
+            }
+        }
+        if (ja.npaths || jb.npaths) {
+            band_points_kernel<<<sms * 4, 256, 0, st>>>(ja, jb, d, scale, add);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
