@@ -1164,8 +1164,7 @@ __global__ void __launch_bounds__(256) band_gemm_kernel(GemmArgs a) {
 // share of the reduction in the same order as band_gemm_kernel, bit for bit (a
 // Gram's gradients are sums of 10^4 terms that cancel: another order moves them by
 // 1e-5).  128 x 128 Gram of 256-point paths, N = 32: 2.98 ms a launch through
-// turned tiles (which still take the transposed contraction and two rows a
-// lane), 2.3 here.
+// turned tiles (which still take two rows a lane), 2.3 here.
 template <int NG>
 struct GrStage {
     static constexpr int LANES = 128 / NG, THREADS = 8 * LANES;
@@ -1323,6 +1322,149 @@ __global__ void __launch_bounds__(GrStage<NG>::THREADS, 512 / GrStage<NG>::THREA
             const float v = g < NH ? acc[g % NH][c].x : acc[g % NH][c].y;
             if (a.ksplit > 1) a.partial[((int64_t)ks * a.M + r) * a.N + n] = v;
             else C[r * a.N + n] = v;
+        }
+    }
+}
+
+// The transposed contraction (the column role's increments as output) for lanes
+// of 4 or 8 coarse rows, again from the slots as they lie.  A thread owns the NG
+// columns of a position and four channels; the cell (row g, column q) is window
+// q + g of the position's slot or, past its end, window q + g - NG of the next
+// one.  A stage is 32 rows (32 / NG lanes) of one row path, double-buffered by
+// cp.async: per lane a thread reads the halves of both slots that it needs (26
+// 16-byte loads for NG = 8) and 8 row quads for 256 FMAs, so that the FMAs bound
+// it and not the shared memory, where the turned tiles above took three barriers
+// and two loads for 16 FMAs.  The upper groups of a window's pairs are kept until
+// the lower ones are added: every output takes the rows in band_gemm_kernel's
+// order, and the gradients stay bit for bit what they were.
+// 8256 pairs (symmetric) of 256-point paths, N = 32: 2.02 -> 1.25 ms a launch.
+template <int NG>
+struct GcStage {
+    static constexpr int LANES = 32 / NG, POS = 128 / NG, THREADS = 8 * POS;
+    static constexpr int SLOT = NG * NG, SS = SLOT + 4;   // padded: a warp's 4 positions, 4 bank quads
+    float g[LANES][POS + 1][SS];
+    float x[32][32];
+};
+
+template <int NG>
+__global__ void __launch_bounds__(GcStage<NG>::THREADS, 512 / GcStage<NG>::THREADS) band_cols_kernel(GemmArgs a) {
+    using St = GcStage<NG>;
+    constexpr int NH = NG / 2, POS = St::POS, LANES = St::LANES, SLOT = St::SLOT, NT = St::THREADS;
+    constexpr int XV = 1024 / NT;                     // row values a thread stages
+    constexpr int SV = SLOT / 4, NV = (POS + 1) * LANES * SV;
+    extern __shared__ __align__(16) float gr_sm[];
+    St *st = reinterpret_cast<St *>(gr_sm);           // two of them
+    const int tid = threadIdx.x, tp = tid >> 3, cq = tid & 7;
+    const int64_t b = blockIdx.z / a.ksplit;
+    const int ks = blockIdx.z - (int)b * a.ksplit;
+    const float *Bm = a.Bm + b * a.b_bstride;
+    float *C = a.C + b * a.c_bstride;
+    const int TperR = a.TperR1 - 1, tpp = (TperR + POS - 1) / POS;
+    const int64_t opath = blockIdx.x / tpp;
+    const int p0 = (int)(blockIdx.x - opath * tpp) * POS;
+    const int n0 = blockIdx.y * 32;
+    // the share in slices of 32 rows (NG slices a row path)
+    const int64_t rhi = a.mode == PM_GRAM_SYM ? opath + 1 : a.nA;
+    const int64_t total = rhi * NG;
+    const int64_t s_lo = total * ks / a.ksplit, s_hi = total * (ks + 1) / a.ksplit;
+
+    float xr[XV];
+    // slice s: its slots into buffer buf (cp.async), its rows' increments into registers
+    auto fetch = [&](int64_t s, int buf) {
+        const int64_t rp = s / NG;
+        const int c0 = (int)(s - rp * NG) * 32;
+        const int64_t k = gemm_pair(a, b, rp, opath);
+        const float *src = a.band + ((k * a.TperR1 + p0) * 32 + c0 / NG) * (int64_t)SLOT;
+        for (int v = tid; v < NV; v += NT) {
+            const int sl = v / SV, e = v - sl * SV, pr = sl / LANES, lr = sl % LANES;
+            if (p0 + pr <= TperR) cp_async<16>(&st[buf].g[lr][pr][4 * e], src + (pr * 32 + lr) * SLOT + 4 * e);
+        }
+        cp_commit();
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {
+            const int v = tid + NT * i, real = c0 + (v >> 5) - a.vrows, n = n0 + (v & 31);
+            xr[i] = real >= 0 && real < a.nx && n < a.N ? __ldg(Bm + (rp * a.nx + real) * a.N + n) : 0.f;
+        }
+    };
+    float acc[NG][4];
+#pragma unroll
+    for (int q = 0; q < NG; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[q][c] = 0.f;
+
+    if (s_lo < s_hi) fetch(s_lo, 0);
+    int buf = 0;
+    for (int64_t s = s_lo; s < s_hi; ++s, buf ^= 1) {
+        St &S = st[buf];
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {
+            const int v = tid + NT * i;
+            S.x[v >> 5][v & 31] = xr[i];
+        }
+        cp_wait<0>();
+        __syncthreads();   // the stage is complete, and the other buffer's readers are done
+        if (s + 1 < s_hi) fetch(s + 1, buf ^ 1);
+        const int c0 = (int)(s % NG) * 32;
+        if (p0 + tp >= TperR) continue;
+        // one lane; MASK: its first `virt` rows are virtual and count as zero whatever the slots hold
+        auto lane = [&](int lr, int virt, auto mask_tag) {
+            constexpr bool MASK = decltype(mask_tag)::value;
+            const float *own = S.g[lr][tp], *nxt = S.g[lr][tp + 1];
+            auto row = [&](int g) { return *reinterpret_cast<const float4 *>(&S.x[lr * NG + g][4 * cq]); };
+            auto add = [&](int q, float v, int g, const float4 &x) {
+                if (MASK && g < virt) v = 0.f;
+                acc[q][0] = fmaf(v, x.x, acc[q][0]);
+                acc[q][1] = fmaf(v, x.y, acc[q][1]);
+                acc[q][2] = fmaf(v, x.z, acc[q][2]);
+                acc[q][3] = fmaf(v, x.w, acc[q][3]);
+            };
+            float hi[NH][NG];   // rows NH + h, until rows 0 .. NH - 1 are added
+#pragma unroll
+            for (int h = 0; h < NH; h += 2) {
+                const float4 xa = row(h), xb = row(h + 1);
+#pragma unroll
+                for (int w = h; w < NG; ++w) {   // the position's own slot: q = w - g >= 0
+                    const float4 v = *reinterpret_cast<const float4 *>(own + w * NG + 2 * h);
+                    add(w - h, v.x, h, xa);
+                    if (w >= h + 1) add(w - h - 1, v.z, h + 1, xb);
+                    if (w >= h + NH) hi[h][w - h - NH] = v.y;
+                    if (w >= h + 1 + NH) hi[h + 1][w - h - 1 - NH] = v.w;
+                }
+#pragma unroll
+                for (int w = 0; w < h + 1 + NH; ++w) {   // the next one: q = w - g + NG < NG
+                    const float4 v = *reinterpret_cast<const float4 *>(nxt + w * NG + 2 * h);
+                    if (w < h) add(w - h + NG, v.x, h, xa);
+                    if (w < h + 1) add(w - h - 1 + NG, v.z, h + 1, xb);
+                    if (w < h + NH) hi[h][w - h - NH + NG] = v.y;
+                    hi[h + 1][w - h - 1 - NH + NG] = v.w;
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const float4 x = row(h + NH);
+#pragma unroll
+                for (int q = 0; q < NG; ++q) add(q, hi[h][q], h + NH, x);
+            }
+        };
+#pragma unroll 1
+        for (int lr = 0; lr < LANES; ++lr) {
+            const int virt = a.vrows - (c0 + lr * NG);
+            if (virt <= 0) lane(lr, 0, std::false_type{});
+            else if (virt < NG) lane(lr, virt, std::true_type{});
+        }
+    }
+    if (p0 + tp >= TperR) return;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+        const int real = (p0 + tp) * NG + q - a.NQV;
+        if (real < 0 || real >= a.ny) continue;
+        const int64_t r = opath * a.ny + real;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int n = n0 + 4 * cq + c;
+            if (n >= a.N) continue;
+            if (a.ksplit > 1) a.partial[((int64_t)ks * a.M + r) * a.N + n] = acc[q][c];
+            else C[r * a.N + n] = acc[q][c];
         }
     }
 }
@@ -2243,8 +2385,6 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             if (ksp > GEMM_MAX_SPLIT) ksp = GEMM_MAX_SPLIT;
             return (int)(ksp < 1 ? 1 : ksp);
         };
-        // the row role's contraction as the slots lie, for 4 and 8 rows a lane
-        const bool by_rows = p.NG >= 4;
         g1.ksplit = split(tiles1, nBall * ((NQc + GT_K - 1) / GT_K));
         g2.ksplit = split(tiles2, nA * (BHr / GT_K));
         g1.partial = g2.partial = part;
@@ -2265,10 +2405,14 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
         g1.NQV = g2.NQV = p.NQV;
         g1.nx = g2.nx = (int)nx;
         g1.ny = g2.ny = (int)ny;
-        auto gemm = [&](const dim3 &gd, const GemmArgs &ga) {
-            if (p.NG == 8) band_gemm_kernel<8><<<gd, 256, 0, st>>>(ga);
-            else if (p.NG == 4) band_gemm_kernel<4><<<gd, 256, 0, st>>>(ga);
-            else band_gemm_kernel<2><<<gd, 256, 0, st>>>(ga);
+        // as the slots lie for 4 and 8 rows a lane, through turned tiles for 2
+        auto go = [&](auto kern, int threads, size_t smem, const dim3 &gd, const GemmArgs &ga) {
+            if (smem > 0) {
+                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (r != cudaSuccess) return r;
+            }
+            kern<<<gd, threads, smem, st>>>(ga);
+            return cudaGetLastError();
         };
         auto as_chain = [&](const GemmArgs &ga, int add) {
             ChainGemm cg;
@@ -2289,18 +2433,10 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             if (tc) {
                 if ((e = launch_chain_gemm_tc5(as_chain(g1, 0), status, st)) != cudaSuccess) return e;
             } else {
-                if (by_rows) {
-                    auto go = [&](auto kern, int threads, int smem) {
-                        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                        if (r == cudaSuccess) kern<<<gd1, threads, smem, st>>>(g1);
-                        return r;
-                    };
-                    if (p.NG == 8) e = go(band_rows_kernel<8>, GrStage<8>::THREADS, 2 * (int)sizeof(GrStage<8>));
-                    else e = go(band_rows_kernel<4>, GrStage<4>::THREADS, 2 * (int)sizeof(GrStage<4>));
-                    if (e != cudaSuccess) return e;
-                } else {
-                    gemm(gd1, g1);
-                }
+                if (p.NG == 8) e = go(band_rows_kernel<8>, GrStage<8>::THREADS, 2 * sizeof(GrStage<8>), gd1, g1);
+                else if (p.NG == 4) e = go(band_rows_kernel<4>, GrStage<4>::THREADS, 2 * sizeof(GrStage<4>), gd1, g1);
+                else e = go(band_gemm_kernel<2>, 256, 0, gd1, g1);
+                if (e != cudaSuccess) return e;
                 if (g1.ksplit > 1)
                     band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g1.ksplit, g1.M * d, 0, dincA);
             }
@@ -2309,7 +2445,10 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
             if (tc) {
                 if ((e = launch_chain_gemm_tc5(as_chain(g2, add_b ? 1 : 0), status, st)) != cudaSuccess) return e;
             } else {
-                gemm(gd2, g2);
+                if (p.NG == 8) e = go(band_cols_kernel<8>, GcStage<8>::THREADS, 2 * sizeof(GcStage<8>), gd2, g2);
+                else if (p.NG == 4) e = go(band_cols_kernel<4>, GcStage<4>::THREADS, 2 * sizeof(GcStage<4>), gd2, g2);
+                else e = go(band_gemm_kernel<2>, 256, 0, gd2, g2);
+                if (e != cudaSuccess) return e;
                 if (g2.ksplit > 1 && add_b)
                     band_split_sum_kernel<<<sms * 4, 256, 0, st>>>(part, g2.ksplit, g2.M * d, 1, g2.C);
                 else if (g2.ksplit > 1 && kb + m < n)   // the last launch's are summed by the point gradients
