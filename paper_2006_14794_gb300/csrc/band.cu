@@ -1360,8 +1360,10 @@ __global__ void __launch_bounds__(GcStage<NG>::THREADS, 512 / GcStage<NG>::THREA
     const float *Bm = a.Bm + b * a.b_bstride;
     float *C = a.C + b * a.c_bstride;
     const int TperR = a.TperR1 - 1, tpp = (TperR + POS - 1) / POS;
-    const int64_t opath = blockIdx.x / tpp;
-    const int p0 = (int)(blockIdx.x - opath * tpp) * POS;
+    // a symmetric Gram's column path j meets j + 1 row paths: the longest first, so
+    // that the short ones fill the last wave (1.25 -> 1.11 ms for 128 of them)
+    const int64_t blk = blockIdx.x / tpp, opath = a.mode == PM_GRAM_SYM ? a.nB - 1 - blk : blk;
+    const int p0 = (int)(blockIdx.x - blk * tpp) * POS;
     const int n0 = blockIdx.y * 32;
     // the share in slices of 32 rows (NG slices a row path)
     const int64_t rhi = a.mode == PM_GRAM_SYM ? opath + 1 : a.nA;
