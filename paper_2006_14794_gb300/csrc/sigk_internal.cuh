@@ -99,13 +99,17 @@ struct PairRef {
 
 // Upper-triangle enumeration (i <= j) of an n x n symmetric Gram matrix.  The
 // row is estimated from the inverse of its offset and corrected to the exact
-// one: in FP32 for n <= 4096 (there the estimate is off by a few rows at most;
-// an FP64 instruction takes a warp 64 cycles here, and every pair of the FP32
-// sweeps asks for its row), in FP64 beyond.
+// one: in FP32 for n <= 4096 (EST32; there the estimate is off by a few rows at
+// most; an FP64 instruction takes a warp 64 cycles here, and every pair of the
+// FP32 band sweeps asks for its row), else in FP64.  chain_f32_kernel keeps the
+// FP64 estimate: the other one moved its code so that an implicit Gram of 17 x
+// 138 paths of 56 and 118 points, order 2, took 104 us instead of 91, for 1 %
+// on symmetric Grams.
+template <bool EST32>
 __host__ __device__ inline void sym_index(int64_t k, int64_t n, int64_t &i, int64_t &j) {
     // row i holds n - i entries, starting at off(i) = i*n - i*(i-1)/2
     int64_t ii;
-    if (n <= 4096) {
+    if (EST32 && n <= 4096) {
         const int m = 2 * (int)n + 1, disc = m * m - 8 * (int)k;   // below 2^27
         ii = (int64_t)(((float)m - sqrtf(disc > 0 ? (float)disc : 0.f)) * 0.5f);
     } else {
@@ -120,6 +124,7 @@ __host__ __device__ inline void sym_index(int64_t k, int64_t n, int64_t &i, int6
     j = ii + (k - (ii * n - ii * (ii - 1) / 2));
 }
 
+template <bool EST32 = true>
 __host__ __device__ inline PairRef pair_ref(const PairSrc &s, int64_t k) {
     PairRef r;
     k += s.kbase;
@@ -135,7 +140,7 @@ __host__ __device__ inline PairRef pair_ref(const PairSrc &s, int64_t k) {
         r.out0 = i * s.out_si + j * s.out_sj;
     } else if (s.mode == PM_GRAM_SYM) {
         int64_t i, j;
-        sym_index(k, s.nb, i, j);
+        sym_index<EST32>(k, s.nb, i, j);
         r.a_row0 = i * s.La; r.la = s.La;
         r.b_row0 = j * s.Lb; r.lb = s.Lb;
         r.out0 = i * s.nb + j;
