@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, MINB) chain_band_kernel(BandA
                         if (j == JOUT && trans && lane == 31) {
                             const int kp = kl - 1;   // row R-1 just finished pair kp's last column
                             if (kp >= 0 && kp < np && a.out) {
-                                const PairRef pr = pair_ref(a.src, k0 + kp);
+                                const PairRef pr = pair_ref<true>(a.src, k0 + kp);
                                 a.out[pr.out0] = KP[i].y;
                                 if (pr.out1 >= 0) a.out[pr.out1] = KP[i].y;
                             }
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(BT5_T, 1) band_coef_tc5_kernel(BandCoefArgs a,
     const int64_t kbeg = (int64_t)blockIdx.x * per;
     const int64_t kend = kbeg + per < a.n_pairs ? kbeg + per : a.n_pairs;
     for (int64_t k = kbeg; k < kend && !failed; ++k) {
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         const float *x = (const float *)a.src.A + pr.a_row0 * d;
         const float *y = (const float *)a.src.B + pr.b_row0 * d;
         const int nx = (int)pr.la - 1, ny = (int)pr.lb - 1;
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(GB_THREADS) band_gbar_kernel(BandGbarArgs a) {
             sr = a.s_a;
             sc = a.s_b;
         } else {
-            const PairRef pr = pair_ref(a.src, k);
+            const PairRef pr = pair_ref<true>(a.src, k);
             const int64_t ia = pr.a_row0 / a.src.La - a.a_first;
             const int64_t jb = a.gram ? pr.b_row0 / a.src.Lb : 0;
             base = a.gbar + ia * a.nx * a.g_ld + jb * a.ny;
@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(BAND_WARPS * 32, 6) chain_band_adj_kernel(Band
             }
             if (lane == 31) {
                 // a symmetric Gram's pair (i, j), i < j, stands for (j, i) too
-                const PairRef pr = pair_ref(a.src, k0 + kl - 1);
+                const PairRef pr = pair_ref<true>(a.src, k0 + kl - 1);
                 gseed = a.gout[pr.out0] + (pr.out1 >= 0 ? a.gout[pr.out1] : 0.f);
             }
         }
@@ -1698,7 +1698,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) rbf_wt_kernel(RbfWtArgs a) {
         const int64_t k = u / per;
         const int t = (int)(u - k * per);
         const int i0 = (t / a.tiles_j) * RW_TI, j0 = (t % a.tiles_j) * RW_TJ;
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         const int nx = (int)pr.la - 1, ny = (int)pr.lb - 1;   // coarse rows / columns; nx + 1 points
         if (i0 > nx || j0 > ny) continue;   // block-uniform
         const float *xp = (const float *)a.src.A + pr.a_row0 * d;

@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
 
     int64_t kn = ubeg / a.tiles;          // the next step's pair and tile
     int tn = (int)(ubeg - kn * a.tiles);
-    PairRef pr = pair_ref(a.src, kn);
+    PairRef pr = pair_ref<true>(a.src, kn);
     int64_t staged = -1;   // the row path whose values xi (and xp) hold
     fetch_y(pr.b_row0, tn, 0, nch);
     float2 acc[NP][NG][NH];
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
         const bool more = u + 1 < uend;
         if (more && ++tn == a.tiles) {
             tn = 0;
-            pr = pair_ref(a.src, ++kn);
+            pr = pair_ref<true>(a.src, ++kn);
         }
         for (int ch = 0; ch < chunks; ++ch) {
             const int64_t c0 = (int64_t)ch * KC_CH;

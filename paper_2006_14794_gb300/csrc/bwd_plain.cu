@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(BWD_THREADS) bwd_plain_kernel(BwdArgs a) {
     const int64_t d = a.src.d;
     unsigned char *slot = a.ws + (int64_t)blockIdx.x * a.slot_bytes;
     for (int64_t k = blockIdx.x; k < a.n_pairs; k += gridDim.x) {
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         const T gk = ((const T *)a.gout)[pr.out0];
         if (pr.la < 2 || pr.lb < 2) continue;   // k = 1 identically: zero gradient
         // rows index the shorter path; its gradient goes to the matching output

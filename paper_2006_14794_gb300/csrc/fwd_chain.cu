@@ -78,7 +78,7 @@ __device__ __forceinline__ int swz(int u) { return u ^ ((u >> 3) & 7); }
 template <int NG, int D4>
 __device__ void load_pair(float4 *ybuf, float4 *xbuf, long long *outs, const ChainArgs &a,
                           int64_t kg, int lane, int vrows) {
-    const PairRef pr = pair_ref<false>(a.src, kg);
+    const PairRef pr = pair_ref(a.src, kg);
     const int d = (int)a.src.d;
     const float *y = (const float *)a.src.B + pr.b_row0 * (int64_t)d;
     const float *x = (const float *)a.src.A + pr.a_row0 * (int64_t)d;

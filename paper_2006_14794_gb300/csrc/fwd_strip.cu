@@ -96,7 +96,7 @@ __global__ void plan_kernel(PairSrc src, int64_t n, PairPlan *plan, int64_t *tot
     __shared__ int64_t part[5][512];
     // pass 1: per-pair shape
     for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
-        const PairRef pr = pair_ref(src, k);
+        const PairRef pr = pair_ref<true>(src, k);
         PairPlan p;
         // rows refine the longer path (more strips, more warps per pair) or,
         // with many pairs in flight, the shorter one (fewer virtual rows and
@@ -1784,7 +1784,7 @@ template <typename T>
 __global__ void strip_trivial_kernel(PairSrc src, int64_t n, T *out) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const PairRef pr = pair_ref(src, k);
+        const PairRef pr = pair_ref<true>(src, k);
         if (pr.la < 2 || pr.lb < 2) {
             out[pr.out0] = (T)1;
             if (pr.out1 >= 0) out[pr.out1] = (T)1;

@@ -124,7 +124,7 @@ __host__ __device__ inline void sym_index(int64_t k, int64_t n, int64_t &i, int6
     j = ii + (k - (ii * n - ii * (ii - 1) / 2));
 }
 
-template <bool EST32 = true>
+template <bool EST32 = false>
 __host__ __device__ inline PairRef pair_ref(const PairSrc &s, int64_t k) {
     PairRef r;
     k += s.kbase;

@@ -93,7 +93,7 @@ __global__ void vb_pairs_kernel(VbArgs a) {
     const int S = 1 << a.lam;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.n;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         VbPair p;
         memset(&p, 0, sizeof(p));
         p.cls = -1;

@@ -201,7 +201,7 @@ __global__ void vs_pairs_kernel(VsArgs a) {
     const int64_t a0 = a.src.a_off[a.src.kbase], b0 = a.src.b_off[a.src.kbase];
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.n;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         VsPair p;
         memset(&p, 0, sizeof(p));
         p.cls = -1;

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(W64_MAX_WARPS * 32) wave64_kernel(Wave64Args a
     double2 *ring = reinterpret_cast<double2 *>(w64_sm + L.ring);
     double *cf = w64_sm + L.coef;
 
-    const PairRef pr = pair_ref(a.src, k);
+    const PairRef pr = pair_ref<true>(a.src, k);
     w64_stage<RBF>(w64_sm, L, (const double *)a.src.A + pr.a_row0 * a.src.d,
                    (const double *)a.src.B + pr.b_row0 * a.src.d, d, a.nx, ny, a.vrows, rank * nrows, nrows, a.scale);
     if constexpr (PRE) w64_all_coefs<RBF>(cf, L.rs, w64_sm, L, d, nrows, ny, a.scale, a.rbf_s, a.src.scheme);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(W64B_MAX_WARPS * 32, 2) wave64_bwd_kernel(Wave
     };
 
     for (int64_t k = blockIdx.x; k < a.n_pairs; k += gridDim.x) {
-        const PairRef pr = pair_ref(a.src, k);
+        const PairRef pr = pair_ref<true>(a.src, k);
         const double *x = (const double *)a.src.A + pr.a_row0 * a.src.d;
         const double *y = (const double *)a.src.B + pr.b_row0 * a.src.d;
         __syncthreads();   // the shared arrays and the slot are free again
