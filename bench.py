@@ -304,11 +304,11 @@ def run_gpu(args):
         if not args.skip_fp64:
             Xd64 = torch.from_numpy(X64).to(dev)
             Yd64 = torch.from_numpy(Y64).to(dev)
-            sigk.gram(Xd64[:8], Yd64[:8], LAM)
+            sigk.gram(Xd64[:8], Yd64[:8], LAM, rec=sigk.REC_PLAIN)
             torch.cuda.synchronize(dev)
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record(st)
-            o64 = sigk.gram(Xd64, Yd64, LAM)
+            o64 = sigk.gram(Xd64, Yd64, LAM, rec=sigk.REC_PLAIN)
             b.record(st)
             torch.cuda.synchronize(dev)
             ms64 = a.elapsed_time(b)
@@ -449,10 +449,10 @@ def _workload(name, batch=0, cache=None):
         es = 8 if f64 else 4
         return dict(
             desc="Gram 8x8, L=M=32, d=3 (time + 2 walks), dyadic order 1, plus 8 straight-line pairs, %s"
-                 % ("fp64 (plain per-pair sweep, the printed scheme)" if f64 else "fp32 (chained register sweep)"),
+                 % ("fp64 (register wavefront, the printed scheme)" if f64 else "fp32 (chained register sweep)"),
             dtype="f64" if f64 else "f32", step=step, cells=cells, pairs=72,
             flop=3 * cells + 2 * 3 * coarse,
-            kernels="plain_kernel<double>" if f64 else "chain_f32_kernel",
+            kernels="wave64_kernel" if f64 else "chain_f32_kernel",
             oracle_rate=oracle_rate, parity=parity, host_step=host_step, host=host,
             h2d=sum(a.nbytes for a in src), d2h=72 * es)
 
@@ -636,7 +636,7 @@ def _workload(name, batch=0, cache=None):
             desc="gradient of sum_b g_b k(X_b, Y_b), %d pairs, L=M=4096, d=64 time-augmented walks, dyadic "
                  "order 1, fp32 (strip adjoint with checkpoints every 64 steps)" % nb,
             dtype="f32", step=step, cells=cells, pairs=nb, flop=2 * 64 * coarse + 13 * cells + 4 * 64 * coarse,
-            kernels="strip_adj_kernel + strip_kernel (checkpointing forward) + coef_tc5_kernel + grad_chain_kernel",
+            kernels="strip_adj_pack_kernel + grad_chain_tile_kernel + strip_kernel (checkpointing forward) + coef_tc5_kernel",
             oracle_rate=oracle_rate, parity=parity, host_step=host_step, host=host,
             h2d=X32.nbytes + Y32.nbytes, d2h=X32.nbytes)
 
@@ -731,9 +731,10 @@ def _workload(name, batch=0, cache=None):
                  "(cells: the forward cells of the U-statistic's %d distinct pairs)"
                  % (nb, nb, "RBF lift (sigma 1), " if rbf_sigma else "", u_pairs),
             dtype="f32", step=step, cells=cells, pairs=u_pairs, flop=flop,
-            kernels=("rbf_coef_kernel + chain_band_kernel + chain_band_adj_kernel + rbf_wt_kernel + "
-                     "dense_gemm_kernel (band form; fused value-and-gradient calls for Kxx and Kxy)" if rbf_sigma else
-                     "chain_band_adj_kernel + band_gemm_kernel + band_coef_kernel + chain_band_kernel "
+            kernels=("band_coef_kernel (lift) + rbf_wt_kernel + chain_band_adj_kernel + dense_gemm_kernel + "
+                     "chain_band_kernel (band form; fused value-and-gradient calls for Kxx and Kxy)" if rbf_sigma else
+                     "chain_band_adj_kernel + band_coef_kernel + band_rows_kernel + chain_band_kernel + "
+                     "band_cols_kernel "
                      "(band form; fused value-and-gradient calls for Kxx and Kxy)"),
             oracle_rate=oracle_rate, parity=parity, host_step=host_step, host=host,
             h2d=X32.nbytes + Y32.nbytes, d2h=X32.nbytes)
@@ -758,7 +759,7 @@ def _workload(name, batch=0, cache=None):
             okw = dict(static_kernel="rbf", sigma=1.0)
             cflop = 9 * d              # |u|^2, <u,dx>, <u,dy>, <dx,dy> and u = x_p - y_q per channel
             what = "RBF lift (sigma = 1), explicit scheme"
-            kern = "rbf_coef_kernel + chain_band_kernel"
+            kern = "band_coef_kernel (lift) + chain_band_kernel"
         n = (L - 1) << lam
         cells = nbx * nby * n * n
         coarse = nbx * nby * (L - 1) * (L - 1)
