@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(VB_PT) vb_plan_kernel(VbArgs a) {
 // twice the time of the operand reads; those are a broadcast over the
 // positions (rows, padded to a conflict-free stride, vb_lane_stride) or over
 // the lanes (columns).  4096 pairs of 16..512 points, d = 16, order 1: the call
-// 1.74 -> 1.41 ms, outputs bit for bit.
+// 1.74-1.78 -> 1.41-1.57 ms (it differs between processes), outputs bit for bit.
 // The unit (lane, position, part of a slot) of thread u of a pair, parts slowest
 // within a group of four positions.
 struct VbUnit {
