@@ -102,7 +102,10 @@ struct Wave64Args {
 
 // Padded coarse rows [P0, P0 + nrows) and all columns of a pair into shared
 // memory: increments (the linear kernel's rows scaled, exactly), and with the
-// RBF lift the points they start at and their squares.  Ends with a barrier.
+// RBF lift the points they start at and their squares.  A virtual row has a zero
+// increment and with the lift the path's first point, so its coefficients are
+// zero and what w64_coefs carries through it into the real rows of the same lane
+// is theirs.  Ends with a barrier.
 template <bool RBF>
 __device__ __forceinline__ void w64_stage(double *sm, const W64Shared &L, const double *x, const double *y, int d,
                                           int nx, int ny, int vrows, int P0, int nrows, double scale) {
@@ -112,7 +115,7 @@ __device__ __forceinline__ void w64_stage(double *sm, const W64Shared &L, const 
         const bool in = p >= 0 && p < nx;
         const double *r = x + (int64_t)(in ? p : 0) * d + c;
         sm[c * L.rs + P] = in ? (r[d] - r[0]) * f : 0.0;
-        if (RBF) sm[L.pts + c * L.rs + P] = in ? r[0] : 0.0;
+        if (RBF) sm[L.pts + c * L.rs + P] = r[0];   // a virtual row rests on the path's first point
     }
     for (int v = threadIdx.x; v < ny * d; v += blockDim.x) {
         const int q = v / d, c = v - q * d;
