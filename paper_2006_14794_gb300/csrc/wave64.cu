@@ -136,10 +136,61 @@ __device__ __forceinline__ void w64_stage(double *sm, const W64Shared &L, const 
     }
 }
 
+// |x| >= 2^e (or not a number), by its exponent bits: an FP64 compare would cost
+// an FP64 instruction.
+__device__ __forceinline__ bool w64_reaches(double x, int e) {
+    return (__double2hiint(x) & 0x7fffffff) >= (1023 + e) << 20;
+}
+// kappa at the end of a step less kappa at its start: exponents e0, e1 and their
+// difference x as the step's own points give it (from a difference of 1 on, where
+// little cancels, the two ends are exact to their own size).
+__device__ __forceinline__ double w64_step(double e0, double e1, double x) {
+    return w64_reaches(x, 0) ? exp(e1) - exp(e0) : exp(e0) * expm1(x);
+}
+// The second difference of kappa over the cell of points x, x + dx (channel
+// stride rs) and y, y + dy as the difference of two steps, along the side whose
+// kappa changes less from corner (p, q), every exponent from its own distance.
+// The product form kappa(p,q) (a b + (1 + a)(1 + b) e) is right where a, b and e
+// are of order one; beside a jump of several bandwidths e^A e^B cancels against
+// e^C (three corners near one another, the fourth five bandwidths off: 1e-9
+// relative, further off no digit is left) or overflows.  Against 80-bit
+// corners, 3 channels, points 0.1 to 10 bandwidths apart, steps of 0.01 to 60:
+// within 1.2e-13 of the value (of 0.001 for smaller ones), where the product form
+// is off by anything.
+__device__ __noinline__ double w64_far_cell(const double *x, const double *dx, int rs, const double *y,
+                                            const double *dy, int d, double rbf_s) {
+    double uu = 0.0, ux = 0.0, uy = 0.0, xx = 0.0, yy = 0.0;
+    for (int k = 0; k < d; ++k) {
+        const double u = x[k * rs] - y[k], xv = dx[k * rs], yv = dy[k];
+        uu = fma(u, u, uu);
+        ux = fma(u, xv, ux);
+        uy = fma(u, yv, uy);
+        xx = fma(xv, xv, xx);
+        yy = fma(yv, yv, yy);
+    }
+    const double A = rbf_s * (2.0 * uy - yy), B = -rbf_s * (2.0 * ux + xx);
+    const bool rows = fabs(A) >= fabs(B);   // steps along x (e: of u), at y_q and at y_{q+1}; else along y
+    double n0 = 0.0, n1 = 0.0, n2 = 0.0, w = 0.0;
+    for (int k = 0; k < d; ++k) {
+        const double u = x[k * rs] - y[k], xv = dx[k * rs], yv = dy[k];
+        const double e = rows ? xv : -yv, v = u + (rows ? -yv : xv);
+        const double a = u + e, b = v + e;
+        n0 = fma(a, a, n0);
+        n1 = fma(v, v, n1);
+        n2 = fma(b, b, n2);
+        w = fma(v, e, w);
+    }
+    return w64_step(-rbf_s * n1, -rbf_s * n2, -rbf_s * (2.0 * w + (rows ? xx : yy))) -
+           w64_step(-rbf_s * uu, -rbf_s * n0, rows ? B : A);
+}
+
 // The coefficients of local coarse rows P .. P + N - 1 at column q (in the
 // grid), the scheme's map applied.  With the RBF lift the second difference of
 // kappa (rbf_second_difference), what consecutive rows share carried down:
 // kappa(p+1, q) = kappa(p, q) (1 + b), expm1(A(p+1, q)) = a + e^A expm1(C).
+// Carried values keep their digits while the exponents stay below one: rows
+// with |A| or |B| of 1/2 or more, or C's that could add up to it, are formed one
+// by one (w64_far_cell).
 template <int N, bool RBF>
 __device__ __forceinline__ void w64_coefs(double (&c)[N], const double *sm, const W64Shared &L, int d, int nrows,
                                           int P, int q, double scale, double rbf_s, int scheme) {
@@ -174,10 +225,26 @@ __device__ __forceinline__ void w64_coefs(double (&c)[N], const double *sm, cons
                 g[i] = fma(xv, dv, g[i]);
             }
         }
-        double kap = exp(-rbf_s * uu), a = expm1(rbf_s * (2.0 * uy - sm[L.norms + nrows + q]));
+        constexpr int LOGN = N == 1 ? 0 : N == 2 ? 1 : N <= 4 ? 2 : N <= 8 ? 3 : 4;
+        static_assert(N <= 16, "LOGN");
+        const double A = rbf_s * (2.0 * uy - sm[L.norms + nrows + q]);
+        bool far = w64_reaches(A, -1);
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            const double b = expm1(-rbf_s * (2.0 * ux[i] + sm[L.norms + P + i])), e = expm1(2.0 * rbf_s * g[i]);
+            ux[i] = -rbf_s * (2.0 * ux[i] + sm[L.norms + P + i]);   // B
+            g[i] = 2.0 * rbf_s * g[i];                               // C
+            far = far || w64_reaches(ux[i], -1) || w64_reaches(g[i], -1 - LOGN);
+        }
+        if (far) {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                c[i] = scheme_coef(w64_far_cell(x0 + i, dx + i, L.rs, y0, dy, d, rbf_s) * scale, scheme);
+            return;
+        }
+        double kap = exp(-rbf_s * uu), a = expm1(A);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const double b = expm1(ux[i]), e = expm1(g[i]);
             const double ea = (1.0 + a) * e;   // expm1(A + C) - expm1(A)
             c[i] = scheme_coef(kap * fma(a, b, (1.0 + b) * ea) * scale, scheme);
             kap = fma(kap, b, kap);
@@ -684,7 +751,7 @@ bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kern
             if (bytes > W64_SMEM) continue;
             const int threads = pre && wpc * 32 < W64_HELP ? W64_HELP : wpc * 32;
             int64_t bps = (228 * 1024) / (bytes + 1024);
-            const int64_t regs = 65536 / (threads * (R > 8 ? 128 : 96));
+            const int64_t regs = 65536 / (threads * (R > 8 || (rbf && !pre) ? 128 : 96));
             if (bps > regs) bps = regs;
             if (bps < 1) continue;
             const double load = (double)(n * C) / sms;             // blocks a SM has to run,
