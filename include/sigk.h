@@ -126,7 +126,8 @@ typedef struct {
     int accumulate;   /* backward calls (sigk_pairs_backward, sigk_gram_backward,
                          sigk_gram_value_and_grad): 0 overwrites dX / dY, 1
                          adds the gradients to what dX / dY hold (a loss that
-                         sums several Grams of the same paths)                */
+                         sums several Grams of the same paths; dX and dY may
+                         then be one buffer, which receives both)             */
     int reserved[1];  /* must be 0                                            */
 } sigk_opts;          /* a NULL pointer means all-zero (automatic) options    */
 

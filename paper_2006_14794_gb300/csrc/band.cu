@@ -1606,7 +1606,8 @@ __global__ void band_split_sum_kernel(const float *partial, int ksplit, int64_t 
 
 // Point gradients from increment gradients: x_p enters dx_{p-1} (+) and dx_p
 // (-), so dX[path][p] = scale (dinc[p-1] - dinc[p]) (terms outside 0..L-2
-// absent).  Overwrites dpts, or adds to it (add).  Both roles in one launch;
+// absent).  Overwrites dpts, or adds to it (add).  Both roles in one launch,
+// where their outputs share no memory;
 // dinc may be the split partials of a contraction, `stride` floats apart, which
 // are then added in band_split_sum_kernel's order (one launch less, the same sums).
 struct PointsJob {
@@ -2472,10 +2473,18 @@ cudaError_t launch_band_bwd_f32(const PairSrc &src0, const BandPlan &p, int64_t 
                 jb.stride = g2.M * d;
             }
         }
-        if (ja.npaths || jb.npaths) {
-            band_points_kernel<<<sms * 4, 256, 0, st>>>(ja, jb, d, scale, add);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // outputs that share memory (one buffer that collects both derivatives of a
+        // Gram of X with itself) take the roles one after the other
+        const float *da = ja.dpts, *db = jb.dpts;
+        const bool shared = ja.npaths && jb.npaths && da < db + jb.npaths * jb.L * d && db < da + ja.npaths * ja.L * d;
+        if (shared) {
+            PointsJob none = jb;
+            none.npaths = 0;
+            band_points_kernel<<<sms * 4, 256, 0, st>>>(ja, none, d, scale, add);
+            ja.npaths = 0;
         }
+        if (ja.npaths || jb.npaths) band_points_kernel<<<sms * 4, 256, 0, st>>>(ja, jb, d, scale, add);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
