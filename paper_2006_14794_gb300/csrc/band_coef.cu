@@ -27,10 +27,14 @@
 // Only a slot's first cell of each row takes kappa, a and b from the points,
 // and its first row takes a in every column; every other cell adds its own
 // <dx,dy> and about 14 operations.  Carried values keep FP32 accuracy while a
-// and b stay of order one or below, so a slot with an |A| or |B| above
-// KC_CARRY, or C's that could add up to it, forms every cell from its points.  Before, each cell formed all six sums
-// (9 d operations), three series and two exponentials, 183 instructions at
-// d = 8, and stored its value alone into a zero-filled band.
+// and b stay of order one or below, so a slot with an |A| or |B| above KC_CARRY,
+// or C's that could add up to it (data rough on the scale of the bandwidth),
+// sums |u|^2 of every cell and forms each with its own exponentials, A and B
+// moved on by C (kc_rough): 256 x 256 Gram of 128-point paths, d = 8, order 2, with a
+// bandwidth of 0.2 where the paths span 1: 9.3 ms, 38 with such cells one at a
+// time from their points, 10.8 before cells were carried at all, when each formed
+// all six sums (9 d operations), three series and two exponentials and stored its
+// value alone into a zero-filled band.
 //
 // Measured: the lift over 3840 pairs of 256-point paths, d = 32, order 1, 2.9 ->
 // 1.16 ms; over a 256 x 256 Gram of 128-point paths, d = 8, order 2, 7.4 (zero
@@ -38,22 +42,24 @@
 // (0.67 in this form with 32 lanes of one position a warp).
 // Padding: rows and columns outside the path repeat its end points, so their
 // increments and with them c are exactly zero.
+#include "rbf.cuh"
 #include "sigk_internal.cuh"
 
 namespace sigk {
 
 namespace {
 
-constexpr int KC_CH = 32;          // channels staged at a time
+constexpr int KC_CH = 32;          // channels staged at a time by the linear kernel (the lift: all)
 // Lanes a warp covers, positions a thread, most positions a unit, most warps a
 // block.  12 warps a SM have 168 registers each; a pair of 33 positions (256
-// points at dyadic order 1) is 36 warp items, three a warp.
+// points at dyadic order 1) is 36 warp items, three a warp.  Narrow lanes run 18
+// warps a SM: two blocks of 9, or with the lift's shared memory one of 18.
 template <int NG, bool RBF>
 struct KcShape {
     static constexpr int LW = NG == 8 ? 8 : 16, NP = NG == 8 ? 1 : NG == 4 ? 2 : 4;
     static constexpr int GP = 32 / LW * NP;   // positions a warp item
     static constexpr int TILE = 36, TILEC = 12;   // (TILEC: with more channels than are staged at once)
-    static constexpr int WARPS = NG == 8 ? 12 : 9, MINB = NG == 8 ? 1 : 2;
+    static constexpr int WARPS = NG == 8 ? 12 : RBF ? 18 : 9, MINB = NG == 8 || RBF ? 1 : 2;
 };
 constexpr float KC_CARRY = 0.5f;   // see above: a, b <= e^1 - 1 along a slot
 
@@ -178,54 +184,24 @@ __device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs
         }
 }
 
-// kappa at the end of a step less kappa at its start, exponents E0 and E1 = E0 + x.
-__device__ __forceinline__ float kc_step(float E0, float E1, float x) {
-    return fabsf(x) <= 4.f ? __expf(E0) * expm1_taylor(x) : expf(E1) - expf(E0);
-}
-// The second difference of kappa over the cell of points x, x + d and y, y + d.
-// Where an exponent from corner (p, q) is above 4 in size (a jump of several
-// bandwidths: e^A overflows, or A cancels against |u|^2), it is the difference
-// of the two steps along the side with the smaller one, every corner from its
-// own distance.
-__device__ __forceinline__ float kc_second_difference(const float *x, const float *y, int64_t d, float s) {
-    float uu = 0.f, ux = 0.f, uy = 0.f, xy = 0.f, xx = 0.f, yy = 0.f;
-    for (int64_t i = 0; i < d; ++i) {
-        const float u = x[i] - y[i], dx = x[i + d] - x[i], dy = y[i + d] - y[i];
-        uu = fmaf(u, u, uu); ux = fmaf(u, dx, ux); uy = fmaf(u, dy, uy);
-        xy = fmaf(dx, dy, xy); xx = fmaf(dx, dx, xx); yy = fmaf(dy, dy, yy);
+// The scheme's map, then to the band.
+template <int NG>
+__device__ __forceinline__ void kc_put(const KcArgs &a, float2 (&v)[NG][NG / 2], int64_t k, int pos, int l) {
+    if (a.src.scheme != SIGK_SCHEME_EXPLICIT) {
+#pragma unroll
+        for (int w = 0; w < NG; ++w)
+#pragma unroll
+            for (int h = 0; h < NG / 2; ++h)
+                v[w][h] = make_float2(scheme_coef(v[w][h].x, a.src.scheme), scheme_coef(v[w][h].y, a.src.scheme));
     }
-    const float A = s * (2.f * uy - yy), B = -s * (2.f * ux + xx);
-    if (fmaxf(fabsf(A), fabsf(B)) <= 4.f) return rbf_second_difference(uu, ux, uy, xy, xx, yy, s);
-    float n01 = 0.f, n10 = 0.f, n11 = 0.f, ux1 = 0.f, uy1 = 0.f;
-    for (int64_t i = 0; i < d; ++i) {
-        const float u01 = x[i] - y[i + d], u10 = x[i + d] - y[i], u11 = x[i + d] - y[i + d];
-        n01 = fmaf(u01, u01, n01); n10 = fmaf(u10, u10, n10); n11 = fmaf(u11, u11, n11);
-        ux1 = fmaf(u01, x[i + d] - x[i], ux1); uy1 = fmaf(u10, y[i + d] - y[i], uy1);
-    }
-    return fabsf(A) >= fabsf(B) ? kc_step(-s * n01, -s * n11, -s * (2.f * ux1 + xx)) - kc_step(-s * uu, -s * n10, B)
-                                : kc_step(-s * n10, -s * n11, s * (2.f * uy1 - yy)) - kc_step(-s * uu, -s * n01, A);
+    kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos, l, v);
 }
 
-// The slot's cells one by one from the points (RBF lift), stored as kc_store does.
+// Entry j of the staged column points as a pair (column, column - NG/2).
 template <int NG>
-__device__ __noinline__ void kc_slot_direct(const KcArgs &a, int64_t k, int64_t row0, int64_t col0, int pos, int l) {
-    constexpr int SLOT = NG * NG;
-    const int64_t d = a.src.d;
-    const int ny = (int)a.src.Lb - 1;
-    const bool tail = pos == a.TperR;
-    float *dst = a.band + band_row(k * a.TperR + pos, l, NG, a.n_pairs * a.TperR + 1);   // tail: slot 0 of the next pair
-    for (int e = 0; e < SLOT; ++e) {
-        const int w = e / NG, g = e - w * NG;
-        const bool other = tail ? w >= g : (pos == 0 && w < g);   // the neighbour pair's cell
-        if (other && k != (tail ? a.n_pairs - 1 : 0)) continue;
-        const int p = l * NG + g - a.vrows, q = pos * NG + w - g - a.NQV;
-        float c = 0.f;
-        if (!other && p >= 0 && q >= 0 && q < ny) {
-            const float *x = (const float *)a.src.A + (row0 + p) * d, *y = (const float *)a.src.B + (col0 + q) * d;
-            c = scheme_coef(kc_second_difference(x, y, d, a.s) * a.scale, a.src.scheme);
-        }
-        dst[band_off(w * NG + 2 * (g % (NG / 2)) + g / (NG / 2))] = c;
-    }
+__device__ __forceinline__ float2 kc_points(const float *q, int j) {
+    if constexpr (kc_pp<NG>() == 2) return reinterpret_cast<const float2 *>(q)[j];
+    else return make_float2(q[j], q[j - NG / 2]);
 }
 
 // The sums of a slot's first cells (RBF lift): rows h, h + NG/2 at entry NG - 1 -
@@ -245,30 +221,143 @@ struct KcFirst {
         float2 xv[NH], dv[NH];
         kc_rows<NG>(xv, xp, l);
         kc_rows<NG>(dv, xi, l);
-        auto pts = [&](int j) {
-            if constexpr (kc_pp<NG>() == 2) return reinterpret_cast<const float2 *>(q)[j];
-            else return make_float2(q[j], q[j - NH]);
-        };
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
-            const float2 u = __ffma2_rn(pts(NG - 1 - h), minus, xv[h]);
+            const float2 u = __ffma2_rn(kc_points<NG>(q, NG - 1 - h), minus, xv[h]);
             uu[h] = __ffma2_rn(u, u, uu[h]);
             ux[h] = __ffma2_rn(u, dv[h], ux[h]);
             uy[h] = __ffma2_rn(u, e[NG - 1 - h], uy[h]);
-            const float2 t = __ffma2_rn(pts(NG + NH - 1 + h), minus, kc2(xv[0].x));
+            const float2 t = __ffma2_rn(kc_points<NG>(q, NG + NH - 1 + h), minus, kc2(xv[0].x));
             ur[h] = __ffma2_rn(t, e[NG + NH - 1 + h], ur[h]);
         }
     }
 };
 
+// A slot that cannot be carried (RBF lift), formed one cell at a time: C and |u|^2 of
+// every cell, and the exponents of its first ones (kc_exponents).
+template <int NG>
+struct KcRough {
+    static constexpr int NH = NG / 2;
+    float2 c[NG][NH], uu[NG][NH];
+    float2 a[NH], b[NH], top[NH];
+};
+// A rough slot: the |u|^2 of its cells over the staged channels (xp, yp: the first
+// one's), then their coefficients, to the band.  In a function of its own, so that
+// the other slots' registers do not pay for it.  kappa comes from each cell's
+// own distance; A and B move on by C, which costs them the rounding of a few
+// additions.  A cell is the product form where A and B are below 1/2, else the
+// difference of the two steps along the side that changes less (rbf.cuh), both
+// for all, without branches; cells beside far jumps, where that rounding shows, are
+// formed from their points.
+template <int NG>
+__device__ __noinline__ void kc_rough(KcRough<NG> &r, const KcArgs &a, const float *xp, const float *yp, int ys, int64_t k,
+                                      int64_t row0, int64_t col0, int pos, int l) {
+    constexpr int NH = NG / 2;
+    const float2 minus = kc2(-1.f);
+    {
+        const int nc = (int)a.src.d;
+        float2 uu[NG][NH];
+#pragma unroll
+        for (int w = 0; w < NG; ++w)
+#pragma unroll
+            for (int h = 0; h < NH; ++h) uu[w][h] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c, xp += kc_xs<NG>(), yp += ys) {
+            float2 xv[NH], yv[2 * NG - 1];
+            kc_rows<NG>(xv, xp, l);
+            if constexpr (NG == 8) {
+                float q[16];
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) {
+                    const float4 t = *reinterpret_cast<const float4 *>(yp + j);
+                    q[j] = t.x; q[j + 1] = t.y; q[j + 2] = t.z; q[j + 3] = t.w;
+                }
+#pragma unroll
+                for (int j = NH; j < 2 * NG - 1; ++j) yv[j] = make_float2(q[j], q[j - NH]);
+            } else {
+#pragma unroll
+                for (int j = NH; j < 2 * NG - 1; ++j) yv[j] = kc_points<NG>(yp, j);
+            }
+#pragma unroll
+            for (int w = 0; w < NG; ++w)
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    const float2 u = __ffma2_rn(yv[NG - 1 + w - h], minus, xv[h]);
+                    uu[w][h] = __ffma2_rn(u, u, uu[w][h]);
+                }
+        }
+#pragma unroll
+        for (int w = 0; w < NG; ++w)
+#pragma unroll
+            for (int h = 0; h < NH; ++h) r.uu[w][h] = uu[w][h];
+    }
+    const float s = a.s;
+    float2 av[NH], bv[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) { av[h] = r.a[h]; bv[h] = r.b[h]; }
+    float most = 0.f;   // the largest exponent so far
+    auto exp2v = [](float2 v) { return make_float2(__expf(v.x), __expf(v.y)); };
+    // a step of x from e0 to e1, series = e^x - 1 where |x| <= 1/2
+    auto step = [](float x, float series, float e0, float e1) { return fabsf(x) <= 0.5f ? e0 * series : e1 - e0; };
+#pragma unroll 1
+    for (int w = 0; w < NG; ++w) {
+        float2 an[NH];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const float2 A = av[h], B = bv[h], C = r.c[w][h], E = __fmul2_rn(kc2(-s), r.uu[w][h]);
+            const bool rx = fabsf(A.x) >= fabsf(B.x), ry = fabsf(A.y) >= fabsf(B.y);
+            // v: the steps' exponent at this corner (the smaller one), o: between the two steps
+            const float2 v = make_float2(rx ? B.x : A.x, ry ? B.y : A.y), o = make_float2(rx ? A.x : B.x, ry ? A.y : B.y);
+            const float2 v1 = __fadd2_rn(v, C), E1 = __fadd2_rn(E, o);
+            const float2 sv = kc_expm1<8>(v), so = kc_expm1<8>(o), sc = kc_expm1<8>(C), s1 = kc_expm1<8>(v1);
+            const float2 e = exp2v(E), ev = exp2v(__fadd2_rn(E, v)), eo = exp2v(E1), eov = exp2v(__fadd2_rn(E1, v1));
+            const float2 eC = __ffma2_rn(so, sc, sc);   // (1 + so) sc
+            const float2 near = __fmul2_rn(e, __ffma2_rn(sv, so, __ffma2_rn(sv, eC, eC)));
+            float2 c = near;
+            if (fmaxf(fabsf(o.x), fabsf(C.x)) > 0.5f) c.x = step(v1.x, s1.x, eo.x, eov.x) - step(v.x, sv.x, e.x, ev.x);
+            if (fmaxf(fabsf(o.y), fabsf(C.y)) > 0.5f) c.y = step(v1.y, s1.y, eo.y, eov.y) - step(v.y, sv.y, e.y, ev.y);
+            // the exponents so far leave an error of their size times 2^-24; to the
+            // points where it shows (a corner's kappa times it above 1e-7), or where
+            // they are too large to tell
+            most = fmaxf(most, fmaxf(fmaxf(fmaxf(fabsf(A.x), fabsf(A.y)), fmaxf(fabsf(B.x), fabsf(B.y))),
+                                     fmaxf(fabsf(C.x), fabsf(C.y))));
+            auto shows = [&](float E0, float top) {
+                const float m = fmaxf(most, fabsf(E0));
+                return m > 32.f && (m * top > 2.f || m > 1e7f);
+            };
+            const bool fx = shows(E.x, fmaxf(fmaxf(e.x, ev.x), fmaxf(eo.x, eov.x)));
+            const bool fy = shows(E.y, fmaxf(fmaxf(e.y, ev.y), fmaxf(eo.y, eov.y)));
+            if (fx || fy) {
+                const int64_t d = a.src.d;
+#pragma unroll 1
+                for (int i = fx ? 0 : 1; i < (fy ? 2 : 1); ++i) {
+                    const int g = h + i * NH, p = l * NG + g - a.vrows, q = pos * NG + w - g - a.NQV;
+                    float t = 0.f;
+                    if (p >= 0 && q >= 0 && q < (int)a.src.Lb - 1)
+                        t = rbf_far_cell((const float *)a.src.A + (row0 + p) * d,
+                                         (const float *)a.src.B + (col0 + q) * d, d, s);
+                    if (i == 0) c.x = t;
+                    else c.y = t;
+                }
+            }
+            r.c[w][h] = __fmul2_rn(kc2(a.scale), c);
+            an[h] = __fadd2_rn(A, C);
+            bv[h] = __fadd2_rn(B, C);
+        }
+#pragma unroll
+        for (int h = NH - 1; h >= 1; --h) av[h] = an[h - 1];
+        av[0] = make_float2(w + 1 < NH ? r.top[w + 1].y : w + 1 < NG ? r.top[w + 1 - NH].x : 0.f, an[NH - 1].x);
+    }
+    kc_put<NG>(a, r.c, k, pos, l);
+}
+
 // A slot's sums <dx,dy> into its coefficients (RBF lift).  Everything is done
 // for rows h and h + NG/2 at once; at window w row g is one column ahead of row
 // g + 1, so a(g + 1) of the next window is a(g) + (1 + a(g)) e(g) of this one.
-// False where the slot was formed cell by cell.
+// False where the slot is rough: r then holds its C's and first exponents.
 template <int NG>
-__device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcFirst<NG> &first, const KcArgs &a,
-                                        int64_t k, const PairRef &pr, int pos, int l, const float *xx,
-                                        const float *yy) {
+__device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcFirst<NG> &first, KcRough<NG> &r,
+                                        const KcArgs &a, int l, const float *xx, const float *yy) {
     constexpr int NH = NG / 2;
     const float s = a.s, s2 = 2.f * s;
     float far = 0.f;
@@ -294,7 +383,16 @@ __device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcFirst
         bv[h] = arg(first.ux[h], sq[h], -1.f);
     }
     if (far > KC_CARRY) {
-        kc_slot_direct<NG>(a, k, pr.a_row0, pr.b_row0, pos, l);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            r.a[h] = av[h];
+            r.b[h] = bv[h];
+            r.top[h] = top[h];
+        }
+#pragma unroll
+        for (int w = 0; w < NG; ++w)
+#pragma unroll
+            for (int h = 0; h < NH; ++h) r.c[w][h] = acc[w][h];
         return false;
     }
 #pragma unroll
@@ -324,8 +422,7 @@ __device__ __forceinline__ bool kc_lift(float2 (&acc)[NG][NG / 2], const KcFirst
     return true;
 }
 
-// MULTI: more channels than are staged at once (one pass; sums kept over the
-// chunks, in more registers than the common case needs)
+// MULTI: more channels than are staged at once (one pass; linear kernel)
 template <int NG, bool RBF, bool MULTI>
 __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>::MINB) band_coef_kernel(KcArgs a) {
     extern __shared__ __align__(16) float kc_sm[];
@@ -334,7 +431,7 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
     const int nt = blockDim.x, tid = threadIdx.x, warp = tid >> 5;
     const int lw = tid & (Sh::LW - 1), jw = (tid & 31) / Sh::LW;   // lane and position in the warp's item
     const int64_t d = a.src.d;
-    const int nch = d < KC_CH ? (int)d : KC_CH, YS = kc_ys(a.tp, NG);
+    const int nch = RBF || d < KC_CH ? (int)d : KC_CH, YS = kc_ys(a.tp, NG);
     float *xi = kc_sm;                                            // row increments (linear: scaled)
     float *y0 = xi + a.xch * XS;                                  // the next step's column points
     float2 *yi = reinterpret_cast<float2 *>(y0 + nch * YS);       // pairs of column increments
@@ -352,8 +449,8 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
     // channels c0 .. c0 + nc - 1 of the row path's increments (and points) from xi[at XS] on
     auto stage_x = [&](int64_t row0, int64_t c0, int nc, int at) {
         const float *x = (const float *)a.src.A + row0 * d + c0;
-        const int gs = kc_group(nc), c = tid & (gs - 1);
-        if (c < nc)
+        const int gs = kc_group(nc);
+        for (int c = tid & (gs - 1); c < nc; c += RBF ? gs : nc)
             for (int P = tid / gs; P < NPP; P += nt / gs) {
                 const int p = P - a.vrows;
                 const float *r = x + (int64_t)(p < 0 ? 0 : p) * d + c;
@@ -365,8 +462,8 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
     // tile t's column points, ends repeated, into y0[c][iq], Q = t tp NG + iq - (NG - 1)
     auto fetch_y = [&](int64_t row0, int t, int64_t c0, int nc) {
         const float *y = (const float *)a.src.B + row0 * d + c0;
-        const int gs = kc_group(nc), c = tid & (gs - 1), Q0 = t * a.tp * NG - (NG - 1) - a.NQV;
-        if (c < nc)
+        const int gs = kc_group(nc), Q0 = t * a.tp * NG - (NG - 1) - a.NQV;
+        for (int c = tid & (gs - 1); c < nc; c += RBF ? gs : nc)
             for (int iq = tid / gs; iq < YS; iq += nt / gs) {
                 int q = Q0 + iq;
                 q = q < 0 ? 0 : (q > ny ? ny : q);
@@ -409,7 +506,6 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
     int64_t staged = -1;   // the row path whose values xi (and xp) hold
     fetch_y(pr.b_row0, tn, 0, nch);
     float2 acc[NP][NG][NH];
-    KcFirst<NG> first[RBF && MULTI ? NP : 1];
     for (int64_t u = ubeg; u < uend; ++u) {
         const PairRef cur = pr;
         const int64_t k = kn;
@@ -421,14 +517,14 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
         }
         for (int ch = 0; ch < chunks; ++ch) {
             const int64_t c0 = (int64_t)ch * KC_CH;
-            const int nc = d - c0 < KC_CH ? (int)(d - c0) : KC_CH;
+            const int nc = RBF ? (int)d : d - c0 < KC_CH ? (int)(d - c0) : KC_CH;
             kc_wait();
             __syncthreads();   // this step's columns are here, and the last step's readers are done
             const bool fresh = !keep || staged != cur.a_row0;
             if (fresh) {
                 if (keep)
-                    for (int64_t c = 0; c < d; c += KC_CH)
-                        stage_x(cur.a_row0, c, d - c < KC_CH ? (int)(d - c) : KC_CH, (int)c);
+                    for (int64_t c = 0; c < d; c += RBF ? d : KC_CH)
+                        stage_x(cur.a_row0, c, RBF ? (int)d : d - c < KC_CH ? (int)(d - c) : KC_CH, (int)c);
                 else
                     stage_x(cur.a_row0, c0, nc, 0);
                 staged = cur.a_row0;
@@ -452,10 +548,6 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
                         for (int w = 0; w < NG; ++w)
 #pragma unroll
                             for (int h = 0; h < NH; ++h) acc[n][w][h] = make_float2(0.f, 0.f);
-                    if constexpr (RBF && MULTI) {
-#pragma unroll
-                        for (int n = 0; n < NP; ++n) first[n].clear();
-                    }
                 }
                 const float2 *yr = yi + rel * NG;   // entry j: columns Q = pos NG - (NG - 1) + j and Q - NG/2
 #pragma unroll 2
@@ -477,31 +569,30 @@ __global__ void __launch_bounds__(KcShape<NG, RBF>::WARPS * 32, KcShape<NG, RBF>
                         f.add(xq + c * XS, xc + c * XS, yr + c * YS + n * NG,
                               yp + (c * YS + (rel + n) * NG) * kc_pp<NG>(), l);
                 };
-                if constexpr (RBF && MULTI) {
-#pragma unroll
-                    for (int n = 0; n < NP; ++n) add_first(first[n], n);
-                }
                 if (!live || ch + 1 < chunks) continue;
+                KcRough<NG> rough[RBF ? NP : 1];
+                unsigned bad = 0;   // the slots that are rough
 #pragma unroll
                 for (int n = 0; n < NP; ++n) {
                     if (n > 0 && (rel + n >= a.tp || pos + n > a.TperR)) break;
                     if constexpr (RBF) {
-                        KcFirst<NG> &f = first[MULTI ? n : 0];
-                        if constexpr (!MULTI) {
-                            f.clear();
-                            add_first(f, n);
+                        KcFirst<NG> f;
+                        f.clear();
+                        add_first(f, n);
+                        if (!kc_lift<NG>(acc[n], f, rough[n], a, l, xx, yy + (rel + n) * NG)) {
+                            bad |= 1u << n;
+                            continue;
                         }
-                        if (!kc_lift<NG>(acc[n], f, a, k, cur, pos + n, l, xx, yy + (rel + n) * NG)) continue;
                     }
-                    if (a.src.scheme != SIGK_SCHEME_EXPLICIT) {
-#pragma unroll
-                        for (int w = 0; w < NG; ++w)
-#pragma unroll
-                            for (int h = 0; h < NH; ++h)
-                                acc[n][w][h] = make_float2(scheme_coef(acc[n][w][h].x, a.src.scheme),
-                                                           scheme_coef(acc[n][w][h].y, a.src.scheme));
-                    }
-                    kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos + n, l, acc[n]);
+                    kc_put<NG>(a, acc[n], k, pos + n, l);
+                }
+                if constexpr (RBF) {
+                    if (bad)
+#pragma unroll 1
+                        for (int n = 0; n < NP; ++n)
+                            if (bad >> n & 1)
+                                kc_rough<NG>(rough[n], a, xq, yp + (rel + n) * NG * kc_pp<NG>(), YS * kc_pp<NG>(), k,
+                                             cur.a_row0, cur.b_row0, pos + n, l);
                 }
             }
         }
@@ -513,14 +604,15 @@ cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
     KcArgs a = a0;
     const int npos = a.TperR + 1;
     using Sh = KcShape<NG, RBF>;
-    const int d = (int)a.src.d, nch = d < KC_CH ? d : KC_CH;
-    a.chunks = (d + KC_CH - 1) / KC_CH;
-    const int most = a.chunks > 1 ? Sh::TILEC : Sh::TILE;
-    a.tiles = (npos + most - 1) / most;
-    a.tp = ((npos + a.tiles - 1) / a.tiles + Sh::NP - 1) / Sh::NP * Sh::NP;
-    const int items = (a.tp + Sh::GP - 1) / Sh::GP * (32 / Sh::LW);
-    a.passes = a.chunks > 1 ? 1 : (items + Sh::WARPS - 1) / Sh::WARPS;
-    const int warps = (items + a.passes - 1) / a.passes;
+    const int d = (int)a.src.d, nch = RBF || d < KC_CH ? d : KC_CH;
+    a.chunks = (d + nch - 1) / nch;
+    // the largest even share of the positions that fits
+    auto share = [&](int most) {
+        a.tiles = (npos + most - 1) / most;
+        a.tp = ((npos + a.tiles - 1) / a.tiles + Sh::NP - 1) / Sh::NP * Sh::NP;
+        return (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch) <= 226 * 1024;
+    };
+    for (int most = a.chunks > 1 ? Sh::TILEC : Sh::TILE; !share(most); most -= Sh::GP) {}
     // a row path's channels all stay where they fit (two chunks do)
     a.xch = d;
     int smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch);
@@ -528,6 +620,10 @@ cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
         smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d);
     else
         a.xch = nch;
+    const int items = (a.tp + Sh::GP - 1) / Sh::GP * (32 / Sh::LW);
+    const int most = RBF && NG < 8 && smem <= 113 * 1024 ? Sh::WARPS / 2 : Sh::WARPS;
+    a.passes = a.chunks > 1 ? 1 : (items + most - 1) / most;
+    const int warps = (items + a.passes - 1) / a.passes;
     auto go = [&](auto kern) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -539,8 +635,55 @@ cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
         kern<<<(int)grid, warps * 32, smem, st>>>(a);
         return cudaGetLastError();
     };
-    return a.chunks > 1 ? go(band_coef_kernel<NG, RBF, true>) : go(band_coef_kernel<NG, RBF, false>);
+    if constexpr (!RBF)
+        if (a.chunks > 1) return go(band_coef_kernel<NG, false, true>);
+    return go(band_coef_kernel<NG, RBF, false>);
 }
+
+// The band as rbf.cuh's tiles write it: coarse cell (p, q) is the padded cell (P, Q)
+// = (p + vrows, q + NQV), in lane P / NG as row g = P % NG, at the position pos and
+// window w with pos NG + w = Q + g.
+template <int NG>
+struct KcTileLayout {
+    PairSrc src;
+    float *band;
+    int64_t nslots;
+    int TperR, NQV, vrows;
+    struct Geo {
+        const float *rows, *cols;
+        int nx, ny;
+        int64_t k;
+    };
+    struct Row {
+        int l, g;
+    };
+    __device__ Geo geo(int64_t k) const {
+        const PairRef pr = pair_ref<true>(src, k);
+        return {(const float *)src.A + pr.a_row0 * src.d, (const float *)src.B + pr.b_row0 * src.d, (int)pr.la - 1,
+                (int)pr.lb - 1, k};
+    }
+    __device__ Row row(const Geo &, int p) const { return {(p + vrows) / NG, (p + vrows) % NG}; }
+    __device__ void store(const Geo &g, const Row &r, int q, float c) const {
+        const int t = q + NQV + r.g, at = t % NG * NG + 2 * (r.g % (NG / 2)) + r.g / (NG / 2);
+        band[band_row(g.k * TperR + t / NG, r.l, NG, nslots) + band_off(at)] = c;
+    }
+};
+
+template <int NG>
+cudaError_t launch_tiles(const KcArgs &a, int sms, cudaStream_t st) {
+    const int64_t nslots = a.n_pairs * a.TperR + 1;
+    const KcTileLayout<NG> lay = {a.src, a.band, nslots, a.TperR, a.NQV, a.vrows};
+    return launch_rbf_coef<float>(lay, a.n_pairs, a.src.La - 1, a.src.Lb - 1, a.src.d, a.src.sigma, (double)a.scale,
+                                  a.src.scheme, a.band, sizeof(float) * (size_t)nslots * 32 * NG * NG, sms, st);
+}
+
+// The lift with more channels than a block stages takes rbf.cuh's tiles, every cell
+// from its own six sums.  Carrying over several passes of channels keeps twice the
+// sums in registers: 1.07 times as fast as the tiles at d = 130 (48 x 48 paths of 100
+// and 90 points, order 1), 0.67 times at d = 100 (96 x 96 of 30 and 33, order 0), and
+// on rough data, where a slot needs every channel once more, a third to a half.  With
+// all of d = 64 staged at once it is 1.4 times as fast (64 x 64 of 128, order 0).
+constexpr int KC_LIFT = 64;
 
 }  // namespace
 
@@ -557,6 +700,9 @@ cudaError_t launch_band_coefs(const PairSrc &src, const BandPlan &p, int64_t n_p
     a.scale = 0.5f / (float)(1 << (2 * p.lam));
     a.s = (float)(0.5 / (src.sigma * src.sigma));
     const bool rbf = src.kernel == SIGK_KERNEL_RBF;
+    if (rbf && src.d > KC_LIFT)
+        return p.NG == 8 ? launch_tiles<8>(a, sms, st)
+                         : p.NG == 4 ? launch_tiles<4>(a, sms, st) : launch_tiles<2>(a, sms, st);
     if (p.NG == 8) return rbf ? launch<8, true>(a, sms, st) : launch<8, false>(a, sms, st);
     if (p.NG == 4) return rbf ? launch<4, true>(a, sms, st) : launch<4, false>(a, sms, st);
     return rbf ? launch<2, true>(a, sms, st) : launch<2, false>(a, sms, st);

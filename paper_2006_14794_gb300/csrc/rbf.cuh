@@ -34,6 +34,44 @@ constexpr int RBF_TC = 32;    // tile columns: 4 per thread
 constexpr int RBF_CH = 32;    // channels staged per pass
 constexpr int RBF_THREADS = 256;
 
+// FP32 cells beside jumps.  kappa at the end of a step less kappa at its start,
+// exponents E0 and E1 = E0 + x:
+__device__ __forceinline__ float rbf_step(float E0, float E1, float x) {
+    return fabsf(x) <= 4.f ? __expf(E0) * expm1_taylor(x) : expf(E1) - expf(E0);
+}
+// The second difference of kappa over the cell of points x, x + d and y, y + d as
+// the difference of the two steps along the side that changes less, every corner
+// from its own distance.
+static __device__ __noinline__ float rbf_far_cell(const float *x, const float *y, int64_t d, float s) {
+    float uu = 0.f, n01 = 0.f, n10 = 0.f, n11 = 0.f, ux = 0.f, uy = 0.f, ux1 = 0.f, uy1 = 0.f, xx = 0.f, yy = 0.f;
+    for (int64_t i = 0; i < d; ++i) {
+        const float u = x[i] - y[i], dx = x[i + d] - x[i], dy = y[i + d] - y[i];
+        const float u01 = x[i] - y[i + d], u10 = x[i + d] - y[i], u11 = x[i + d] - y[i + d];
+        uu = fmaf(u, u, uu); ux = fmaf(u, dx, ux); uy = fmaf(u, dy, uy);
+        xx = fmaf(dx, dx, xx); yy = fmaf(dy, dy, yy);
+        n01 = fmaf(u01, u01, n01); n10 = fmaf(u10, u10, n10); n11 = fmaf(u11, u11, n11);
+        ux1 = fmaf(u01, dx, ux1); uy1 = fmaf(u10, dy, uy1);
+    }
+    const float A = s * (2.f * uy - yy), B = -s * (2.f * ux + xx);
+    return fabsf(A) >= fabsf(B) ? rbf_step(-s * n01, -s * n11, -s * (2.f * ux1 + xx)) - rbf_step(-s * uu, -s * n10, B)
+                                : rbf_step(-s * n10, -s * n11, s * (2.f * uy1 - yy)) - rbf_step(-s * uu, -s * n01, A);
+}
+// The second difference from the exponents E = -s |u|^2, A, B and C
+// (sigk_internal.cuh).  Above 4 in size they overflow, or cancel, in the product
+// form: the two steps instead, their corners' exponents from this one's.  That
+// leaves an error of the exponents' size times 2^-24: from the points where it shows
+// (a corner's kappa times it above 1e-7), or where they are too large to tell.
+__device__ __forceinline__ float rbf_cell(float E, float A, float B, float C, float s, const float *x, const float *y,
+                                          int64_t d) {
+    const float far = fmaxf(fmaxf(fabsf(A), fabsf(B)), fabsf(C));
+    if (far <= 4.f) return __expf(E) * (expm1_taylor(A) * expm1_taylor(B) + __expf(A + B) * expm1_taylor(C));
+    const bool rows = fabsf(A) >= fabsf(B);
+    const float v = rows ? B : A, E1 = E + (rows ? A : B), v1 = v + C, most = fmaxf(far, fabsf(E));
+    if (most <= 32.f || (most < 1e7f && most * __expf(fmaxf(fmaxf(E, E1), fmaxf(E + v, E1 + v1))) <= 2.f))
+        return rbf_step(E1, E1 + v1, v1) - rbf_step(E, E + v, v);
+    return rbf_far_cell(x, y, d, s);
+}
+
 template <typename T, class Layout>
 __global__ void __launch_bounds__(RBF_THREADS) rbf_coef_kernel(Layout lay, int64_t n_pairs, int tiles_r,
                                                                int tiles_c, int64_t d, T s, T scale,
@@ -132,10 +170,12 @@ __global__ void __launch_bounds__(RBF_THREADS) rbf_coef_kernel(Layout lay, int64
                     if (q < g.ny) {
                         const int h = j >> 1;
                         const bool hi = j & 1;
-                        const float G = rbf_second_difference(
-                            hi ? uu2[i][h].y : uu2[i][h].x, hi ? ux2[i][h].y : ux2[i][h].x,
-                            hi ? uy2[i][h].y : uy2[i][h].x, hi ? xy2[i][h].y : xy2[i][h].x, nxs[i],
-                            hi ? ny2[h].y : ny2[h].x, (float)s);
+                        const float f = (float)s, uyv = hi ? uy2[i][h].y : uy2[i][h].x;
+                        const float G = rbf_cell(-f * (hi ? uu2[i][h].y : uu2[i][h].x),
+                                                 f * (2.f * uyv - (hi ? ny2[h].y : ny2[h].x)),
+                                                 -f * (2.f * (hi ? ux2[i][h].y : ux2[i][h].x) + nxs[i]),
+                                                 2.f * f * (hi ? xy2[i][h].y : xy2[i][h].x), f,
+                                                 g.rows + (int64_t)p * d, g.cols + (int64_t)q * d, d);
                         lay.store(g, row, q, scheme_coef(G * (float)scale, scheme));
                     }
                 }
