@@ -157,13 +157,15 @@ __device__ __forceinline__ float2 kc_expm1(float2 x) {
 // own slot; position 0 leaves the cells w < g to the previous pair (pair 0:
 // zeros); position TperR is the pair's tail (w < g), in slot 0 of the next
 // pair (after the last pair the slot has no owner and its other cells are
-// zeroed).
+// zeroed).  Virtual columns (in positions 0 and 1) are zero whatever the points: the
+// adjoint multiplies the first one with the previous pair's zero A, and a NaN or an
+// infinity must stay in the pair whose path holds it.
 template <int NG>
-__device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs, int TperR, int pos, int l,
+__device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs, int TperR, int NQV, int pos, int l,
                                          const float2 (&v)[NG][NG / 2]) {
     constexpr int SLOT = NG * NG, NH = NG / 2;
     float *dst = band + band_row(k * TperR + pos, l, NG, n_pairs * TperR + 1);   // (the tail: the next pair's slot 0)
-    if (pos > 0 && pos < TperR) {
+    if (pos > (NQV > 1) && pos < TperR) {
 #pragma unroll
         for (int i = 0; i < SLOT / 4; ++i) {
             const float2 u = v[2 * i / NH][2 * i % NH], t = v[(2 * i + 1) / NH][(2 * i + 1) % NH];
@@ -179,7 +181,7 @@ __device__ __forceinline__ void kc_store(float *band, int64_t k, int64_t n_pairs
         for (int g = 0; g < NG; ++g) {
             const float c = g < NH ? v[w][g % NH].x : v[w][g % NH].y;
             const int at = band_off(w * NG + 2 * (g % NH) + g / NH);
-            if (tail ? w < g : w >= g) dst[at] = c;
+            if (tail ? w < g : pos > 0 || w >= g) dst[at] = pos * NG + w - g < NQV ? 0.f : c;
             else if (zero) dst[at] = 0.f;
         }
 }
@@ -194,7 +196,7 @@ __device__ __forceinline__ void kc_put(const KcArgs &a, float2 (&v)[NG][NG / 2],
             for (int h = 0; h < NG / 2; ++h)
                 v[w][h] = make_float2(scheme_coef(v[w][h].x, a.src.scheme), scheme_coef(v[w][h].y, a.src.scheme));
     }
-    kc_store<NG>(a.band, k, a.n_pairs, a.TperR, pos, l, v);
+    kc_store<NG>(a.band, k, a.n_pairs, a.TperR, a.NQV, pos, l, v);
 }
 
 // Entry j of the staged column points as a pair (column, column - NG/2).
