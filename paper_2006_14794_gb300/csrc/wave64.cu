@@ -136,61 +136,67 @@ __device__ __forceinline__ void w64_stage(double *sm, const W64Shared &L, const 
     }
 }
 
-// |x| >= 2^e (or not a number), by its exponent bits: an FP64 compare would cost
-// an FP64 instruction.
-__device__ __forceinline__ bool w64_reaches(double x, int e) {
-    return (__double2hiint(x) & 0x7fffffff) >= (1023 + e) << 20;
-}
+// |x| by its exponent bits (a NaN above all): an FP64 compare would cost an FP64
+// instruction.
+__device__ __forceinline__ int w64_size(double x) { return __double2hiint(x) & 0x7fffffff; }
+constexpr int w64_pow2(int e) { return (1023 + e) << 20; }
 // kappa at the end of a step less kappa at its start: exponents e0, e1 and their
-// difference x as the step's own points give it (from a difference of 1 on, where
-// little cancels, the two ends are exact to their own size).
+// difference x (from a difference of 1 on, where little cancels, the two ends are
+// exact to their own size).
 __device__ __forceinline__ double w64_step(double e0, double e1, double x) {
-    return w64_reaches(x, 0) ? exp(e1) - exp(e0) : exp(e0) * expm1(x);
+    return w64_size(x) >= w64_pow2(0) ? exp(e1) - exp(e0) : exp(e0) * expm1(x);
 }
 // The second difference of kappa over the cell of points x, x + dx (channel
 // stride rs) and y, y + dy as the difference of two steps, along the side whose
-// kappa changes less from corner (p, q), every exponent from its own distance.
-// The product form kappa(p,q) (a b + (1 + a)(1 + b) e) is right where a, b and e
-// are of order one; beside a jump of several bandwidths e^A e^B cancels against
-// e^C (three corners near one another, the fourth five bandwidths off: 1e-9
-// relative, further off no digit is left) or overflows.  Against 80-bit
-// corners, 3 channels, points 0.1 to 10 bandwidths apart, steps of 0.01 to 60:
-// within 1.2e-13 of the value (of 0.001 for smaller ones), where the product form
-// is off by anything.
+// kappa changes less from corner (p, q).  E = -s |x - y|^2 and A, B, C as in
+// sigk_internal.cuh.  The product form kappa(p,q) (a b + (1 + a)(1 + b) e) is right
+// where a, b and e are of order one; beside a jump of several bandwidths e^A e^B
+// cancels against e^C (three corners near one another, the fourth five bandwidths
+// off: 1e-9 relative, further off no digit is left) or overflows.  The corners'
+// exponents are sums of these four, which leaves an error of their size times
+// 2^-53; from a size (that of the row's earlier cells too) of 32 on, and where a
+// corner's kappa counts or the sums are too large to tell, every exponent comes
+// from its own distance. 
 __device__ __noinline__ double w64_far_cell(const double *x, const double *dx, int rs, const double *y,
-                                            const double *dy, int d, double rbf_s) {
-    double uu = 0.0, ux = 0.0, uy = 0.0, xx = 0.0, yy = 0.0;
-    for (int k = 0; k < d; ++k) {
-        const double u = x[k * rs] - y[k], xv = dx[k * rs], yv = dy[k];
-        uu = fma(u, u, uu);
-        ux = fma(u, xv, ux);
-        uy = fma(u, yv, uy);
-        xx = fma(xv, xv, xx);
-        yy = fma(yv, yv, yy);
+                                            const double *dy, int d, double rbf_s, double E, double A, double B,
+                                            double C, int size) {
+    const bool rows = fabs(A) >= fabs(B);   // steps along x, at y_q and at y_{q+1}; else along y
+    double e0 = E, s0 = rows ? B : A, e1 = E + (rows ? A : B), s1 = s0 + C, f0 = e0 + s0, f1 = e1 + s1;
+    if (size >= w64_pow2(5) && (fmax(fmax(e0, e1), fmax(f0, f1)) > -16.0 || size >= w64_pow2(20))) {
+        e0 = e1 = f0 = f1 = 0.0;
+        double w0 = 0.0, w1 = 0.0, ee = 0.0;
+        for (int k = 0; k < d; ++k) {
+            const double u = x[k * rs] - y[k], xv = dx[k * rs], yv = dy[k];
+            const double e = rows ? xv : -yv, v = u + (rows ? -yv : xv);   // the step, and u at its other side
+            const double a = u + e, b = v + e;
+            e0 = fma(u, u, e0);
+            e1 = fma(v, v, e1);
+            f0 = fma(a, a, f0);
+            f1 = fma(b, b, f1);
+            w0 = fma(u, e, w0);
+            w1 = fma(v, e, w1);
+            ee = fma(e, e, ee);
+        }
+        e0 *= -rbf_s;
+        e1 *= -rbf_s;
+        f0 *= -rbf_s;
+        f1 *= -rbf_s;
+        s0 = -rbf_s * (2.0 * w0 + ee);
+        s1 = -rbf_s * (2.0 * w1 + ee);
     }
-    const double A = rbf_s * (2.0 * uy - yy), B = -rbf_s * (2.0 * ux + xx);
-    const bool rows = fabs(A) >= fabs(B);   // steps along x (e: of u), at y_q and at y_{q+1}; else along y
-    double n0 = 0.0, n1 = 0.0, n2 = 0.0, w = 0.0;
-    for (int k = 0; k < d; ++k) {
-        const double u = x[k * rs] - y[k], xv = dx[k * rs], yv = dy[k];
-        const double e = rows ? xv : -yv, v = u + (rows ? -yv : xv);
-        const double a = u + e, b = v + e;
-        n0 = fma(a, a, n0);
-        n1 = fma(v, v, n1);
-        n2 = fma(b, b, n2);
-        w = fma(v, e, w);
-    }
-    return w64_step(-rbf_s * n1, -rbf_s * n2, -rbf_s * (2.0 * w + (rows ? xx : yy))) -
-           w64_step(-rbf_s * uu, -rbf_s * n0, rows ? B : A);
+    return w64_step(e1, f1, s1) - w64_step(e0, f0, s0);
 }
 
 // The coefficients of local coarse rows P .. P + N - 1 at column q (in the
 // grid), the scheme's map applied.  With the RBF lift the second difference of
 // kappa (rbf_second_difference), what consecutive rows share carried down:
 // kappa(p+1, q) = kappa(p, q) (1 + b), expm1(A(p+1, q)) = a + e^A expm1(C).
-// Carried values keep their digits while the exponents stay below one: rows
-// with |A| or |B| of 1/2 or more, or C's that could add up to it, are formed one
-// by one (w64_far_cell).
+// The product form and the carried values keep their digits while the exponents
+// stay of order one: rows with |A| or |B| of 1 or more (a single cell: 2), or C's that
+// could add up to it, are formed one by one (w64_far_cell), their exponents carried.
+// Against 80-bit corners, 3 channels, points 0.1 to 10 bandwidths apart, steps of 0.01
+// to 60: within 3e-13 of the value (of 0.001 for smaller ones), where the product form
+// is off by anything.
 template <int N, bool RBF>
 __device__ __forceinline__ void w64_coefs(double (&c)[N], const double *sm, const W64Shared &L, int d, int nrows,
                                           int P, int q, double scale, double rbf_s, int scheme) {
@@ -226,19 +232,27 @@ __device__ __forceinline__ void w64_coefs(double (&c)[N], const double *sm, cons
             }
         }
         constexpr int LOGN = N == 1 ? 0 : N == 2 ? 1 : N <= 4 ? 2 : N <= 8 ? 3 : 4;
+        constexpr int FAR = N == 1 ? 1 : 0;   // 2^FAR: a single cell's 1 + a loses e^2, a carried one e a row
         static_assert(N <= 16, "LOGN");
-        const double A = rbf_s * (2.0 * uy - sm[L.norms + nrows + q]);
-        bool far = w64_reaches(A, -1);
+        double A = rbf_s * (2.0 * uy - sm[L.norms + nrows + q]);
+        bool far = w64_size(A) >= w64_pow2(FAR);
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             ux[i] = -rbf_s * (2.0 * ux[i] + sm[L.norms + P + i]);   // B
             g[i] = 2.0 * rbf_s * g[i];                               // C
-            far = far || w64_reaches(ux[i], -1) || w64_reaches(g[i], -1 - LOGN);
+            far = far || w64_size(ux[i]) >= w64_pow2(FAR) || w64_size(g[i]) >= w64_pow2(FAR - LOGN);
         }
         if (far) {
+            double E = -rbf_s * uu;
+            int size = w64_size(E);
 #pragma unroll
-            for (int i = 0; i < N; ++i)
-                c[i] = scheme_coef(w64_far_cell(x0 + i, dx + i, L.rs, y0, dy, d, rbf_s) * scale, scheme);
+            for (int i = 0; i < N; ++i) {
+                size = max(max(size, w64_size(A)), max(w64_size(ux[i]), w64_size(g[i])));
+                c[i] = scheme_coef(w64_far_cell(x0 + i, dx + i, L.rs, y0, dy, d, rbf_s, E, A, ux[i], g[i], size) * scale,
+                                   scheme);
+                E += ux[i];
+                A += g[i];
+            }
             return;
         }
         double kap = exp(-rbf_s * uu), a = expm1(A);
