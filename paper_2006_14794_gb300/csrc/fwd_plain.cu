@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(PLAIN_THREADS) plain_kernel(PairSrc src, int64
     const T scale = (T)0.5 / (T)(1LL << (2 * lam));
     const T rbf_s = (T)(0.5 / (src.sigma * src.sigma));
     for (int64_t k = blockIdx.x; k < n_pairs; k += gridDim.x) {
-        const PairRef pr = pair_ref<true>(src, k);
+        const PairRef pr = pair_ref(src, k);
         if (pr.la < 2 || pr.lb < 2) {
             if (threadIdx.x == 0) {
                 out[pr.out0] = (T)1;
