@@ -72,6 +72,13 @@ __host__ __device__ constexpr bool w64_mform(int R, int lam) { return lam >= 2 &
 // odd strides: staged columns one column apart, and rows one channel apart, hit distinct banks
 __host__ __device__ inline int w64_odd(int64_t v) { return (int)(v | 1); }
 __host__ __device__ inline int w64_nmac(int ny, int lam) { return ((ny << lam) + 31 + W64_MAC - 1) / W64_MAC; }
+// Macro-steps before the first lane with a real row enters the grid: nothing to do,
+// as the virtual rows above stay at K = 1 (less than 31 steps, so that a first warp
+// without real rows still hands on all of its columns).
+__host__ __device__ inline int w64_first(int vrows, int R, int lam) {
+    const int m = (vrows << lam) / R / W64_MAC;
+    return m < 3 ? m : 3;
+}
 
 // Shared memory of a block, in doubles: row increments (scaled) [d][coarse
 // rows, odd], column increments [ny][d, odd], with the RBF lift the first
@@ -267,23 +274,30 @@ __device__ __forceinline__ void w64_coefs(double (&c)[N], const double *sm, cons
     }
 }
 
-// All coefficients of nrows padded coarse rows into dst[q][P] (row stride ld):
-// a warp takes 32 rows and four columns (RBF: one) at a time.
+// All coefficients of nrows padded coarse rows, the first `virt` of them virtual,
+// into dst[q][P] (row stride ld): a warp takes 32 rows and four columns at a time,
+// with the lift (whose cells cost several hundred FP64 operations) 32 real cells in
+// the order of dst.
 template <bool RBF>
 __device__ __forceinline__ void w64_all_coefs(double *dst, int64_t ld, const double *sm, const W64Shared &L, int d,
-                                              int nrows, int ny, double scale, double rbf_s, int scheme) {
-    constexpr int QB = RBF ? 1 : 4;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int rb = (nrows + 31) / 32, qb = (ny + QB - 1) / QB;
-    for (int u = threadIdx.x >> 5; u < rb * qb; u += nw) {
-        const int r = u / qb, q0 = (u - r * qb) * QB;
-        const int P = r * 32 + lane;
-        const int Pc = P < nrows ? P : nrows - 1;
-        if constexpr (RBF) {
+                                              int nrows, int virt, int ny, double scale, double rbf_s, int scheme) {
+    if constexpr (RBF) {
+        const int real = nrows - virt;
+        for (int v = threadIdx.x; v < virt * ny; v += blockDim.x) dst[v / virt * ld + v % virt] = 0.0;
+        for (int v = threadIdx.x; v < real * ny; v += blockDim.x) {
+            const int q = v / real, P = virt + v - q * real;
             double c[1];
-            w64_coefs<1, true>(c, sm, L, d, nrows, Pc, q0, scale, rbf_s, scheme);
-            if (P < nrows) dst[q0 * ld + P] = c[0];
-        } else {
+            w64_coefs<1, true>(c, sm, L, d, nrows, P, q, scale, rbf_s, scheme);
+            dst[q * ld + P] = c[0];
+        }
+    } else {
+        constexpr int QB = 4;
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        const int rb = (nrows + 31) / 32, qb = (ny + QB - 1) / QB;
+        for (int u = threadIdx.x >> 5; u < rb * qb; u += nw) {
+            const int r = u / qb, q0 = (u - r * qb) * QB;
+            const int P = r * 32 + lane;
+            const int Pc = P < nrows ? P : nrows - 1;
             const double *dx = sm + Pc;
             const double *dy[QB];
             double g[QB];
@@ -325,7 +339,11 @@ __global__ void __launch_bounds__(W64_MAX_WARPS * 32) wave64_kernel(Wave64Args a
     const PairRef pr = pair_ref<true>(a.src, k);
     w64_stage<RBF>(w64_sm, L, (const double *)a.src.A + pr.a_row0 * a.src.d,
                    (const double *)a.src.B + pr.b_row0 * a.src.d, d, a.nx, ny, a.vrows, rank * nrows, nrows, a.scale);
-    if constexpr (PRE) w64_all_coefs<RBF>(cf, L.rs, w64_sm, L, d, nrows, ny, a.scale, a.rbf_s, a.src.scheme);
+    if constexpr (PRE) {
+        const int virt = a.vrows - rank * nrows;   // of the block's rows
+        w64_all_coefs<RBF>(cf, L.rs, w64_sm, L, d, nrows, virt < 0 ? 0 : virt < nrows ? virt : nrows, ny, a.scale,
+                           a.rbf_s, a.src.scheme);
+    }
     auto barrier = [&]() {
         if (C > 1) cg::this_cluster().sync();
         else __syncthreads();
@@ -352,7 +370,7 @@ __global__ void __launch_bounds__(W64_MAX_WARPS * 32) wave64_kernel(Wave64Args a
     const int ol = lane & (S - 1), lq = lane >> LAM;
     const int nmac = w64_nmac(ny, LAM), total = nmac + W64_LAG / W64_MAC * (W - 1);
     const int tend = (ny << LAM) + 30;   // lane 31's step on the last column
-    for (int m = 0; m < total; ++m) {
+    for (int m = w64_first(a.vrows, R, LAM); m < total; ++m) {
         const int mm = m - W64_LAG / W64_MAC * g;
         if (mine && mm >= 0 && mm < nmac) {
 #pragma unroll 1
@@ -469,7 +487,7 @@ __global__ void __launch_bounds__(W64B_MAX_WARPS * 32, 2) wave64_bwd_kernel(Wave
     double *Cm = a.ws + (int64_t)blockIdx.x * a.slot;
     double *Sm = Cm + sl.coef, *Gb = Sm + sl.sums;
     const int nmac = w64_nmac(ny, LAM), T = W64_MAC * nmac;
-    const int total = nmac + W64_LAG / W64_MAC * (W - 1);
+    const int total = nmac + W64_LAG / W64_MAC * (W - 1), m0 = w64_first(a.vrows, R, LAM);
     const int ol = lane & (S - 1), lq = lane >> LAM;
     const bool mine = g < W;
     const int P = ((g * 32 + lane) * R) >> LAM;
@@ -490,7 +508,7 @@ __global__ void __launch_bounds__(W64B_MAX_WARPS * 32, 2) wave64_bwd_kernel(Wave
         __syncthreads();   // the shared arrays and the slot are free again
         // 1. increments and coefficients
         w64_stage<RBF>(w64_sm, L, x, y, d, nx, ny, a.vrows, 0, nrows, a.scale);
-        w64_all_coefs<RBF>(Cm, nrows, w64_sm, L, d, nrows, ny, a.scale, a.rbf_s, a.src.scheme);
+        w64_all_coefs<RBF>(Cm, nrows, w64_sm, L, d, nrows, a.vrows, ny, a.scale, a.rbf_s, a.src.scheme);
         __syncthreads();
         // 2. forward, keeping the sums
         {
@@ -499,9 +517,9 @@ __global__ void __launch_bounds__(W64B_MAX_WARPS * 32, 2) wave64_bwd_kernel(Wave
             for (int r = 0; r < R; ++r) K[r] = 1.0;
 #pragma unroll
             for (int i = 0; i < NG; ++i) chi[i] = 0.0;
-            window(cnx, 0);
+            window(cnx, g == 0 ? (m0 * W64_MAC) >> LAM : 0);   // the warp's first one
             double kout = 1.0, qout = 0.0;
-            for (int m = 0; m < total; ++m) {
+            for (int m = m0; m < total; ++m) {
                 const int mm = m - W64_LAG / W64_MAC * g;
                 if (mine && mm >= 0 && mm < nmac) {
 #pragma unroll 1
@@ -563,7 +581,7 @@ __global__ void __launch_bounds__(W64B_MAX_WARPS * 32, 2) wave64_bwd_kernel(Wave
             window(cpre, (T >> LAM) - 2);
             double vout = 0.0;
             const int Nj = ny << LAM;
-            for (int m = 0; m < total; ++m) {
+            for (int m = 0; m < total - m0; ++m) {
                 const int mm = nmac - 1 - (m - W64_LAG / W64_MAC * (W - 1 - g));
                 if (mine && mm >= 0 && mm < nmac) {
 #pragma unroll 1
@@ -771,7 +789,8 @@ bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kern
             const double load = (double)(n * C) / sms;             // blocks a SM has to run,
             const double on = load < 1 ? 1 : (load < bps ? load : (double)bps);   // at once,
             const double waves = load <= bps ? 1 : load / bps;     // and how often
-            const double steps = (double)W64_MAC * w64_nmac(ny, lam) + (double)W64_LAG * (W - 1);
+            const double steps = (double)W64_MAC * (w64_nmac(ny, lam) - w64_first(W * pw - nx, R, lam)) +
+                                 (double)W64_LAG * (W - 1);
             double ops = (mf ? 2.0 : 3.0) * R + (mf ? 4.0 * ng / (1 << lam) : 0.0), first = 0.0;
             if (pre) first = 19.2 * on * (double)(wpc * pw) * ny / 32 * (w64_coef_ops((double)d, rbf) + 1);
             else ops += ng * (rbf ? 3.0 * d + 140.0 : (double)d) / (1 << lam);
@@ -845,12 +864,15 @@ bool wave64_bwd_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int 
     const int sms = sm_count();
     double best = 1e300;
     p.lam = lam;
-    auto consider = [&](int R) {
+    // FP64 warp operations besides the sweeps, spread over all warps: coefficients and
+    // chain rule
+    const double cells = (double)nx * ny / 32, dd = (double)d;
+    const double around = rbf ? cells * (w64_coef_ops(dd, true) + 6.0 * dd + 60.0) : cells * 3.0 * dd;
+    auto consider = [&](int R, int threads) {
         const int pw = w64_coarse(R, lam), W = (nx + pw - 1) / pw;
-        if (W > W64B_MAX_WARPS) return;
+        if (W * 32 > threads) return;
         const int64_t bytes = 8 * w64_shared(W * pw, W, ny, d, rbf, false).total;
         if (bytes > W64_SMEM) return;
-        const int threads = W64B_MAX_WARPS * 32;
         int64_t bps = (228 * 1024) / (bytes + 1024);
         if (bps > 65536 / (threads * 128)) bps = 65536 / (threads * 128);
         if (bps < 1) return;
@@ -860,17 +882,24 @@ bool wave64_bwd_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int 
         if (grid > n) grid = n;
         while (grid > 1 && grid * slot * 8 > W64_BWD_WS_CAP) grid = (grid + 1) / 2;
         if (grid * slot * 8 > 4 * W64_BWD_WS_CAP) return;
-        const double on = grid <= sms ? 1.0 : (double)grid / sms, waves = (double)n / grid > 1 ? (double)n / grid : 1.0;
-        const double steps = (double)W64_MAC * w64_nmac(ny, lam) + (double)W64_LAG * (W - 1);
-        const double cost = waves * (w64_cycles(steps, 3.0 * R, on * W) + w64_cycles(steps, 4.0 * R, on * W) +
-                                     12.0 * (W > 1) * steps);
+        const double on = (double)((grid + sms - 1) / sms), waves = (double)n / grid > 1 ? (double)n / grid : 1.0;
+        const double steps = (double)W64_MAC * (w64_nmac(ny, lam) - w64_first(W * pw - nx, R, lam)) +
+                             (double)W64_LAG * (W - 1);
+        const double own = 64.5 * 32 / threads, shared = 19.2 * on;
+        const double cost = waves * (around * (own > shared ? own : shared) + w64_cycles(steps, 3.0 * R, on * W) +
+                                     w64_cycles(steps, 4.0 * R, on * W) + 12.0 * (W > 1) * steps);
         if (cost < best) {
             best = cost;
             p.R = R; p.W = W; p.threads = threads; p.smem = (int)bytes; p.slot = slot; p.grid = grid;
             p.vrows = W * pw - nx;
         }
     };
-#define X(r, l) if (l == lam) consider(r);
+    // Fewer warps a block, and more blocks a SM, for pairs with less than two coarse cells a
+    // thread of a full one (1310 pairs of 5 and 11 points, d = 9: 149 -> 62 us, 100 plain);
+    // the slots of more blocks at once fall out of the L1 otherwise (801 pairs of 31 and
+    // 242 points with the lift: 2.98 ms in full blocks, 3.49 in smaller ones).
+    const int least = (int64_t)nx * ny <= 64 * W64B_MAX_WARPS ? 64 : 32 * W64B_MAX_WARPS;
+#define X(r, l) if (l == lam) for (int t = 32 * W64B_MAX_WARPS; t >= least; t /= 2) consider(r, t);
     SIGK_W64_BWD(X)
 #undef X
     return best < 1e300;

@@ -41,3 +41,42 @@ def test_two_plain_blocks_share_a_multiprocessor():
     one = us(lambda: sigk.pairs(X[:sms], Y[:sms], 0, rec=sigk.REC_PLAIN))
     two = us(lambda: sigk.pairs(X, Y, 0, rec=sigk.REC_PLAIN))
     assert two <= 1.5 * one
+
+
+# (pairs, L, M, d, dyadic order): one and two coarse rows, short sides, tiny grids
+SHORT = [(1310, 5, 11, 9, 0), (1316, 2, 2, 2, 1), (628, 25, 11, 18, 0), (217, 83, 7, 17, 0), (1457, 4, 3, 32, 1)]
+
+
+@pytest.mark.parametrize("kernel", ["linear", "rbf"])
+@pytest.mark.parametrize("B,L,M,d,lam", SHORT)
+def test_short_paths_backward(B, L, M, d, lam, kernel):
+    need_gpu()
+    X, Y = paths(73 + L, B, L, d), paths(74 + M, B, M, d)
+    g = torch.ones(B, dtype=torch.float64, device="cuda")
+    v = sigk.Variant(static_kernel=kernel)
+    default = us(lambda: sigk.pairs_backward(g, X, Y, lam, variant=v))
+    plain = us(lambda: sigk.pairs_backward(g, X, Y, lam, variant=v, rec=sigk.REC_PLAIN))
+    assert default <= 1.25 * plain
+
+
+# coarse rows around the steps that a sweep without virtual rows leaves out (8, 16, 24 lanes)
+@pytest.mark.parametrize("kernel", ["linear", "rbf"])
+@pytest.mark.parametrize("lam", [0, 1, 2, 3])
+@pytest.mark.parametrize("nx", [1, 4, 7, 8, 9, 16, 24, 25, 31, 32, 33, 40, 70])
+def test_virtual_rows_are_left_out(nx, lam, kernel):
+    need_gpu()
+    kw = dict(static_kernel=kernel, sigma=1.0)
+    rng = np.random.default_rng(nx)
+    for B, ny in ((3, nx), (5, nx + 30), (400, nx + 3)):
+        if B > 5 and nx > 33:
+            continue
+        X = inputs.random_paths(75 + nx, B, nx + 1, 3, time_channel=True)
+        Y = inputs.random_paths(76 + ny, B, ny + 1, 3, time_channel=True)
+        Xd, Yd = to_dev(X, torch.float64), to_dev(Y, torch.float64)
+        v = sigk.Variant(**kw)
+        assert rel_err(sigk.pairs(Xd, Yd, lam, variant=v).cpu().numpy(), oracle.pairs(X, Y, lam, **kw)) <= 1e-11
+        g = rng.normal(size=B)
+        n = min(B, 8)   # the oracle's share
+        got = sigk.pairs_backward(to_dev(g, torch.float64), Xd, Yd, lam, variant=v)
+        for a, b in zip(got, oracle.pairs_grad(X[:n], Y[:n], lam, g[:n], **kw)):
+            assert np.max(np.abs(a[:n].cpu().numpy() - b)) <= 1e-10 * np.max(np.abs(b))
