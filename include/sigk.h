@@ -79,7 +79,8 @@ typedef enum { SIGK_F32 = 0, SIGK_F64 = 1 } sigk_dtype;   /* storage AND arithme
  *  AUTO: CHAIN for f32 (PLAIN when CHAIN has no instance).  For f64 pairs of
  *    uniform lengths and Grams the register wavefront with one cluster of
  *    blocks per pair (dyadic_order <= 3 and increments that fit a block's
- *    shared memory; forward and backward), else PLAIN. */
+ *    shared memory; forward and backward), else PLAIN, which also takes the
+ *    forward calls whose increments fill a multiprocessor's shared memory. */
 typedef enum {
     SIGK_REC_AUTO = 0, SIGK_REC_CHAIN = 1, SIGK_REC_PLAIN = 2, SIGK_REC_STRIP = 3, SIGK_REC_BAND = 4
 } sigk_rec;

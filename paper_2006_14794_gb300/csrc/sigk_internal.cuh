@@ -78,8 +78,14 @@ __device__ __forceinline__ float rbf_second_difference(float uu, float ux, float
 }
 __device__ __forceinline__ double rbf_second_difference(double uu, double ux, double uy, double xy,
                                                         double nx, double ny, double s) {
-    const double A = s * (2.0 * uy - ny), B = -s * (2.0 * ux + nx), C = 2.0 * s * xy;
-    return exp(-s * uu) * (expm1(A) * expm1(B) + exp(A + B) * expm1(C));
+    const double A = s * (2.0 * uy - ny), B = -s * (2.0 * ux + nx), C = 2.0 * s * xy, E = -s * uu;
+    if (fmax(fmax(fabs(A), fabs(B)), fabs(C)) < 2.0) return exp(E) * (expm1(A) * expm1(B) + exp(A + B) * expm1(C));
+    // beside a jump of several bandwidths that product overflows or cancels: the
+    // difference of the two steps along the side that changes less
+    const bool rows = fabs(A) >= fabs(B);
+    const double v = rows ? B : A, E1 = E + (rows ? A : B), v1 = v + C;
+    const double far = fabs(v1) < 1.0 ? exp(E1) * expm1(v1) : exp(E1 + v1) - exp(E1);
+    return far - (fabs(v) < 1.0 ? exp(E) * expm1(v) : exp(E + v) - exp(E));
 }
 
 // dc'/dc of that map, written through c' = c / (1 - c/2): (1 + c'/2)^2.  The

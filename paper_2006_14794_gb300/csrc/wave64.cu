@@ -47,6 +47,7 @@
 // and 16 paths of 64 points, d = 32, order 1: 5.47 -> 1.03 ms (1.78 with the
 // coefficients formed by the sweep warps alone).
 #include <cooperative_groups.h>
+#include <math.h>
 #include <string.h>
 
 #include "sigk_internal.cuh"
@@ -755,15 +756,28 @@ double w64_cycles(double steps, double ops, double warps) {
     const double share = warps * (19.2 / 64.5);
     return steps * (64.5 * ops * (share > 1.0 ? share : 1.0) + 60.0);
 }
-// FP64 operations of one coarse cell's coefficient (RBF: three special functions)
+// FP64 operations of one coarse cell's coefficient (RBF: four special functions)
 double w64_coef_ops(double d, bool rbf) { return rbf ? 5.0 * d + 200.0 : d; }
+// Cycles of the plain sweep (fwd_plain.cu) on the same pairs: two blocks a SM, a
+// barrier per anti-diagonal, each refined cell with its coefficient anew (with the
+// lift at order 0 a diagonal takes 665 operations' time at d = 63, 559 at d = 50).
+double w64_plain_cycles(int64_t n, double nx, double ny, double d, int lam, bool rbf, int sms) {
+    const double Ni = nx * (1 << lam), warps = Ni / 32 > 1 ? Ni / 32 : 1.0;
+    const double on = n > sms ? 2.0 : 1.0, waves = ceil((double)n / (sms * on));
+    const double share = warps * on * (19.2 / 64.5);
+    return waves * (Ni + ny * (1 << lam)) * (64.5 * (rbf ? 9.0 * d + 100.0 : 3.0 * d + 10.0) * (share > 1.0 ? share : 1.0));
+}
 
 }  // namespace
 
 // The cheapest of the instances and cluster shapes for these sizes by
 // w64_cycles: one warp a pair where the pairs alone fill the partitions (least
 // fill and drain), more warps, blocks and helpers a pair the fewer pairs there
-// are.  False where the staged increments fit no block.
+// are.  False where the staged increments fit no block, and where they leave room
+// for one or two warps a SM, which form their coefficients alone, and the plain sweep
+// with its two pairs a SM is faster (195 pairs of 24 and 161 points, d = 63, order 0,
+// with the lift: 5.6 ms against 4.1; 318 of 210 and 227, d = 51: 146 against 26; for
+// 693 random shapes the default was then slower than plain by 15 % in one).
 bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kernel, Wave64Plan &p) {
     if (La < 2 || Lb < 2 || lam < 0 || lam > 3 || La > Lb) return false;
     // longer paths are refused by the plain sweep, which would take them otherwise
@@ -771,7 +785,7 @@ bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kern
     const bool rbf = kernel == SIGK_KERNEL_RBF;
     const int nx = (int)(La - 1), ny = (int)(Lb - 1);
     const int sms = sm_count();
-    double best = 1e300;
+    double best = 1e300, full = 0.0;   // (full: of lone warps, in whole waves)
     p.lam = lam;
     auto consider = [&](int R, bool pre) {
         const int pw = w64_coarse(R, lam), wt = (nx + pw - 1) / pw, ng = w64_ng(R, lam);
@@ -797,6 +811,8 @@ bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kern
             const double cost = waves * (first + w64_cycles(steps, ops, on * wpc) + (C > 1 ? 30.0 : 6.0) * (W > 1) * steps);
             if (cost < best) {
                 best = cost;
+                full = !pre && bps * wpc <= 2 ? cost / waves * ceil(waves) : 0.0;
+                if (rbf && ng == 1) full *= (5.0 * d + 135.0) / (3.0 * d + 140.0);
                 p.R = R; p.pre = pre; p.wpc = wpc; p.cluster = C; p.threads = threads; p.smem = (int)bytes;
                 p.vrows = W * pw - nx;
             }
@@ -808,7 +824,7 @@ bool wave64_plan(int64_t n, int64_t La, int64_t Lb, int64_t d, int lam, int kern
 #define X(r, l) if (l == lam) consider(r, true);
     SIGK_W64_PRE(X)
 #undef X
-    return best < 1e300;
+    return best < 1e300 && full <= 1.1 * w64_plain_cycles(n, nx, ny, (double)d, lam, rbf, sms);
 }
 
 cudaError_t launch_wave64(const PairSrc &src, const Wave64Plan &p, int64_t n, double *out, cudaStream_t st) {

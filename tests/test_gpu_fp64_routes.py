@@ -80,3 +80,38 @@ def test_virtual_rows_are_left_out(nx, lam, kernel):
         got = sigk.pairs_backward(to_dev(g, torch.float64), Xd, Yd, lam, variant=v)
         for a, b in zip(got, oracle.pairs_grad(X[:n], Y[:n], lam, g[:n], **kw)):
             assert np.max(np.abs(a[:n].cpu().numpy() - b)) <= 1e-10 * np.max(np.abs(b))
+
+
+# increments that leave a multiprocessor one block of one warp, with the lift at order 0
+WIDE = [(195, 24, 161, 63, 0), (1200, 24, 161, 63, 0), (300, 60, 200, 50, 0), (150, 24, 161, 63, 0), (300, 20, 120, 90, 1)]
+
+
+@pytest.mark.parametrize("kernel", ["linear", "rbf"])
+@pytest.mark.parametrize("B,L,M,d,lam", WIDE)
+def test_wide_paths_forward(B, L, M, d, lam, kernel):
+    need_gpu()
+    X, Y = paths(77 + L, B, L, d), paths(78 + M, B, M, d)
+    v = sigk.Variant(static_kernel=kernel)
+    default = us(lambda: sigk.pairs(X, Y, lam, variant=v), 1)
+    plain = us(lambda: sigk.pairs(X, Y, lam, variant=v, rec=sigk.REC_PLAIN), 1)
+    assert default <= 1.25 * plain
+    n = 4
+    want = oracle.pairs(X[:n].cpu().numpy(), Y[:n].cpu().numpy(), lam, static_kernel=kernel, sigma=1.0)
+    assert rel_err(sigk.pairs(X, Y, lam, variant=v)[:n].cpu().numpy(), want) <= 1e-11
+
+
+@pytest.mark.parametrize("rec", [sigk.REC_PLAIN, sigk.REC_CHAIN])
+@pytest.mark.parametrize("size", [6.0, 9.0, 30.0])
+def test_jumps_on_the_general_routes(size, rec):
+    """A point of X and of Y some bandwidths off, apart and together: plain and strip sweeps."""
+    need_gpu()
+    kw = dict(static_kernel="rbf", sigma=1.0)
+    X = inputs.random_paths(79, 6, 30, 3, time_channel=True) + 0.5
+    Y = inputs.random_paths(80, 6, 33, 3, time_channel=True) + 0.5
+    X[:3, 11] += size / 3 ** 0.5
+    Y[:3, 20] -= size / 3 ** 0.5
+    X[3:, 11:] += size / 3 ** 0.5
+    Y[3:, 20:] += size / 3 ** 0.5
+    got = sigk.pairs(to_dev(X, torch.float64), to_dev(Y, torch.float64), 1, rec=rec, variant=sigk.Variant(**kw))
+    k, nodes = oracle.pairs_surface(X, Y, 1, **kw)
+    assert np.max(np.abs(got.cpu().numpy() - k) / np.abs(nodes).max(axis=(1, 2))) <= 1e-11
