@@ -497,7 +497,7 @@ template <int NG>
 cudaError_t launch_coef_tc5(const BandCoefArgs &a, int sms, int *status, cudaStream_t st) {
     const int smem = bt5_smem_bytes(a.src.d);
     auto kern = band_coef_tc5_kernel<NG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     int64_t grid = sms;
     if (grid > a.n_pairs) grid = a.n_pairs;

@@ -612,22 +612,22 @@ cudaError_t launch(const KcArgs &a0, int sms, cudaStream_t st) {
     auto share = [&](int most) {
         a.tiles = (npos + most - 1) / most;
         a.tp = ((npos + a.tiles - 1) / a.tiles + Sh::NP - 1) / Sh::NP * Sh::NP;
-        return (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch) <= 226 * 1024;
+        return (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch) <= SMEM_LIMIT;
     };
     for (int most = a.chunks > 1 ? Sh::TILEC : Sh::TILE; !share(most); most -= Sh::GP) {}
     // a row path's channels all stay where they fit (two chunks do)
     a.xch = d;
     int smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, nch);
-    if (d <= 4 * KC_CH && (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d) <= 226 * 1024)
+    if (d <= 4 * KC_CH && (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d) <= SMEM_LIMIT)
         smem = (int)sizeof(float) * kc_smem_floats<NG, RBF>(a.tp, nch, d);
     else
         a.xch = nch;
     const int items = (a.tp + Sh::GP - 1) / Sh::GP * (32 / Sh::LW);
-    const int most = RBF && NG < 8 && smem <= 113 * 1024 ? Sh::WARPS / 2 : Sh::WARPS;
+    const int most = RBF && NG < 8 && smem <= SMEM_LIMIT / 2 ? Sh::WARPS / 2 : Sh::WARPS;
     a.passes = a.chunks > 1 ? 1 : (items + most - 1) / most;
     const int warps = (items + a.passes - 1) / a.passes;
     auto go = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem)) != cudaSuccess) return e;

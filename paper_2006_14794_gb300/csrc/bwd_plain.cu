@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(BWD_THREADS) bwd_plain_kernel(BwdArgs a) {
 template <typename T, bool QF>
 int grid_of(int64_t n_pairs, int64_t smem) {
     auto kern = bwd_plain_kernel<T, QF>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
         cudaSuccess)
         return 0;
     int dev = 0, sms = 0, per_sm = 0;

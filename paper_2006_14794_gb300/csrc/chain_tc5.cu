@@ -348,7 +348,7 @@ template <int NS, int P>
 cudaError_t cg_launch(const CgArgs &a, int64_t grid, cudaStream_t st) {
     auto kern = chain_gemm_tc5_kernel<CG_PARTS, NS, P>;
     const int smem = cg_smem_bytes<CG_PARTS, NS, P>(a.NP);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, CG_T, smem, st>>>(a);
     return cudaGetLastError();

@@ -318,8 +318,7 @@ cudaError_t launch_one(const ChainArgs &args, const ChainPlan &p, cudaStream_t s
     auto kern = args.sband ? chain_f32_kernel<R, LAM, D4, MINB, false, true>
                            : args.src.scheme == SIGK_SCHEME_IMPLICIT ? chain_f32_kernel<R, LAM, D4, MINB, true>
                                                                      : chain_f32_kernel<R, LAM, D4, MINB, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         p.smem_bytes);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     kern<<<p.grid, CHAIN_WARPS * 32, p.smem_bytes, st>>>(args);
     return cudaGetLastError();
@@ -329,7 +328,7 @@ template <int R, int LAM, int D4, int MINB>
 int occupancy(int smem) {
     int nb = 0;
     auto kern = chain_f32_kernel<R, LAM, D4, MINB, false>;   // the implicit instance has the same resources
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT) != cudaSuccess)
         return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, CHAIN_WARPS * 32, smem) != cudaSuccess)
         return 0;

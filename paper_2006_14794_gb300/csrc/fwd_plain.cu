@@ -157,7 +157,7 @@ cudaError_t launch_plain_t(const PairSrc &src, int64_t n_pairs, int lam, T *out,
     const int64_t smem = (QF ? 4 : 3) * W * (int64_t)sizeof(T);
     if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
     auto kern = plain_kernel<T, QF>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);

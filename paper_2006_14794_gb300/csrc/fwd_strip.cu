@@ -1957,7 +1957,7 @@ static cudaError_t launch_coef(const PairSrc &src, const PairPlan *plan, int64_t
     if (tc5) {
         const int smem = tc5_smem_bytes(src.d);
         auto tk = coef_tc5_kernel<R, LAM>;
-        if ((e = cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT)) != cudaSuccess)
             return e;
         tk<<<sms, TC5_T, smem, st>>>(src, plan, n, totals, (const float *)incA, (const float *)incB,
                                      (float *)cbuf, status, 1LL << 26);
@@ -1968,7 +1968,7 @@ static cudaError_t launch_coef(const PairSrc &src, const PairPlan *plan, int64_t
         const int XS = tc_stride(src.d);
         const int smem = (4 * 64 * XS + 64 * TC_CS) * 4;
         auto tk = coef_tc_kernel<R, LAM>;
-        if ((e = cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT)) != cudaSuccess)
             return e;
         tk<<<sms * 2, 256, smem, st>>>(src, plan, n, totals, (const float *)incA, (const float *)incB,
                                        (float *)cbuf);
@@ -1977,7 +1977,7 @@ static cudaError_t launch_coef(const PairSrc &src, const PairPlan *plan, int64_t
     const int D4 = (int)((src.d + 3) / 4);
     const int smem = (GT + 2 * GT - 1) * (D4 | 1) * 4 * (int)sizeof(T);
     auto ck = coef_kernel<T, R, LAM>;
-    if ((e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT)) != cudaSuccess)
         return e;
     ck<<<sms * 4, 256, smem, st>>>(src, plan, n, totals, incA, incB, cbuf);
     return cudaGetLastError();

@@ -9,6 +9,12 @@ namespace sigk {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// The dynamic shared memory that a kernel may use is a setting of the kernel, not of
+// the call, so kernels whose need depends on the shape are all set to the same limit
+// (1 KB is left for static shared memory): a thread with a smaller shape cannot lower
+// it between another thread's setting and its launch.
+constexpr int SMEM_LIMIT = 226 * 1024;
+
 // How a flat pair index maps to (row path, column path, output slots).
 // The grid's rows refine the "A" path and its columns the "B" path.
 enum PairMode { PM_PAIRS = 0, PM_GRAM = 1, PM_GRAM_SYM = 2, PM_VARLEN = 3 };

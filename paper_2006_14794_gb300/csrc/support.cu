@@ -92,7 +92,7 @@ static cudaError_t launch_support_t(const T *K, const T *alpha, T *beta, int64_t
     const bool ks = base + N * N * (int64_t)sizeof(T) <= SR_SMEM;
     const int smem = (int)(ks ? base + N * N * (int64_t)sizeof(T) : base);
     auto k = ks ? support_kernel<T, true> : support_kernel<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     // a warp per Gram row up to 32 warps: fewer warps at a barrier for small N
     const int threads = (int)(N < 32 ? 32 * N : SR_THREADS);

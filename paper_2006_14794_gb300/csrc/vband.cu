@@ -745,7 +745,7 @@ template <int NG, int WQ, int HB>
 cudaError_t vb_launch_coef_pair(const VbArgs &a, int cls, int dc, int tmax, int sms, cudaStream_t st) {
     auto kern = vb_coef_pair_kernel<NG, WQ, HB>;
     const int smem = (int)sizeof(float) * dc * (vb_xstride<NG>() + vb_ystride(tmax, NG));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, VB_CT, smem)) != cudaSuccess) return e;
@@ -758,7 +758,7 @@ template <int NG, int WQ>
 cudaError_t vb_launch_coef(const VbArgs &a, int cls, int dc, int tmax, int sms, cudaStream_t st) {
     auto kern = vb_coef_kernel<NG, WQ>;
     const int smem = (int)sizeof(float) * dc * (vb_xstride<NG>() + vb_ystride(tmax, NG));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, VB_CT, smem)) != cudaSuccess) return e;

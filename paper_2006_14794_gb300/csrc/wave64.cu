@@ -853,7 +853,7 @@ cudaError_t launch_wave64(const PairSrc &src, const Wave64Plan &p, int64_t n, do
     cfg.attrs = &at;
     cfg.numAttrs = p.cluster > 1 ? 1 : 0;
     auto go = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
         return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, kern, a);
     };
     const bool rbf = src.kernel == SIGK_KERNEL_RBF;
@@ -939,7 +939,7 @@ cudaError_t launch_wave64_bwd(const PairSrc &src, const Wave64BwdPlan &p, int64_
     a.scale = 0.5 / (double)(1 << (2 * p.lam));
     a.rbf_s = 0.5 / (src.sigma * src.sigma);
     auto go = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
         if (e != cudaSuccess) return e;
         kern<<<(int)p.grid, p.threads, p.smem, st>>>(a);
         return cudaGetLastError();
