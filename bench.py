@@ -449,7 +449,7 @@ def _workload(name, batch=0, cache=None):
         es = 8 if f64 else 4
         return dict(
             desc="Gram 8x8, L=M=32, d=3 (time + 2 walks), dyadic order 1, plus 8 straight-line pairs, %s"
-                 % ("fp64 (register wavefront, the printed scheme)" if f64 else "fp32 (chained register sweep)"),
+                 % ("fp64 (register wavefront, difference form)" if f64 else "fp32 (chained register sweep)"),
             dtype="f64" if f64 else "f32", step=step, cells=cells, pairs=72,
             flop=3 * cells + 2 * 3 * coarse,
             kernels="wave64_kernel" if f64 else "chain_f32_kernel",

@@ -141,8 +141,9 @@ __device__ __forceinline__ void kc_cols(float2 (&v)[N], const float2 *r) {
 
 __device__ __forceinline__ float2 kc2(float v) { return make_float2(v, v); }
 // e^x - 1 of two values, |x| <= KC_CARRY / 2^(8 - D) or so: the Taylor series
-// through x^D / D!, whose truncation x^D / (D + 1)! is below 3e-9 of the value
-// for D = 8 and |x| <= 1/2, D = 7 and 1/4, D = 6 and 1/8, D = 5 and 1/16.
+// through x^D / D!, whose truncation is x^D / (D + 1)! of the value: 1.1e-8 for
+// D = 8 and |x| <= 1/2 (a fifth of a rounding), below 2e-9 for D = 7 and 1/4, D = 6
+// and 1/8, D = 5 and 1/16.
 template <int D>
 __device__ __forceinline__ float2 kc_expm1(float2 x) {
     constexpr float F[9] = {1.f, 1.f, 1.f / 2.f, 1.f / 6.f, 1.f / 24.f, 1.f / 120.f, 1.f / 720.f, 1.f / 5040.f,

@@ -1222,10 +1222,7 @@ __global__ void __launch_bounds__(256) grad_chain_kernel(PairSrc src, const Pair
                                                          const T *incA, const T *incB, const T *gout,
                                                          T *dA, T *dB, T scale) {
     using V4 = typename Vec4<T>::type;
-    // rows padded by one element against bank conflicts, except in double
-    // precision, where the padding would pass the 48 KB static limit
-    constexpr int GP = sizeof(T) == 4 ? CT + 1 : CT;
-    __shared__ T Gs[CT][GP];
+    __shared__ T Gs[CT][CT];   // (a row of padding would pass the 48 KB static limit)
     __shared__ V4 Vs[CT][8];
     const int64_t d = src.d;
     const int64_t D4 = (d + 3) / 4;

@@ -113,10 +113,13 @@ struct PairRef {
 // row is estimated from the inverse of its offset and corrected to the exact
 // one: in FP32 for n <= 4096 (EST32; there the estimate is off by a few rows at
 // most; an FP64 instruction takes a warp 64 cycles here, and every pair of the
-// FP32 band sweeps asks for its row), else in FP64.  chain_f32_kernel keeps the
-// FP64 estimate: the other one moved its code so that an implicit Gram of 17 x
-// 138 paths of 56 and 118 points, order 2, took 104 us instead of 91, for 1 %
-// on symmetric Grams.
+// FP32 band sweeps asks for its row), else in FP64.  chain_f32_kernel and
+// plain_kernel ask once for a pair of thousands of cells and keep the FP64 one,
+// whose code is smaller: with the other the plain sweep took 84 registers instead
+// of 64 (FP32: 64 instead of 40), one block of 512 threads a SM instead of two
+// (FP64 Gram of 256 x 256 paths of 128 points, d = 8, order 2: 1147 ms instead of
+// 984), and an implicit Gram of 17 x 138 paths of 56 and 118 points, order 2, in
+// the chain 104 us instead of 91, for 1 % on symmetric Grams.
 template <bool EST32>
 __host__ __device__ inline void sym_index(int64_t k, int64_t n, int64_t &i, int64_t &j) {
     // row i holds n - i entries, starting at off(i) = i*n - i*(i-1)/2
